@@ -3,9 +3,11 @@
 //  - velocity/temperature gradients -> viscous flux vectors f^v, g^v, h^v
 //    (Sec. 2.1 stresses and heat flux, 4th-order central differences),
 //  - statistics (conservation sums, kinetic energy, enstrophy, extrema, CFL)
-//    with a deterministic two-level FP64 reduction (warp shuffles + fixed-order
-//    partials).
+//    with a deterministic two-level FP64 reduction (fixed-order folds per block, then
+//    over the blocks' partials).
 #include <math.h>
+
+#include <algorithm>
 
 #include "df.cuh"
 #include "df2.cuh"
@@ -253,83 +255,69 @@ __global__ void __launch_bounds__(VT_X * VT_Y, 4) k_visc32t(const double* __rest
 
 // ---- statistics ------------------------------------------------------------
 constexpr int ST_THREADS = 256;
-constexpr int ST_MAX_BLOCKS = 4096;
+constexpr int ST_SLOTS = 152 * 4;  // CTAs of k_stats_tiled the GPU holds at once (4 per SM)
 constexpr int NSUM = 7;   // mass, 3 momenta, energy, ke, enstrophy
 constexpr int NRED = 10;  // + rho_min, p_min, max wavespeed/dx
+constexpr int ST_FINAL_THREADS = 32 * NRED;
 
-struct Red {
-  double s[NSUM];
-  double rmin, pmin, wmax;
-};
-
-__device__ __forceinline__ void red_combine(Red& a, const Red& b) {
-#pragma unroll
-  for (int m = 0; m < NSUM; ++m) a.s[m] += b.s[m];
-  a.rmin = fmin(a.rmin, b.rmin);
-  a.pmin = fmin(a.pmin, b.pmin);
-  a.wmax = fmax(a.wmax, b.wmax);
+// Order of the doubles as signed 64-bit integers (for minima without the FP64 pipe): a < b if and
+// only if dkey(a) < dkey(b); NaNs lie outside [dkey(-inf), dkey(+inf)].  Its own inverse.
+__device__ __forceinline__ long long dkey(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
+}
+constexpr long long DKEY_NINF = (long long)0x800fffffffffffffULL, DKEY_PINF = 0x7ff0000000000000LL;
+// kmin = min(kmin, dkey(x)), a NaN x ignored (as fmin)
+__device__ __forceinline__ void key_min(long long& kmin, double x) {
+  const long long k = dkey(x);
+  if (k < kmin && k >= DKEY_NINF) kmin = k;
 }
 
-__device__ __forceinline__ Red warp_reduce(Red r) {
+// Sum (M = 0), minimum (1) or maximum (2) of the lanes' values in a fixed order; the result in lane 0.
+template <int M>
+__device__ __forceinline__ double warp_fold(double x) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    Red o;
-#pragma unroll
-    for (int m = 0; m < NSUM; ++m) o.s[m] = __shfl_down_sync(0xffffffffu, r.s[m], off);
-    o.rmin = __shfl_down_sync(0xffffffffu, r.rmin, off);
-    o.pmin = __shfl_down_sync(0xffffffffu, r.pmin, off);
-    o.wmax = __shfl_down_sync(0xffffffffu, r.wmax, off);
-    red_combine(r, o);
+    const double y = __shfl_down_sync(0xffffffffu, x, off);
+    x = (M == 0) ? x + y : (M == 1) ? fmin(x, y) : fmax(x, y);
   }
-  return r;
+  return x;
 }
 
-// Fixed-shape block reduction: lane order, then warp order.  Result valid in thread 0.
-__device__ Red block_reduce(Red r) {
-  __shared__ double sh[ST_THREADS / 32][NRED];
-  r = warp_reduce(r);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-#pragma unroll
-    for (int m = 0; m < NSUM; ++m) sh[wid][m] = r.s[m];
-    sh[wid][7] = r.rmin;
-    sh[wid][8] = r.pmin;
-    sh[wid][9] = r.wmax;
+// Fold of one quantity (0..NSUM-1: sum, NSUM and NSUM+1: minimum, last: maximum) by one warp over
+// n values v[0], v[stride], ...: every lane folds its values in order, then the lanes.
+__device__ __forceinline__ double fold_column(int q, const double* v, int n, int lane) {
+  double x = (q < NSUM) ? 0.0 : (q < NRED - 1) ? INFINITY : 0.0;
+  if (q < NSUM) {
+    for (int i = lane; i < n; i += 32) x += v[i];
+    return warp_fold<0>(x);
   }
-  __syncthreads();
-  if (wid == 0) {
-    Red t;
-    if (lane < ST_THREADS / 32) {
-#pragma unroll
-      for (int m = 0; m < NSUM; ++m) t.s[m] = sh[lane][m];
-      t.rmin = sh[lane][7];
-      t.pmin = sh[lane][8];
-      t.wmax = sh[lane][9];
-    } else {
-#pragma unroll
-      for (int m = 0; m < NSUM; ++m) t.s[m] = 0.0;
-      t.rmin = INFINITY;
-      t.pmin = INFINITY;
-      t.wmax = 0.0;
-    }
-    r = warp_reduce(t);
+  if (q < NRED - 1) {
+    for (int i = lane; i < n; i += 32) x = fmin(x, v[i]);
+    return warp_fold<1>(x);
   }
-  return r;
+  for (int i = lane; i < n; i += 32) x = fmax(x, v[i]);
+  return warp_fold<2>(x);
 }
 
-// Statistics: a block walks its tiles of
-// 32 x 8 x-y columns times VT_CZ planes in a fixed order; the velocity planes, with a 2-point
-// x-y halo, are converted to double-float once into a 5-plane ring (z-2 .. z+2) for the
-// vorticity stencils.  The accumulation order is fixed by the grid shape, so the result is
-// deterministic.  Sums, minima and counts in FP64; kinetic energy, vorticity, enstrophy and
-// wave speed in double-float on the FP32 pipe.  DFT: the temperature plane holds
-// double-float pairs (prim_point<true>).
+// Statistics: a block walks its tiles of 32 x 8 x-y columns times cz planes in a fixed order; the
+// velocity planes, with a 2-point x-y halo, are converted to double-float once into a 5-plane ring
+// (z-2 .. z+2) for the vorticity stencils.  The accumulation order is fixed by the grid shape, so
+// the result is deterministic.  Sums in FP64; kinetic energy, vorticity, enstrophy and wave speed in
+// double-float on the FP32 pipe, their low words summed apart (compensated, FP32) so that a point
+// costs 7 FP64 additions; minima as integers.  DFT: the temperature plane holds double-float pairs
+// (prim_point<true>).
+// What bounds it: FP64 additions and plane-load latency.  The block ends with one fold per quantity
+// by one warp each through shared memory: 84 FP64 warp instructions where ten shuffle reductions by
+// every warp took 400, and stats_plan launches no block without a tile.  128^3: 185 -> 86 us,
+// 256^3: 618 -> 568 us, 32^3: 59 -> 11 us (ncu, cold cache).
 constexpr int SR_SMEM = VT_RING * 3 * VT_PLANE * (int)sizeof(float2);  // 51,840 bytes
+static_assert(NRED * ST_THREADS * (int)sizeof(double) <= SR_SMEM, "the block's fold fits the ring");
 
 template <bool DFT>
 __global__ void __launch_bounds__(ST_THREADS, 4) k_stats_tiled(const double* __restrict__ u, const double* __restrict__ pm,
                                                                 const Grid g, double* __restrict__ partials, int ntx,
-                                                                int nty, long long ntiles) {
+                                                                int nty, long long ntiles, int cz) {
   extern __shared__ float2 ring[];  // [VT_RING][3][VT_HY][VT_HX]
   static_assert(VT_X * VT_Y == ST_THREADS, "one point per thread and plane");
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
@@ -340,18 +328,21 @@ __global__ void __launch_bounds__(ST_THREADS, 4) k_stats_tiled(const double* __r
   const int tid = threadIdx.x, tx = tid % VT_X, ty = tid / VT_X;
   constexpr int NPOS = (VT_PLANE + ST_THREADS - 1) / ST_THREADS;
   df wmax{0.0f, 0.0f};
-  Red r;
+  double sum[NSUM];
 #pragma unroll
-  for (int m = 0; m < NSUM; ++m) r.s[m] = 0.0;
-  r.rmin = INFINITY;
-  r.pmin = INFINITY;
-  r.wmax = 0.0;
+  for (int m = 0; m < NSUM; ++m) sum[m] = 0.0;
+  df klo{0.0f, 0.0f}, elo{0.0f, 0.0f};  // low words of the kinetic energy and the enstrophy
+  long long rmin = DKEY_PINF, pmin = DKEY_PINF;
   auto ld = [](const float2* P, int i) { const float2 v = P[i]; return df{v.x, v.y}; };
+  auto add_lo = [](df& s, float x) {  // compensated
+    const df t = two_sum(s.hi, x);
+    s = df{t.hi, __fadd_rn(s.lo, t.lo)};
+  };
   for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int x0 = (int)(t % ntx) * VT_X;
     const long long rest = t / ntx;
-    const int y0 = (int)(rest % nty) * VT_Y, z0 = (int)(rest / nty) * VT_CZ;
-    const int z1 = min(z0 + VT_CZ, nz);
+    const int y0 = (int)(rest % nty) * VT_Y, z0 = (int)(rest / nty) * cz;
+    const int z1 = min(z0 + cz, nz);
     auto slot = [&](int zz) { return ring + ((zz - z0 + 2) % VT_RING) * 3 * VT_PLANE; };
     int xy[NPOS];
 #pragma unroll
@@ -385,16 +376,17 @@ __global__ void __launch_bounds__(ST_THREADS, 4) k_stats_tiled(const double* __r
         const float2 *Zm2 = slot(z - 2), *Zm1 = slot(z - 1), *Z0 = slot(z), *Zp1 = slot(z + 1), *Zp2 = slot(z + 2);
         const double rho = __ldg(u + p);
         const double pr = __ldg(pm + PM_P * N + p);
-        r.s[0] += rho;
-        r.s[1] += __ldg(u + N + p);
-        r.s[2] += __ldg(u + 2 * N + p);
-        r.s[3] += __ldg(u + 3 * N + p);
-        r.s[4] += __ldg(u + 4 * N + p);
+        sum[0] += rho;
+        sum[1] += __ldg(u + N + p);
+        sum[2] += __ldg(u + 2 * N + p);
+        sum[3] += __ldg(u + 3 * N + p);
+        sum[4] += __ldg(u + 4 * N + p);
         const df rd = d2df_bits(rho);
         const df rh2{0.5f * rd.hi, 0.5f * rd.lo};  // rho / 2, exact
         const df vd[3] = {ld(Z0, c), ld(Z0 + VT_PLANE, c), ld(Z0 + 2 * VT_PLANE, c)};
         const df ke = df_mul_u(rh2, df_add_pos_u(df_sqr_u(vd[0]), df_add_pos_u(df_sqr_u(vd[1]), df_sqr_u(vd[2]))));
-        r.s[5] = (r.s[5] + f2d_bits(ke.hi)) + f2d_bits(ke.lo);
+        sum[5] += f2d_bits(ke.hi);
+        add_lo(klo, ke.lo);
         // vorticity: dv_m/dx_d for m != d
         auto gx = [&](int m) {
           const float2* P = Z0 + m * VT_PLANE;
@@ -412,9 +404,10 @@ __global__ void __launch_bounds__(ST_THREADS, 4) k_stats_tiled(const double* __r
         const df wy = df_add_fast(gz(0), df_neg(gx(2)));
         const df wz = df_add_fast(gx(1), df_neg(gy(0)));
         const df en = df_mul_u(rh2, df_add_pos_u(df_sqr_u(wx), df_add_pos_u(df_sqr_u(wy), df_sqr_u(wz))));
-        r.s[6] = (r.s[6] + f2d_bits(en.hi)) + f2d_bits(en.lo);
-        r.rmin = fmin(r.rmin, rho);
-        r.pmin = fmin(r.pmin, pr);
+        sum[6] += f2d_bits(en.hi);
+        add_lo(elo, en.lo);
+        key_min(rmin, rho);
+        key_min(pmin, pr);
         const df cs = df_sqrt(DFT ? load_df(pm + PM_T * N + p) : d2df_bits(__ldg(pm + PM_T * N + p)));
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
@@ -425,45 +418,30 @@ __global__ void __launch_bounds__(ST_THREADS, 4) k_stats_tiled(const double* __r
       __syncthreads();  // the slot of plane z - 2 takes plane z + 3 next
     }
   }
-  r.wmax = f2d_bits(wmax.hi) + f2d_bits(wmax.lo);
-  r = block_reduce(r);
-  if (threadIdx.x == 0) {
-    double* o = partials + (long long)blockIdx.x * NRED;
+  // the block's fold: quantity q of every thread side by side in shared memory, then one warp each
+  double* sh = reinterpret_cast<double*>(ring);  // [NRED][ST_THREADS]
+  sum[5] += f2d_bits(klo.hi) + f2d_bits(klo.lo);
+  sum[6] += f2d_bits(elo.hi) + f2d_bits(elo.lo);
 #pragma unroll
-    for (int m = 0; m < NSUM; ++m) o[m] = r.s[m];
-    o[7] = r.rmin;
-    o[8] = r.pmin;
-    o[9] = r.wmax;
+  for (int m = 0; m < NSUM; ++m) sh[m * ST_THREADS + tid] = sum[m];
+  sh[7 * ST_THREADS + tid] = __longlong_as_double(rmin ^ (long long)((unsigned long long)(rmin >> 63) >> 1));
+  sh[8 * ST_THREADS + tid] = __longlong_as_double(pmin ^ (long long)((unsigned long long)(pmin >> 63) >> 1));
+  sh[9 * ST_THREADS + tid] = f2d_bits(wmax.hi) + f2d_bits(wmax.lo);
+  __syncthreads();
+  for (int q = tid / 32; q < NRED; q += ST_THREADS / 32) {
+    const double r = fold_column(q, sh + q * ST_THREADS, ST_THREADS, tid & 31);
+    if ((tid & 31) == 0) partials[(long long)q * gridDim.x + blockIdx.x] = r;
   }
 }
 
-__global__ void __launch_bounds__(ST_THREADS) k_stats_final(const double* __restrict__ partials, int nblocks,
-                                                            const int* __restrict__ status, double vol,
-                                                            double inv_n, double* __restrict__ out) {
-  Red r;
-#pragma unroll
-  for (int m = 0; m < NSUM; ++m) r.s[m] = 0.0;
-  r.rmin = INFINITY;
-  r.pmin = INFINITY;
-  r.wmax = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-    const double* q = partials + (long long)b * NRED;
-    Red t;
-#pragma unroll
-    for (int m = 0; m < NSUM; ++m) t.s[m] = q[m];
-    t.rmin = q[7];
-    t.pmin = q[8];
-    t.wmax = q[9];
-    red_combine(r, t);
-  }
-  r = block_reduce(r);
+// partials [NRED][nblocks] of k_stats_tiled -> the statistics; one warp folds each quantity.
+__global__ void __launch_bounds__(ST_FINAL_THREADS) k_stats_final(const double* __restrict__ partials, int nblocks,
+                                                                  const int* __restrict__ status, double vol,
+                                                                  double inv_n, double* __restrict__ out) {
+  const int q = threadIdx.x / 32, lane = threadIdx.x & 31;
+  const double r = fold_column(q, partials + (long long)q * nblocks, nblocks, lane);
+  if (lane == 0) out[q] = (q < 5) ? r * vol : (q < NSUM) ? r * inv_n : r;
   if (threadIdx.x == 0) {
-    for (int m = 0; m < 5; ++m) out[m] = r.s[m] * vol;
-    out[5] = r.s[5] * inv_n;
-    out[6] = r.s[6] * inv_n;
-    out[7] = r.rmin;
-    out[8] = r.pmin;
-    out[9] = r.wmax;
     out[10] = (double)(*status);
     out[11] = 0.0;
   }
@@ -518,29 +496,49 @@ cudaError_t launch_visc32(const Grid& g, const double* u, float* fv, double gamm
   return cudaGetLastError();
 }
 
-int stats_num_blocks(const Grid& g) {
-  long long b = (g.N + ST_THREADS - 1) / ST_THREADS;
-  return (int)(b < ST_MAX_BLOCKS ? (b > 0 ? b : 1) : ST_MAX_BLOCKS);
+// Tiles of the statistics kernel: cz planes each, chosen so that the rounds of ST_SLOTS resident
+// blocks times a tile's planes (cz to fold and 4 halo planes, which only load: counted half) are
+// fewest.  256^3: 37 planes in 3 rounds where 16 take 7; small grids get short tiles (32^3: one
+// plane) so that more SMs share the serial plane loop.
+struct StatsPlan {
+  int cz, ntx, nty, blocks;
+  long long ntiles;
+};
+static StatsPlan stats_plan(const Grid& g) {
+  StatsPlan p;
+  p.ntx = (g.n[0] + VT_X - 1) / VT_X;
+  p.nty = (g.n[1] + VT_Y - 1) / VT_Y;
+  long long best = -1;
+  for (int cz = std::min(g.n[2], 64); cz >= 1; --cz) {
+    const long long tiles = (long long)p.ntx * p.nty * ((g.n[2] + cz - 1) / cz);
+    const long long cost = ((tiles + ST_SLOTS - 1) / ST_SLOTS) * (cz + 2);
+    if (best < 0 || cost < best) {
+      best = cost;
+      p.cz = cz;
+      p.ntiles = tiles;
+    }
+  }
+  p.blocks = (int)std::min<long long>(p.ntiles, ST_SLOTS);
+  return p;
 }
+
+int stats_num_blocks(const Grid& g) { return stats_plan(g).blocks; }
 
 cudaError_t launch_stats(const Grid& g, const double* u, const double* pm, double gamma, double* partials,
                          cudaStream_t s, int df) {
   (void)gamma;
-  const int ntx = (g.n[0] + VT_X - 1) / VT_X, nty = (g.n[1] + VT_Y - 1) / VT_Y, ntz = (g.n[2] + VT_CZ - 1) / VT_CZ;
-  const long long ntiles = (long long)ntx * nty * ntz;
-  // exactly stats_num_blocks(g) blocks: the partials k_stats_final reduces (blocks without a
-  // tile write neutral partials)
+  const StatsPlan p = stats_plan(g);
   if (df)
-    k_stats_tiled<true><<<stats_num_blocks(g), ST_THREADS, SR_SMEM, s>>>(u, pm, g, partials, ntx, nty, ntiles);
+    k_stats_tiled<true><<<p.blocks, ST_THREADS, SR_SMEM, s>>>(u, pm, g, partials, p.ntx, p.nty, p.ntiles, p.cz);
   else
-    k_stats_tiled<false><<<stats_num_blocks(g), ST_THREADS, SR_SMEM, s>>>(u, pm, g, partials, ntx, nty, ntiles);
+    k_stats_tiled<false><<<p.blocks, ST_THREADS, SR_SMEM, s>>>(u, pm, g, partials, p.ntx, p.nty, p.ntiles, p.cz);
   return cudaGetLastError();
 }
 
 cudaError_t launch_stats_final(const Grid& g, const double* partials, int nblocks, const int* status, double* out,
                                cudaStream_t s) {
-  k_stats_final<<<1, ST_THREADS, 0, s>>>(partials, nblocks, status, g.h[0] * g.h[1] * g.h[2], 1.0 / (double)g.N,
-                                         out);
+  k_stats_final<<<1, ST_FINAL_THREADS, 0, s>>>(partials, nblocks, status, g.h[0] * g.h[1] * g.h[2],
+                                               1.0 / (double)g.N, out);
   return cudaGetLastError();
 }
 

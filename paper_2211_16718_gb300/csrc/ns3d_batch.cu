@@ -571,7 +571,6 @@ int ns3d_batch_init(const ns3d_params* params, int count, void* cuda_stream, ns3
   b->ivar.assign(count, 0);
   b->inst.resize(count);
   b->pt_off.assign(count + 1, 0);
-  long long maxN = 0;
   for (int i = 0; i < count; ++i) {
     const ns3d_params& p = params[i];
     Inst& in = b->inst[i];
@@ -586,7 +585,7 @@ int ns3d_batch_init(const ns3d_params* params, int count, void* cuda_stream, ns3
     in.kappa = (p.mu_eff > 0.0) ? p.mu_eff / ((p.gamma - 1.0) * p.prandtl) : 0.0;
     for (int d = 0; d < 3; ++d) in.r12[d] = 1.0 / (12.0 * in.g.h[d]);
     b->pt_off[i + 1] = b->pt_off[i] + in.g.N;
-    if (in.g.N > maxN) maxN = in.g.N;
+    b->nstat_blocks = std::max(b->nstat_blocks, stats_num_blocks(in.g));
     // scratch: primitives, viscous fluxes, two stage states, RK accumulator, RHS accumulator
     const size_t sizes[6] = {7, 12, 5, 5, 5, 5};
     for (int a = 0; a < 6; ++a) {
@@ -605,9 +604,6 @@ int ns3d_batch_init(const ns3d_params* params, int count, void* cuda_stream, ns3
     in.pm = b->bufs[6 * i + 0];
     in.fv = b->bufs[6 * i + 1];
   }
-  Grid gmax;
-  gmax.N = maxN;
-  b->nstat_blocks = stats_num_blocks(gmax);
   bool ok = cudaMalloc(&b->d_inst, sizeof(Inst) * count) == cudaSuccess &&
             cudaMalloc(&b->d_pt_off, sizeof(long long) * (count + 1)) == cudaSuccess &&
             cudaMalloc(&b->d_tile_off, sizeof(long long) * 3 * (count + 1)) == cudaSuccess &&
