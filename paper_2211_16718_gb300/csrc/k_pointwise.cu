@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(PW_THREADS) k_visc(const double* __restrict__ 
 }
 
 // Tiled NS3D_FP64 viscous-flux kernel (primitives in the layout of prim_point<true>).  A CTA
-// owns a 32 x 8 block of x-y columns and marches along z through VT_CZ planes.  Each plane of
+// owns a 32 x 8 block of x-y columns and marches along z through cz planes (visc_chunk).  Each plane of
 // (u, v, w, T), with a 2-point x-y halo, is converted to double-float once into a ring of 5
 // planes (z-2 .. z+2) in shared memory, so every stencil value is converted once rather than
 // once per stencil that uses it (12 times).  The ring holds the fields in pairs, (u, v) and
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(PW_THREADS) k_visc(const double* __restrict__ 
 // arithmetic is that of visc_point_df_ijk: the same conversions, the same gradient and flux
 // operations, so the same bits.
 constexpr int VT_X = 32, VT_Y = 8, VT_HX = VT_X + 4, VT_HY = VT_Y + 4, VT_PLANE = VT_HX * VT_HY;
-constexpr int VT_RING = 5, VT_CZ = VISC_ZCHUNK;
+constexpr int VT_RING = 5;
 constexpr int VT_SMEM = VT_RING * 2 * VT_PLANE * (int)sizeof(float4);  // 69,120 bytes
 
 // d4_dfv on two lanes.
@@ -72,12 +72,12 @@ __device__ __forceinline__ df2 d4_dfv2(df2 qm2, df2 qm1, df2 qp1, df2 qp2, df2 r
 
 __global__ void __launch_bounds__(VT_X * VT_Y, 3) k_visc_tiled(const double* __restrict__ pm, double* __restrict__ fv,
                                                                 const Grid g, double mu, double kappa, int only_d,
-                                                                int zc0) {
+                                                                int zb, int ze, int cz) {
   extern __shared__ float4 ring4[];  // [VT_RING][2][VT_HY][VT_HX]: (u, v) and (w, T)
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const long long N = g.N;
-  const int x0 = blockIdx.x * VT_X, y0 = blockIdx.y * VT_Y, z0 = (zc0 + blockIdx.z) * VT_CZ;
-  const int z1 = min(z0 + VT_CZ, nz);
+  const int x0 = blockIdx.x * VT_X, y0 = blockIdx.y * VT_Y, z0 = zb + blockIdx.z * cz;
+  const int z1 = min(z0 + cz, ze);
   const int tid = threadIdx.x, tx = tid % VT_X, ty = tid / VT_X;
   const df2 r12[3] = {df2_splat(d2df_bits(g.r12h[0])), df2_splat(d2df_bits(g.r12h[1])),
                       df2_splat(d2df_bits(g.r12h[2]))};
@@ -153,7 +153,7 @@ inline dim3 plane_grid(const Grid& g) { return dim3((g.n[0] + 31) / 32, (g.n[1] 
 
 // ---- FP32-bulk viscous fluxes (NS3D_FP32_BULK) ---------------------------------------
 // The tiled form of k_visc_tiled in FP32, straight from the conserved state: a CTA owns a
-// 32 x 8 block of x-y columns and marches along z through VT_CZ planes; every plane of
+// 32 x 8 block of x-y columns and marches along z through cz planes (visc_chunk); every plane of
 // (u, v, w, T), with a 2-point x-y halo, is formed once from the state (converted to FP32 by
 // bit manipulation) into a ring of 5 planes (z-2 .. z+2) of float4 in shared memory.  Each
 // point then takes the 12 gradients with the 4th-order central difference and writes the
@@ -172,12 +172,12 @@ constexpr int V32_SMEM = VT_RING * VT_PLANE * (int)sizeof(float4);  // 34,560 by
 
 __global__ void __launch_bounds__(VT_X * VT_Y, 4) k_visc32t(const double* __restrict__ u, float* __restrict__ fv,
                                                              const Grid g, float gamma, float mu, float kappa,
-                                                             int only_d) {
+                                                             int only_d, int cz) {
   extern __shared__ float4 ring4[];  // [VT_RING][VT_HY][VT_HX]: u, v, w, T
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const long long N = g.N;
-  const int x0 = blockIdx.x * VT_X, y0 = blockIdx.y * VT_Y, z0 = blockIdx.z * VT_CZ;
-  const int z1 = min(z0 + VT_CZ, nz);
+  const int x0 = blockIdx.x * VT_X, y0 = blockIdx.y * VT_Y, z0 = blockIdx.z * cz;
+  const int z1 = min(z0 + cz, nz);
   const int tid = threadIdx.x, tx = tid % VT_X, ty = tid / VT_X;
   const float r12[3] = {(float)g.r12h[0], (float)g.r12h[1], (float)g.r12h[2]};
   const float gm1 = gamma - 1.0f;
@@ -461,6 +461,27 @@ cudaError_t launch_prim(const Grid& g, const double* u, double* pm, double gamma
   return cudaGetLastError();
 }
 
+// Planes per CTA of the tiled viscous kernels over nz planes of g, with `slots` CTAs resident at
+// once: the chunk for which the rounds of resident CTAs times the planes a CTA walks (its chunk
+// and 4 halo planes, which only load: counted half) are fewest, the longest of equals.  A fixed
+// chunk of 16 left 32^3 with 8 CTAs of 20 serial planes, 64^3 with 64, and 128^3 with 512 CTAs on
+// 456 slots, a second round for 56 of them.  Per launch (ncu): 32^3 43 -> 7 us, 64^3 44 -> 22 us,
+// 128^3 115 -> 97 us, 256^3 685 -> 672 us.
+static int visc_chunk(const Grid& g, int nz, int slots) {
+  const long long nxy = (long long)((g.n[0] + VT_X - 1) / VT_X) * ((g.n[1] + VT_Y - 1) / VT_Y);
+  long long best = -1;
+  int chunk = 1;
+  for (int cz = std::min(nz, 64); cz >= 1; --cz) {
+    const long long ctas = nxy * ((nz + cz - 1) / cz);
+    const long long cost = ((ctas + slots - 1) / slots) * (cz + 2);
+    if (best < 0 || cost < best) {
+      best = cost;
+      chunk = cz;
+    }
+  }
+  return chunk;
+}
+
 cudaError_t launch_visc(const Grid& g, const double* pm, double* fv, double mu, double kappa, cudaStream_t s,
                         int only_d, int df, int z0, int z1) {
   const double rx = g.r12h[0], ry = g.r12h[1], rz = g.r12h[2];
@@ -469,10 +490,9 @@ cudaError_t launch_visc(const Grid& g, const double* pm, double* fv, double mu, 
   if (z0 < 0 || z1 > nz || z0 > z1) return cudaErrorInvalidValue;
   if (z0 == z1) return cudaSuccess;
   if (df) {
-    if (z0 % VT_CZ != 0 || (z1 % VT_CZ != 0 && z1 != nz)) return cudaErrorInvalidValue;
-    const int zc0 = z0 / VT_CZ, zc1 = (z1 + VT_CZ - 1) / VT_CZ;
-    const dim3 grid((g.n[0] + VT_X - 1) / VT_X, (g.n[1] + VT_Y - 1) / VT_Y, zc1 - zc0);
-    k_visc_tiled<<<grid, VT_X * VT_Y, VT_SMEM, s>>>(pm, fv, g, mu, kappa, only_d, zc0);
+    const int cz = visc_chunk(g, z1 - z0, 3 * 152);
+    const dim3 grid((g.n[0] + VT_X - 1) / VT_X, (g.n[1] + VT_Y - 1) / VT_Y, (z1 - z0 + cz - 1) / cz);
+    k_visc_tiled<<<grid, VT_X * VT_Y, VT_SMEM, s>>>(pm, fv, g, mu, kappa, only_d, z0, z1, cz);
   } else {
     dim3 grid = plane_grid(g);
     grid.z = z1 - z0;
@@ -491,8 +511,9 @@ cudaError_t prepare_visc_kernels() {
 
 cudaError_t launch_visc32(const Grid& g, const double* u, float* fv, double gamma, double mu, double kappa,
                           cudaStream_t s, int only_d) {
-  const dim3 grid((g.n[0] + VT_X - 1) / VT_X, (g.n[1] + VT_Y - 1) / VT_Y, (g.n[2] + VT_CZ - 1) / VT_CZ);
-  k_visc32t<<<grid, VT_X * VT_Y, V32_SMEM, s>>>(u, fv, g, (float)gamma, (float)mu, (float)kappa, only_d);
+  const int cz = visc_chunk(g, g.n[2], 4 * 152);
+  const dim3 grid((g.n[0] + VT_X - 1) / VT_X, (g.n[1] + VT_Y - 1) / VT_Y, (g.n[2] + cz - 1) / cz);
+  k_visc32t<<<grid, VT_X * VT_Y, V32_SMEM, s>>>(u, fv, g, (float)gamma, (float)mu, (float)kappa, only_d, cz);
   return cudaGetLastError();
 }
 

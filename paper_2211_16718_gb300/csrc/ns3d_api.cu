@@ -464,9 +464,9 @@ namespace {
 
 // Whether ns3d_step_host overlaps its copies with the kernels: the direction passes of
 // NS3D_FP64 / NS3D_FP64_STRICT with all viscous fluxes stored, on grids of at least four
-// viscous z chunks (smaller grids copy in well under a millisecond).
+// slabs (smaller grids copy in well under a millisecond).
 bool slab_pipeline_ok(const ns3d_ctx* c, int nsteps) {
-  return nsteps >= 1 && !c->lean && c->p.precision != NS3D_FP32_BULK && c->g.n[2] >= 4 * VISC_ZCHUNK;
+  return nsteps >= 1 && !c->lean && c->p.precision != NS3D_FP32_BULK && c->g.n[2] >= 4 * ns3d_ctx::SLAB_PLANES;
 }
 
 int ensure_copy_stream(ns3d_ctx* c) {
@@ -513,8 +513,8 @@ int ns3d_step_host(ns3d_ctx* c, double* u_host, double dt, int nsteps, ns3d_stat
     const Grid& g = c->g;
     const long long plane = (long long)g.n[0] * g.n[1];
     SlabPipe pin, pout;
-    const int chunks = g.n[2] / VISC_ZCHUNK;
-    slab_bounds(pin, min(chunks, (int)ns3d_ctx::MAX_SLABS), chunks, VISC_ZCHUNK, g.n[2]);
+    const int chunks = g.n[2] / ns3d_ctx::SLAB_PLANES;
+    slab_bounds(pin, min(chunks, (int)ns3d_ctx::MAX_SLABS), chunks, ns3d_ctx::SLAB_PLANES, g.n[2]);
     pin.ev = c->slab_ev;
     int tp = 0, w = 0;
     dir_tile_shape(c->p.precision == NS3D_FP64_STRICT ? 0 : 1, c->variant, &tp, &w);

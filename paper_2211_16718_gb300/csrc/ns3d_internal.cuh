@@ -87,9 +87,7 @@ cudaError_t launch_prim(const Grid& g, const double* u, double* pm, double gamma
                         int df = 0, long long p0 = 0, long long p1 = -1);
 // only_d < 0: all three viscous flux vectors into fv[12][N]; only_d = d: the flux along d into fv[4][N];
 // df: the NS3D_FP64 form (double-float from the stencil values on; primitives from launch_prim(df=1))
-// [z0, z1): the planes of a partial launch (z1 < 0: through nz); with df, z0 and z1 (unless nz) must be
-// multiples of VISC_ZCHUNK, the z extent of one CTA of the tiled kernel.
-constexpr int VISC_ZCHUNK = 16;
+// [z0, z1): the planes of a partial launch (z1 < 0: through nz)
 cudaError_t launch_visc(const Grid& g, const double* pm, double* fv, double mu, double kappa, cudaStream_t s,
                         int only_d = -1, int df = 0, int z0 = 0, int z1 = -1);
 // FP32-bulk viscous fluxes, straight from the state u: FP32 planes fv[12][N] (only_d = d: fv[4][N])

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2211_16718_gb300 import inputs as I
-from tests._util import rel_err
+from tests._util import flux_scale, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -56,3 +56,22 @@ def test_stats_minima_of_bad_states(ns3d):
     assert sg["status"] == ns3d.NS3D_ENONPHYSICAL
     assert sg["rho_min"] == np.nanmin(rho)
     assert sg["p_min"] == pytest.approx(np.nanmin(p), rel=1e-14)
+
+
+# one-plane chunks, a shorter last chunk, more x-y tiles than resident blocks, one plane of points
+@pytest.mark.parametrize("nx,ny,nz", [(33, 9, 70), (21, 40, 131), (640, 256, 3), (40, 24, 1)])
+def test_viscous_chunks(ns3d, orc, nx, ny, nz):
+    u = I.random_smooth(nx, ny, nz, seed=6, amp=0.1, mach=0.4)
+    ref = orc.rhs(orc.Params(nx, ny, nz, mu_eff=0.02), u)
+    out = []
+    for storage in (1, 2):
+        s = ns3d.Solver(nx, ny, nz, mu_eff=0.02, storage=storage)
+        out.append(s.rhs(_gpu(u)).cpu().numpy())
+        s.close()
+    assert rel_err(out[0], ref) <= 1e-12  # the tolerance of one right-hand side
+    assert np.array_equal(out[0], out[1])
+    s = ns3d.Solver(nx, ny, nz, mu_eff=0.02, precision=1)
+    r32 = s.rhs(_gpu(u)).cpu().numpy()
+    s.close()
+    # FP32 fluxes: 1e-5 of the flux scale over the smallest spacing (as the FP32-bulk tests)
+    assert np.abs(r32 - ref).max() <= 1e-5 * flux_scale(u, (2 * np.pi,) * 3)
