@@ -1,6 +1,6 @@
 // Standalone launches of the fused direction pass (one tile per CTA); the tile
-// computation itself is dir_tile in k_dir_impl.cuh.  Tile shapes (points along
-// the pencil x lines) are template variants: a context uses the one set by
+// computation itself is dir_tile in k_dir_impl.cuh.  Tile shapes (points along the
+// pencil, at most, x lines; the pencil is cut into tiles of equal length) are template variants: a context uses the one set by
 // ns3d_set_variant (default 0); an ensemble's autotuner picks one per grid size.
 //   MODE 0 (all FP64):              32 x 4
 //   MODE 1 (FP64 + double-float):   variant 0: 24 x 4, 1: 16 x 4, 2: 40 x 2
@@ -15,12 +15,11 @@ namespace {
 template <int D, int MODE, int TP, int W>
 __global__ void __launch_bounds__(Plan<MODE, TP, W>::THREADS, Plan<MODE, TP, W>::MIN_CTAS) k_dir(const DirArgs a) {
   extern __shared__ __align__(16) double sm[];
-  if (D == 2) {
-    const int tz = a.zorder ? blockIdx.y : blockIdx.x, tl = a.zorder ? blockIdx.x : blockIdx.y;
-    dir_tile<D, MODE, TP, W>(a, sm, a.t0 + tz, tl, blockIdx.z);
-  } else {
-    dir_tile<D, MODE, TP, W>(a, sm, blockIdx.x, blockIdx.y, a.t0 + blockIdx.z);
-  }
+  const bool swap = (D == 2 && a.zorder);
+  const int tile = (swap ? blockIdx.y : blockIdx.x) + (D == 2 ? a.t0 : 0);
+  int s0, len;
+  tile_span(D, a.g.n[D], a.tile_u, a.tile_r, tile, s0, len);
+  dir_tile<D, MODE, TP, W>(a, sm, s0, len, swap ? blockIdx.x : blockIdx.y, blockIdx.z + (D == 2 ? 0 : a.t0));
 }
 
 // Tiles [lo, hi) along the range axis (hi < 0: all): the tiles along z for D = 2 (blockIdx.x, or
@@ -43,6 +42,7 @@ cudaError_t launch_t(const DirArgs& a, cudaStream_t s, int lo = 0, int hi = -1) 
   ext = (unsigned)(hi - lo);
   DirArgs r = a;
   r.t0 = lo;
+  tile_split_units(D, a.g.n[D], (a.g.n[D] + TP - 1) / TP, r.tile_u, r.tile_r);
   k_dir<D, MODE, TP, W><<<grid, PL::THREADS, PL::BYTES, s>>>(r);
   return cudaGetLastError();
 }
@@ -112,6 +112,16 @@ void dir_tile_shape(int mode, int variant, int* tp, int* w) {
     *tp = 32;
     *w = 4;
   }
+}
+
+int dir_tile_start(const Grid& g, int d, int mode, int variant, int t) {
+  int tp = 0, w = 0, u = 0, r = 0, s0 = 0, len = 0;
+  dir_tile_shape(mode, variant, &tp, &w);
+  const int nt = (g.n[d] + tp - 1) / tp;
+  if (t >= nt) return g.n[d];
+  tile_split_units(d, g.n[d], nt, u, r);
+  tile_span(d, g.n[d], u, r, t, s0, len);
+  return s0;
 }
 
 cudaError_t launch_dir(int d, const DirArgs& a, cudaStream_t s) {

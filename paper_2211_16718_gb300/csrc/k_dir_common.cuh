@@ -24,6 +24,63 @@ __device__ __forceinline__ void tile_split(int item, int npos, int& pos, int& li
   }
 }
 
+// ---- balanced tiles -----------------------------------------------------------------
+// A pencil of n points is cut into nt = ceil(n / TP) tiles of nearly equal length (at most TP)
+// instead of full tiles and a remainder, and a tile computes no more than its own points and
+// halo.  Lengths are whole units of points: 4 along x, so that the tiles' rows start on 32-byte
+// sectors, 1 along y and z.  Tile t covers tile_unit * [t u + min(t, r), ...) with
+// u = units / nt, r = units % nt (the first r tiles are one unit longer).
+__host__ __device__ constexpr int tile_unit(int d) { return d == 0 ? 4 : 1; }
+__host__ __device__ __forceinline__ void tile_split_units(int d, int n, int nt, int& u, int& r) {
+  const int units = (n + tile_unit(d) - 1) / tile_unit(d);
+  u = units / nt;
+  r = units - u * nt;
+}
+// First point and number of points of tile t.
+__host__ __device__ __forceinline__ void tile_span(int d, int n, int u, int r, int t, int& s0, int& len) {
+  s0 = tile_unit(d) * (t * u + (t < r ? t : r));
+  const int end = s0 + tile_unit(d) * (u + (t < r ? 1 : 0));
+  len = (end < n ? end : n) - s0;
+}
+
+// ceil(2^20 / d): i / d = (i * c_rcp20[d]) >> 20 for the item numbers of a tile (i d < 2^20, and the
+// product below 2^32), d a run-time extent of the tile.
+struct Rcp20 {
+  unsigned v[64];
+  constexpr Rcp20() : v() {
+    for (unsigned d = 1; d < 64; ++d) v[d] = ((1u << 20) + d - 1) / d;
+  }
+};
+static __constant__ const Rcp20 c_rcp20 = Rcp20();
+
+// Item numbers of a phase over (scalar m, position < npos, line < W): the order of tile_idx with the
+// run-time extent npos (rcp = c_rcp20.v[npos]).
+template <int D, int W>
+__device__ __forceinline__ void item_split(int item, int npos, unsigned rcp, int& m, int& pos, int& line) {
+  if (D == 0) {
+    const int ml = (int)(((unsigned)item * rcp) >> 20);
+    pos = item - ml * npos;
+    m = ml / W;
+    line = ml % W;
+  } else {
+    const int mp = item / W;
+    line = item % W;
+    m = (int)(((unsigned)mp * rcp) >> 20);
+    pos = mp - m * npos;
+  }
+}
+// The same without the scalar.
+template <int D, int W>
+__device__ __forceinline__ void item_split(int item, int npos, unsigned rcp, int& pos, int& line) {
+  if (D == 0) {
+    line = (int)(((unsigned)item * rcp) >> 20);
+    pos = item - line * npos;
+  } else {
+    line = item % W;
+    pos = item / W;
+  }
+}
+
 // Flat grid index of pencil coordinate c on line la of the tile row bz.
 template <int D>
 __device__ __forceinline__ long long tile_flat(const Grid& g, int c, int la, int bz) {

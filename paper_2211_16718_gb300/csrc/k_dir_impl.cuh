@@ -150,27 +150,30 @@ __device__ __forceinline__ df2 df2_offset(df2 B1, df2 B2, df2 B3, df2 e, df2 ta,
   return df2_div(num, df2_mul_f_u(den, 6.0f));
 }
 
-// One tile (tx, ty, tz) of the direction-D pass, executed by the whole CTA on the
-// shared memory sm (PL::BYTES).  Used by the standalone kernels (one tile per CTA),
-// the batched kernels and the persistent ensemble kernel (many tiles per CTA,
-// with a barrier between tiles).  NC selects read-only-cache loads, valid only when
-// the inputs are not written during the kernel (false in the persistent kernel).
+// One tile of the direction-D pass, executed by the whole CTA on the shared memory sm (PL::BYTES):
+// the points [s0, s0 + len) along D (len <= TP), line group ty, tile row bz.  Used by the standalone
+// kernels (one tile per CTA), the batched kernels and the persistent ensemble kernel (many tiles per
+// CTA, with a barrier between tiles).  NC selects read-only-cache loads, valid only when the inputs
+// are not written during the kernel (false in the persistent kernel).
+// The phases loop over the extents of this tile, not the plan's: a 32-point line as 24 + 8 with all
+// 24 computed in the second tile did the work of 48 points, balanced and trimmed 16 + 16 that of 32.
 template <int D, int MODE, int TP_, int W_, bool NC = true>
-__device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, int ty, int tz) {
+__device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, int len, int ty, int bz) {
   using PL = Plan<MODE, TP_, W_>;
   constexpr int TP = PL::TP, NP = PL::NP, NW = PL::NW, NI = PL::NI, W = PL::W;
   constexpr int W2 = (W + 1) / 2;  // line pairs (MODE 1)
   static_assert(MODE == 0 || W % 2 == 0, "MODE 1 tiles pair their lines");
+  static_assert(NP < 64, "extents fit c_rcp20");
+  const int np = len + 6, nw = len + 4, ni = len + 1;  // this tile's points with halo, windows, interfaces
   const int nD = a.g.n[D];
   constexpr int AX = (D == 0) ? 1 : 0;   // axis of the W lines
   constexpr int BX = (D == 2) ? 1 : 2;   // axis of blockIdx.z
   const int na = a.g.n[AX];
   const int nx = a.g.n[0], ny = a.g.n[1];
   const long long N = a.g.N;
-  const int s0 = tx * TP;
   const int a0 = ty * W;
-  const int bz = tz;
   const int tid = threadIdx.x;
+  auto wrap = [&](int c) { return (c < 0 || c >= nD) ? wrap_idx(c, nD) : c; };
 
   auto flat = [&](int c, int la) -> long long {
     int idx[3];
@@ -181,10 +184,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
   };
 
   // ---- A: load --------------------------------------------------------------
-  for (int item = tid; item < NP * W; item += PL::THREADS) {
+  for (int item = tid; item < np * W; item += PL::THREADS) {
     int pos, line;
-    tile_split<D, W>(item, NP, pos, line);
-    const int c = wrap_idx(s0 - 3 + pos, nD);
+    item_split<D, W>(item, np, c_rcp20.v[np], pos, line);
+    const int c = wrap(s0 - 3 + pos);
     const int la = min(a0 + line, na - 1);
     const long long p = flat(c, la);
     double U[5];
@@ -219,7 +222,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
 
   // ---- A2 (MODE 1): first differences g_j = q_{j+1} - q_j in FP64, kept as double-float,
   //      and the point values q_j of the five flux scalars copied to interface j - 2
-  constexpr int PF0 = (MODE == 1) ? PL::THREADS - NP * W : 0;  // first prefetching thread (MODE 1)
+  const int pf = tid - (PL::THREADS - np * W);  // prefetched point of this thread (MODE 1; none if negative)
   static_assert(MODE == 0 || NP * W <= PL::THREADS, "one prefetched point per thread");
   if constexpr (MODE == 1) {
     constexpr int NG = PL::NG;
@@ -227,17 +230,18 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
     float4* G = reinterpret_cast<float4*>(sm + PL::OFF_G);
     double* R = sm + PL::OFF_R;
     // one item per line pair (lines 2 lp, 2 lp + 1), stored as (hi0, hi1, lo0, lo1)
-    for (int item = tid; item < NQ * NG * W2; item += PL::THREADS) {
-      const int m = item / (NG * W2);
-      int j, lp;
-      tile_split<D, W2>(item - m * NG * W2, NG, j, lp);
+    const int ng = len + 5;
+    const unsigned rcp_ng = c_rcp20.v[ng];
+    for (int item = tid; item < NQ * ng * W2; item += PL::THREADS) {
+      int m, j, lp;
+      item_split<D, W2>(item, ng, rcp_ng, m, j, lp);
       const double* qm = q + m * NP * W;
       const int l0 = 2 * lp, l1 = l0 + 1;
       const double qa0 = qm[tile_idx<D, W>(j, l0, NP)], qb0 = qm[tile_idx<D, W>(j + 1, l0, NP)];
       const double qa1 = qm[tile_idx<D, W>(j, l1, NP)], qb1 = qm[tile_idx<D, W>(j + 1, l1, NP)];
       const df g0 = d2df_bits(qb0 - qa0), g1 = d2df_bits(qb1 - qa1);
       G[m * NG * W2 + tile_idx<D, W2>(j, lp, NG)] = make_float4(g0.hi, g1.hi, g0.lo, g1.lo);
-      if (m >= 4 && j >= 2 && j < NI + 2) {
+      if (m >= 4 && j >= 2 && j < ni + 2) {
         R[(1 + m) * NI * W + tile_idx<D, W>(j - 2, l0, NI)] = qa0;
         R[(1 + m) * NI * W + tile_idx<D, W>(j - 2, l1, NI)] = qa1;
       }
@@ -247,10 +251,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
     // their space while phases B and C run.  One point per thread, on the last NP*W
     // threads (those with the fewest phase-C items), which also convert their Roe
     // inputs to double-float in place before the barrier that ends phase C.
-    if (tid >= PF0) {
+    if (pf >= 0) {
       int pos, line;
-      tile_split<D, W>(tid - PF0, NP, pos, line);
-      const long long p = flat(wrap_idx(s0 - 3 + pos, nD), min(a0 + line, na - 1));
+      item_split<D, W>(pf, np, c_rcp20.v[np], pos, line);
+      const long long p = flat(wrap(s0 - 3 + pos), min(a0 + line, na - 1));
       const int sp = tile_idx<D, W>(pos, line, NP);
       double* r = sm + PL::OFF_ROE + sp;
       cp_async8(r + 0 * NP * W, a.pm + PM_SR * N + p);
@@ -271,10 +275,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
   int need_scale = 0;
   if constexpr (MODE == 0) {
     const double* q = sm + PL::OFF_Q;
-    for (int item = tid; item < NQ * NW * W; item += PL::THREADS) {
-      const int m = item / (NW * W);
-      int w, line;
-      tile_split<D, W>(item - m * NW * W, NW, w, line);
+    const unsigned rcp_nw = c_rcp20.v[nw];
+    for (int item = tid; item < NQ * nw * W; item += PL::THREADS) {
+      int m, w, line;
+      item_split<D, W>(item, nw, rcp_nw, m, w, line);
       const int o = tile_idx<D, W>(w, line, NW);
       const double* qm = q + m * NP * W;
       const double x = qm[tile_idx<D, W>(w, line, NP)];
@@ -298,10 +302,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
     float4* S = reinterpret_cast<float4*>(sm + PL::OFF_S);
     const df2 c133 = df2_splat(df{a.c133_hi, a.c133_lo});
     const df2 eps4 = df2_splat(df{a.eps4_hi, a.eps4_lo});
-    for (int item = tid; item < NQ * NW * W2; item += PL::THREADS) {
-      const int m = item / (NW * W2);
-      int w, lp;
-      tile_split<D, W2>(item - m * NW * W2, NW, w, lp);
+    const unsigned rcp_nw = c_rcp20.v[nw];
+    for (int item = tid; item < NQ * nw * W2; item += PL::THREADS) {
+      int m, w, lp;
+      item_split<D, W2>(item, nw, rcp_nw, m, w, lp);
       const int o = tile_idx<D, W2>(w, lp, NW);
       const float4* G = reinterpret_cast<const float4*>(sm + PL::OFF_G) + m * PL::NG * W2;
       const df2 dgm = df2_from4(G[tile_idx<D, W2>(w, lp, PL::NG)]);
@@ -310,7 +314,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
       // third difference T_w = s_w - s_{w+1} (phase C needs T_f, T_{f+1}, T_{f+2}; the last
       // window has no s_{w+1} in the tile and its T is never read)
       df2 T{f2splat(0.0f), f2splat(0.0f)};
-      if (w + 2 < PL::NG) {
+      if (w + 1 < nw) {
         const df2 g2 = df2_from4(G[tile_idx<D, W2>(w + 2, lp, PL::NG)]);
         T = df2_add_fast(ds, df2_neg(df2_add_fast(g2, df2_neg(dgp))));
       }
@@ -351,10 +355,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
   if constexpr (MODE == 0) {
     const double* q = sm + PL::OFF_Q;
     double* rec = sm + PL::OFF_R;
-    for (int item = tid; item < NQ * NI * W; item += PL::THREADS) {
-      const int m = item / (NI * W);
-      int f, line;
-      tile_split<D, W>(item - m * NI * W, NI, f, line);
+    const unsigned rcp_ni = c_rcp20.v[ni];
+    for (int item = tid; item < NQ * ni * W; item += PL::THREADS) {
+      int m, f, line;
+      item_split<D, W>(item, ni, rcp_ni, m, f, line);
       const double* qm = q + m * NP * W;
       const double P0 = qm[tile_idx<D, W>(f, line, NP)], P1 = qm[tile_idx<D, W>(f + 1, line, NP)];
       const double P2 = qm[tile_idx<D, W>(f + 2, line, NP)], P3 = qm[tile_idx<D, W>(f + 3, line, NP)];
@@ -388,10 +392,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
     float2* rf = reinterpret_cast<float2*>(sm + PL::OFF_R);
     auto phase_c = [&](auto scaled) {
       constexpr bool SCALE = decltype(scaled)::value;
-      for (int item = tid; item < NQ * NI * W2; item += PL::THREADS) {
-        const int m = item / (NI * W2);
-        int f, lp;
-        tile_split<D, W2>(item - m * NI * W2, NI, f, lp);
+      const unsigned rcp_ni = c_rcp20.v[ni];
+      for (int item = tid; item < NQ * ni * W2; item += PL::THREADS) {
+        int m, f, lp;
+        item_split<D, W2>(item, ni, rcp_ni, m, f, lp);
         const float4* S = reinterpret_cast<const float4*>(sm + PL::OFF_S) + m * NW * W2;
         const float4* G = reinterpret_cast<const float4*>(sm + PL::OFF_G) + m * PL::NG * W2;
         const float4* b = reinterpret_cast<const float4*>(sm + PL::OFF_B) + m * 3 * NW * W2;
@@ -424,10 +428,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
     else
       phase_c(std::false_type{});
     cp_async_wait_all();  // this thread's ROE / FV copies; the barrier publishes them
-    if (tid >= PF0) {  // velocities to double-float, in place (sqrt(rho) and H arrive as
+    if (pf >= 0) {  // velocities to double-float, in place (sqrt(rho) and H arrive as
                        // double-float: planes of the NS3D_FP64 primitive layout)
       int pos, line;
-      tile_split<D, W>(tid - PF0, NP, pos, line);
+      item_split<D, W>(pf, np, c_rcp20.v[np], pos, line);
       double* r = sm + PL::OFF_ROE + tile_idx<D, W>(pos, line, NP);
 #pragma unroll
       for (int k = 1; k < 4; ++k) {
@@ -446,10 +450,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
   static_assert(PL::TP * PL::W <= PL::THREADS, "one epilogue point per thread");
   static_assert(15 * PL::TP * PL::W <= NQ * 3 * PL::NW * PL::W, "prefetch slots fit the indicator space");
   double* pre = sm + PL::OFF_B + 15 * tid;
-  if (tid < TP * W) {
+  if (tid < len * W) {
     int pp, line;
-    tile_split<D, W>(tid, TP, pp, line);
-    if (s0 + pp < nD && a0 + line < na) epilogue_prefetch(a, flat(s0 + pp, a0 + line), pre);
+    item_split<D, W>(tid, len, c_rcp20.v[len], pp, line);
+    if (a0 + line < na) epilogue_prefetch(a, flat(s0 + pp, a0 + line), pre);
   }
   cp_async_commit();
 
@@ -459,9 +463,9 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
     const double* r = sm + PL::OFF_ROE;
     double* rec = sm + PL::OFF_R;
     int bad = 0, range_bad = 0;
-    for (int item = tid; item < NI * W; item += PL::THREADS) {
+    for (int item = tid; item < ni * W; item += PL::THREADS) {
       int f, line;
-      tile_split<D, W>(item, NI, f, line);
+      item_split<D, W>(item, ni, c_rcp20.v[ni], f, line);
       const int o = tile_idx<D, W>(f, line, NI);
       const int sa = tile_idx<D, W>(f + 2, line, NP), sb = tile_idx<D, W>(f + 3, line, NP);
       if (MODE == 1) {
@@ -614,10 +618,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int tx, i
     const double r12 = a.g.r12h[D];
     const double* F = sm + PL::OFF_R;
     const double* fvs = sm + PL::OFF_FV;
-    for (int item = tid; item < TP * W; item += PL::THREADS) {
+    for (int item = tid; item < len * W; item += PL::THREADS) {
       int pp, line;
-      tile_split<D, W>(item, TP, pp, line);
-      if (s0 + pp >= nD || a0 + line >= na) continue;
+      item_split<D, W>(item, len, c_rcp20.v[len], pp, line);
+      if (a0 + line >= na) continue;
       double cv[5];
       const int op = tile_idx<D, W>(pp + 1, line, NI), om = tile_idx<D, W>(pp, line, NI);
       if (MODE == 1) {  // interface fluxes already divided by dx; viscous fluxes double-float

@@ -41,6 +41,7 @@ DirArgs base_args(ns3d_ctx* c, const double* u) {
   a.mode = (c->p.precision == NS3D_FP64_STRICT) ? 0 : (c->p.precision == NS3D_FP32_BULK) ? 2 : 1;
   a.variant = c->variant;
   a.t0 = 0;
+  a.tile_u = a.tile_r = 0;
   a.zorder = (c->zorder >= 0) ? c->zorder : dir_zorder(c->g);
   const double c133 = 13.0 / 3.0, eps4 = 4.0 * c->p.weno_eps;
   a.c133_hi = (float)c133;
@@ -141,7 +142,8 @@ int rhs_pass(ns3d_ctx* c, const double* u, int epi, double* out, const double* u
   // on the copy stream while the next slabs compute
   for (int j = 0; j < pout->n; ++j) {
     if ((rc = dir(2, pout->lo[j], pout->lo[j + 1]))) return rc;
-    const int z0 = pout->lo[j] * pout->tp, z1 = min(pout->lo[j + 1] * pout->tp, g.n[2]);
+    const int z0 = dir_tile_start(g, 2, a.mode, a.variant, pout->lo[j]);
+    const int z1 = dir_tile_start(g, 2, a.mode, a.variant, pout->lo[j + 1]);
     cudaError_t e = cudaEventRecord(pout->ev[j], c->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_stream, pout->ev[j], 0);
     for (int v = 0; v < 5 && e == cudaSuccess; ++v) {
@@ -522,7 +524,6 @@ int ns3d_step_host(ns3d_ctx* c, double* u_host, double dt, int nsteps, ns3d_stat
     slab_bounds(pout, min(ztiles, (int)ns3d_ctx::MAX_SLABS), ztiles, 1, ztiles);
     pout.ev = c->slab_ev + ns3d_ctx::MAX_SLABS;
     pout.host = u_host;
-    pout.tp = tp;
     cudaEvent_t entry = c->slab_ev[2 * ns3d_ctx::MAX_SLABS];
     e = cudaEventRecord(entry, c->stream);  // the copies follow the work already on the stream
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->copy_stream, entry, 0);

@@ -105,7 +105,10 @@ __device__ __forceinline__ void phase_dir(const BatchView& b, int s, double* sm,
     const long long r = lt / ntx;
     const int ty = (int)(r % nty);
     const int tz = (int)(r / nty);
-    dir_tile<D, MODE, TP, W, NC>(in.dir[s][D], sm, tx, ty, tz);
+    int u, rr, s0, len;
+    tile_split_units(D, in.g.n[D], ntx, u, rr);
+    tile_span(D, in.g.n[D], u, rr, tx, s0, len);
+    dir_tile<D, MODE, TP, W, NC>(in.dir[s][D], sm, s0, len, ty, tz);
     __syncthreads();  // the next tile reuses the shared memory
   }
 }

@@ -125,7 +125,6 @@ struct SlabPipe {
   int lo[ns3d_ctx::MAX_SLABS + 1] = {};
   cudaEvent_t* ev = nullptr;  // ev[j]: slab j is on the device (in) / final on the device (out)
   double* host = nullptr;     // out: destination of the slabs ([5][N] like the device state)
-  int tp = 0;                 // out: points along z of a z-pass tile
 };
 // One right-hand-side evaluation of u with the given z-pass epilogue (ns3d_api.cu).  pin: u arrives
 // slab by slab (the primitive, viscous, x and y kernels run per slab after its event); pout: the z

@@ -62,16 +62,38 @@ def test_stats_minima_of_bad_states(ns3d):
 @pytest.mark.parametrize("nx,ny,nz", [(33, 9, 70), (21, 40, 131), (640, 256, 3), (40, 24, 1)])
 def test_viscous_chunks(ns3d, orc, nx, ny, nz):
     u = I.random_smooth(nx, ny, nz, seed=6, amp=0.1, mach=0.4)
-    ref = orc.rhs(orc.Params(nx, ny, nz, mu_eff=0.02), u)
+    ref = orc.rhs(orc.Params(nx, ny, nz, mu_eff=1e-4), u)
     out = []
     for storage in (1, 2):
-        s = ns3d.Solver(nx, ny, nz, mu_eff=0.02, storage=storage)
+        s = ns3d.Solver(nx, ny, nz, mu_eff=1e-4, storage=storage)
         out.append(s.rhs(_gpu(u)).cpu().numpy())
         s.close()
-    assert rel_err(out[0], ref) <= 1e-12  # the tolerance of one right-hand side
+    # mu is small because the composite second difference amplifies the double-float rounding of the
+    # temperature (a few 2^-48) by (18/12)^2 / dx^2, times kappa = mu / (0.4 * 0.72): at 640 points and
+    # mu = 1e-4 that is 3.5e-4 * 4 * 3.6e-15 * 2.25 * 1.04e4 = 1.2e-13, below the 1e-12 of a right-hand
+    # side (max |R| is 2)
+    assert rel_err(out[0], ref) <= 1e-12
     assert np.array_equal(out[0], out[1])
-    s = ns3d.Solver(nx, ny, nz, mu_eff=0.02, precision=1)
+    s = ns3d.Solver(nx, ny, nz, mu_eff=1e-4, precision=1)
     r32 = s.rhs(_gpu(u)).cpu().numpy()
     s.close()
     # FP32 fluxes: 1e-5 of the flux scale over the smallest spacing (as the FP32-bulk tests)
     assert np.abs(r32 - ref).max() <= 1e-5 * flux_scale(u, (2 * np.pi,) * 3)
+
+
+# lines shorter than a tile, one point over one and two tiles, one-point lines, lengths that are no
+# multiple of 4 (x tiles start on 32-byte sectors), wide remainders; every tile shape, both FP64 modes
+@pytest.mark.parametrize("nx,ny,nz", [(25, 49, 33), (32, 23, 7), (1, 26, 5), (47, 3, 64), (73, 17, 25), (2, 41, 97)])
+def test_balanced_tiles(ns3d, orc, nx, ny, nz):
+    u = I.random_smooth(nx, ny, nz, seed=7, amp=0.1, mach=0.5)
+    ref = orc.rhs(orc.Params(nx, ny, nz, mu_eff=0.003), u)
+    for prec, variants in ((0, (0, 1, 2)), (2, (0,))):
+        out = []
+        for v in variants:
+            s = ns3d.Solver(nx, ny, nz, mu_eff=0.003, precision=prec)
+            ns3d.set_solver_variant(s, v)
+            out.append(s.rhs(_gpu(u)).cpu().numpy())
+            s.close()
+            assert rel_err(out[-1], ref) <= 1e-12, (prec, v)
+            assert np.array_equal(out[0], out[-1]), (prec, v)
+
