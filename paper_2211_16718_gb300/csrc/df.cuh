@@ -171,6 +171,20 @@ __device__ __forceinline__ df df_div(df x, df y) {
   return fast_two_sum(q1, q2);
 }
 
+// The same with the reciprocal seed refined once (two more FMAs): the remainder is then multiplied
+// by a reciprocal of error 2^-24 instead of up to 2^-23, and the error falls to about 2^-47.5.
+__device__ __forceinline__ df df_div_r(df x, df y) {
+  float r = rcp_seed(y.hi);
+  r = __fmaf_rn(r, __fmaf_rn(-y.hi, r, 1.0f), r);
+  const float q1 = __fmul_rn(x.hi, r);
+  df p = two_prod(q1, y.hi);
+  float rem = __fsub_rn(x.hi, p.hi);
+  rem = __fsub_rn(rem, p.lo);
+  rem = __fadd_rn(rem, x.lo);
+  rem = __fmaf_rn(-q1, y.lo, rem);
+  return fast_two_sum(q1, __fmul_rn(rem, r));
+}
+
 // Square root of a positive double-word (hi a normal float): float seed r, one
 // correction (x - r^2)/(2r) with the exact square of the seed (Dekker's method).
 __device__ __forceinline__ df df_sqrt(df x) {
@@ -180,6 +194,20 @@ __device__ __forceinline__ df df_sqrt(df x) {
   d = __fsub_rn(d, p.lo);
   d = __fadd_rn(d, x.lo);
   return fast_two_sum(r, __fmul_rn(d, __fmul_rn(0.5f, rcp_seed(r))));
+}
+
+// The same with the reciprocal in the correction refined once and the correction's second-order
+// term -q^2/(2r) added (five more operations): the seed's error then enters with its cube.
+__device__ __forceinline__ df df_sqrt_r(df x) {
+  const float r = sqrt_seed(x.hi);
+  const df p = two_prod(r, r);
+  float d = __fsub_rn(x.hi, p.hi);
+  d = __fsub_rn(d, p.lo);
+  d = __fadd_rn(d, x.lo);
+  float y = rcp_seed(r);
+  y = __fmul_rn(0.5f, __fmaf_rn(y, __fmaf_rn(-r, y, 1.0f), y));
+  const float q = __fmul_rn(d, y);
+  return fast_two_sum(r, __fmaf_rn(-__fmul_rn(q, q), y, q));
 }
 
 __device__ __forceinline__ df df_abs(df x) { return (x.hi < 0.0f) ? df_neg(x) : x; }

@@ -26,14 +26,12 @@
 // MODE 0 (all FP64): fhat = sum_k omega_k F_k with one FP64 division.
 // MODE 1 (FP64 values, double-float weights): since sum omega = 1,
 //   fhat = F_2 + omega_1 (F_1 - F_2) + omega_3 (F_3 - F_2),
-// where F_1 - F_2 and F_3 - F_2 are third differences of the data (FP64, from the
-// window second differences s) and the weights, which only multiply these small
+// where F_1 - F_2 and F_3 - F_2 are third differences of the data and the weights, which only multiply these small
 // differences, are evaluated in double-float arithmetic (~48 bits) on the FP32
 // pipe.  The reconstructed values themselves are never formed: the Roe flux needs
-// fhat_L + fhat_R = P_i + P_{i+1} + (dL + dR) and the jump fhat_R - fhat_L =
-// (P_{i+1} - P_i) + dR - dL, both kept in double-float, so the FP64 pipe sees
-// only the first differences, the point sums and one combination per flux
-// component.  The result agrees with the all-FP64 evaluation to rounding.
+// fhat_L + fhat_R and the jump fhat_R - fhat_L, whose linear parts combine (phase C),
+// both kept in double-float, so the FP64 pipe sees only the first differences, the
+// point sums and one combination per flux component.  The result agrees with the all-FP64 evaluation to rounding.
 // Phases A2, B and C of MODE 1 take two lines of the tile per item and run their
 // double-float arithmetic on both at once with the packed FP32 instructions
 // (df2.cuh): each lane computes what a one-line evaluation would, with half the
@@ -113,26 +111,36 @@ __device__ __forceinline__ double weno_combine(double B1, double B2, double B3, 
   return num / den;
 }
 
-// Range of the squared indicators inside which df2_offset needs no rescaling: products of
-// two stay below 2^80, so that they times a third difference (below 2^12 for such tiles,
-// since |third difference| <= 4 |first differences| <= 4 B^(1/4)) and the denominator times
-// the candidate difference stay inside the float range; and above 2^-100, so that their
-// TwoProd error terms stay normal floats and the products keep full precision.
-constexpr float DFW_LO = 0x1p-50f, DFW_HI = 0x1p40f;
+// Range of the scaled indicators b_k inside which df2_offset3 needs no rescaling of the B_k = b_k^2:
+// products of two B_k stay below 2^80, so that they times a third difference (below 2^12 for such
+// tiles, since |third difference| <= 4 |first differences| <= 4 b^(1/2)) stay inside the float
+// range; and above 2^-100, so that their TwoProd error terms stay normal floats and the products
+// keep full precision.  b_k >= 4 eps, so the lower end is a condition on eps alone (with a margin
+// for the rounding of b_k).
+constexpr float DFB_LO = 0x1.01p-25f, DFB_HI = 0x1p20f;
 
-// Offset of one reconstruction from its candidate-2 value, in double-float, from the three
-// squared scaled indicators B_k (candidate order 1, 2, 3) and three differences:
-//   d = e/6 + omega_1/3 * ta + omega_3/6 * tb,   omega_k = c_k prod_{m!=k} B_m / den,
-// over the common denominator 6 den = 6 (B2 B3 + 6 B1 B3 + 3 B1 B2):
-//   d = [den * e + 2 B2 B3 * ta + 3 B1 B2 * tb] / (6 den)        (one division).
-// Left-biased: e = 2 g2 + g1, ta = s0 - s1, tb = s1 - s2; right-biased (mirrored):
-// e = -(2 g2 + g3), ta = s3 - s2, tb = -(s1 - s2).
+// 1/6 as a double-float.
+__device__ __forceinline__ df2 df2_sixth() {
+  constexpr float hi = (float)(1.0 / 6.0), lo = (float)(1.0 / 6.0 - (double)hi);
+  return df2_splat(df{hi, lo});
+}
+
+// Offset omega_1 (F_1 - F_2) + omega_3 (F_3 - F_2) of one reconstruction from its candidate 2, in
+// double-float, from the three squared scaled indicators B_k (candidate order 1, 2, 3) and the third
+// differences ta = 3 (F_1 - F_2), tb = 6 (F_3 - F_2), both given divided by 6; with
+// omega_k = c_k prod_{m!=k} B_m / den and den = B2 B3 + 6 B1 B3 + 3 B1 B2,
+//   d = B2 [2 B3 ta/6 + 3 B1 tb/6] / [B2 B3 + 3 B1 (2 B3 + B2)]        (one division).
 // SCALE: rescale the B_k by a common power of two first (the weights are scale-free);
-// without it every B_k must lie in [DFW_LO, DFW_HI).
+// without it every B_k must lie in [DFB_LO^2, DFB_HI^2).
+// The numerator and denominator are renormalised and the division's seed refined (8 of the 71 packed
+// operations): at a jump the offsets are a third of it, and their rounding is what is left of the
+// reconstruction's error there.  In units of 2^-48 of the largest difference, against long double:
+// a jump of 0.9 in noise of 0.01 1.7 (1.5 for the form over the common denominator that includes the
+// linear part, 3.8 without these), random differences 1.0 (4.5), smooth data below 0.1 (5.6).
 // Evaluated for two lines at once (two-lane double-float; each lane exactly as the
 // one-lane evaluation, its scale chosen from its own B_k).
 template <bool SCALE = true>
-__device__ __forceinline__ df2 df2_offset(df2 B1, df2 B2, df2 B3, df2 e, df2 ta, df2 tb) {
+__device__ __forceinline__ df2 df2_offset3(df2 B1, df2 B2, df2 B3, df2 ta6, df2 tb6) {
   if (SCALE) {
     const int E0 = max(exponent_of(B1.hi.x), max(exponent_of(B2.hi.x), exponent_of(B3.hi.x)));
     const int E1 = max(exponent_of(B1.hi.y), max(exponent_of(B2.hi.y), exponent_of(B3.hi.y)));
@@ -141,6 +149,19 @@ __device__ __forceinline__ df2 df2_offset(df2 B1, df2 B2, df2 B3, df2 e, df2 ta,
     B2 = df2_scale(B2, sc);
     B3 = df2_scale(B3, sc);
   }
+  const df2 b1 = df2_mul_f_u(B1, 3.0f), b3 = df2_twice(B3);
+  const df2 den = df2_add_pos_u(df2_mul_u(B2, B3), df2_mul_u(b1, df2_add_pos_u(b3, B2)));
+  const df2 num = df2_mul(B2, df2_add_fast(df2_mul_u(b3, ta6), df2_mul_u(b1, tb6)));
+  return df2_div_ru(num, fast_two_sum2(den.hi, den.lo));
+}
+
+// The same reconstruction as an offset from the point value, its linear part e/6 over the common
+// denominator 6 den: d = [den e + 2 B2 B3 ta + 3 B1 B2 tb] / (6 den), for B_k that need no rescaling.
+// The direction pass used this form until its linear parts were combined across the interface
+// (phase C); it stays as the composition that the two-lane check compares with scalar code.
+template <bool SCALE>
+__device__ __forceinline__ df2 df2_offset(df2 B1, df2 B2, df2 B3, df2 e, df2 ta, df2 tb) {
+  static_assert(!SCALE, "unscaled form only");
   const df2 p23 = df2_mul_u(B2, B3);
   const df2 p13 = df2_mul_u(B1, B3);
   const df2 p12 = df2_mul_u(B1, B2);
@@ -296,55 +317,65 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       bw[(m * 3 + 2) * NW * W + o] = b3 * b3;
     }
   } else {
-    // one item per line pair: two-lane double-float arithmetic (packed FP32 instructions)
+    // one item per line pair and two adjacent windows: two-lane double-float arithmetic (packed FP32
+    // instructions); the windows share a second difference, and a 24-point tile has 252 items for
+    // its 256 threads
     int range_bad = 0;
+    need_scale = !(a.eps4_hi >= DFB_LO);
     float4* bw = reinterpret_cast<float4*>(sm + PL::OFF_B);
     float4* S = reinterpret_cast<float4*>(sm + PL::OFF_S);
     const df2 c133 = df2_splat(df{a.c133_hi, a.c133_lo});
     const df2 eps4 = df2_splat(df{a.eps4_hi, a.eps4_lo});
-    const unsigned rcp_nw = c_rcp20.v[nw];
-    for (int item = tid; item < NQ * nw * W2; item += PL::THREADS) {
-      int m, w, lp;
-      item_split<D, W2>(item, nw, rcp_nw, m, w, lp);
-      const int o = tile_idx<D, W2>(w, lp, NW);
+    const int nw2 = (nw + 1) / 2;
+    const unsigned rcp_nw2 = c_rcp20.v[nw2];
+    for (int item = tid; item < NQ * nw2 * W2; item += PL::THREADS) {
+      int m, w2, lp;
+      item_split<D, W2>(item, nw2, rcp_nw2, m, w2, lp);
       const float4* G = reinterpret_cast<const float4*>(sm + PL::OFF_G) + m * PL::NG * W2;
-      const df2 dgm = df2_from4(G[tile_idx<D, W2>(w, lp, PL::NG)]);
-      const df2 dgp = df2_from4(G[tile_idx<D, W2>(w + 1, lp, PL::NG)]);
-      const df2 ds = df2_add_fast(dgp, df2_neg(dgm));  // second difference s_w
-      // third difference T_w = s_w - s_{w+1} (phase C needs T_f, T_{f+1}, T_{f+2}; the last
-      // window has no s_{w+1} in the tile and its T is never read)
-      df2 T{f2splat(0.0f), f2splat(0.0f)};
-      if (w + 1 < nw) {
-        const df2 g2 = df2_from4(G[tile_idx<D, W2>(w + 2, lp, PL::NG)]);
-        T = df2_add_fast(ds, df2_neg(df2_add_fast(g2, df2_neg(dgp))));
+      auto ldG = [&](int j) { return df2_from4(G[tile_idx<D, W2>(j, lp, PL::NG)]); };
+      df2 g0 = ldG(2 * w2), g1 = ldG(2 * w2 + 1);
+      df2 s0 = df2_add_fast(g1, df2_neg(g0));  // second difference of the window
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int w = 2 * w2 + k;
+        if (w >= nw) break;
+        const int o = tile_idx<D, W2>(w, lp, NW);
+        // third difference T_w = s_w - s_{w+1}, divided by 6 (phase C needs T_f, T_{f+1}, T_{f+2}; the
+        // last window has no s_{w+1} in the tile and its T is never read)
+        const df2 g2 = ldG(min(w + 2, len + 4));
+        const df2 s1 = df2_add_fast(g2, df2_neg(g1));
+        S[m * NW * W2 + o] = df2_to4(df2_mul_u(df2_add_fast(s0, df2_neg(s1)), df2_sixth()));
+        // scaled indicators b_k = u_k^2 + aa, aa = (13/3) s^2 + 4 eps, with u_2 = z - x and
+        // u_1 = x - 4y + 3z = u_2 + 2s, u_3 = 3x - 4y + z = 2s - u_2:
+        //   b_2 = u_2^2 + aa,  b_{1,3} = (b_2 + 4 s^2) +- 4 u_2 s   (b_k >= aa >= (13/3) s^2, so
+        // b_2 + 4 s^2 <= ~3 b_{1,3}: no harmful cancellation)
+        const df2 s2 = df2_sqr_u(s0);
+        const df2 aa = df2_add_pos_u(df2_mul_u(s2, c133), eps4);
+        const df2 u2 = df2_add_fast(g0, g1);
+        const df2 b2 = df2_add_pos_u(df2_sqr_u(u2), aa);
+        // Fast2Sum order with margins: b_2 >= aa >= (13/12) 4 s^2, and
+        // pq = u_2^2 + (4 + 13/3) s^2 + 4 eps >= 1.44 |4 u_2 s| (minimum over u_2)
+        const float2 four = f2splat(4.0f);
+        const df2 pq = df2_add_ordered_u(b2, df2_scale(s2, four));
+        const df2 r4 = df2_scale(df2_mul_u(u2, s0), four);
+        const df2 B1 = df2_sqr_u(df2_add_ordered(pq, r4));
+        const df2 B2 = df2_sqr_u(b2);
+        const df2 B3 = df2_sqr_u(df2_add_ordered(pq, df2_neg(r4)));
+        bw[(m * 3 + 0) * NW * W2 + o] = df2_to4(B1);
+        bw[(m * 3 + 1) * NW * W2 + o] = df2_to4(B2);
+        bw[(m * 3 + 2) * NW * W2 + o] = df2_to4(B3);
+        // every b_k of both lanes is at most the sum of the lanes' pq + |r4|.  The float exponent
+        // range bounds the indicators (differences of the data up to ~1e9); beyond it the host
+        // reports NS3D_ERANGE instead of a NaN
+        if (!((pq.hi.x + fabsf(r4.hi.x)) + (pq.hi.y + fabsf(r4.hi.y)) < DFB_HI)) {
+          need_scale = 1;
+          range_bad |= !(fmaxf(B1.hi.x, fmaxf(B2.hi.x, B3.hi.x)) < 1e36f) ||
+                       !(fmaxf(B1.hi.y, fmaxf(B2.hi.y, B3.hi.y)) < 1e36f);
+        }
+        g0 = g1;
+        g1 = g2;
+        s0 = s1;
       }
-      S[m * NW * W2 + o] = df2_to4(T);
-      // scaled indicators b_k = u_k^2 + aa, aa = (13/3) s^2 + 4 eps, with u_2 = z - x and
-      // u_1 = x - 4y + 3z = u_2 + 2s, u_3 = 3x - 4y + z = 2s - u_2:
-      //   b_2 = u_2^2 + aa,  b_{1,3} = (b_2 + 4 s^2) +- 4 u_2 s   (b_k >= aa >= (13/3) s^2, so
-      // b_2 + 4 s^2 <= ~3 b_{1,3}: no harmful cancellation)
-      const df2 s2 = df2_sqr_u(ds);
-      const df2 aa = df2_add_pos_u(df2_mul_u(s2, c133), eps4);
-      const df2 u2 = df2_add_fast(dgm, dgp);
-      const df2 b2 = df2_add_pos_u(df2_sqr_u(u2), aa);
-      // Fast2Sum order with margins: b_2 >= aa >= (13/12) 4 s^2, and
-      // pq = u_2^2 + (4 + 13/3) s^2 + 4 eps >= 1.44 |4 u_2 s| (minimum over u_2)
-      const df2 pq = df2_add_ordered_u(b2, df2_twice(df2_twice(s2)));
-      const df2 r4 = df2_twice(df2_twice(df2_mul_u(u2, ds)));
-      const df2 B1 = df2_sqr_u(df2_add_ordered(pq, r4));
-      const df2 B2 = df2_sqr_u(b2);
-      const df2 B3 = df2_sqr_u(df2_add_ordered(pq, df2_neg(r4)));
-      bw[(m * 3 + 0) * NW * W2 + o] = df2_to4(B1);
-      bw[(m * 3 + 1) * NW * W2 + o] = df2_to4(B2);
-      bw[(m * 3 + 2) * NW * W2 + o] = df2_to4(B3);
-      // the float exponent range bounds the indicators (differences of the data
-      // up to ~1e9); beyond it the host reports NS3D_ERANGE instead of a NaN
-      const float bmax0 = fmaxf(B1.hi.x, fmaxf(B2.hi.x, B3.hi.x));
-      const float bmax1 = fmaxf(B1.hi.y, fmaxf(B2.hi.y, B3.hi.y));
-      const float bmin0 = fminf(B1.hi.x, fminf(B2.hi.x, B3.hi.x));
-      const float bmin1 = fminf(B1.hi.y, fminf(B2.hi.y, B3.hi.y));
-      range_bad |= !(bmax0 < 1e36f) || !(bmax1 < 1e36f);
-      need_scale |= !(bmax0 < DFW_HI && bmin0 >= DFW_LO && bmax1 < DFW_HI && bmin1 >= DFW_LO);
     }
     if (__any_sync(0xffffffffu, range_bad) && (tid & 31) == 0) atomicOr(a.status, ST_DF_RANGE);
   }
@@ -380,14 +411,12 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       rec[(2 * m + 1) * NI * W + o] = weno_combine(B3f3, B2f2, B1f1, xL, eL, eR);
     }
   } else {
-    // fhat_L = P2 + dL, fhat_R = P3 + dR with the offsets (differences only)
-    //   dL =  (2 g2 + g1)/6 + w1 (s0 - s1) + w3 (s1 - s2)      [w1 = omega_1/3, w3 = omega_3/6]
-    //   dR = -(2 g2 + g3)/6 + v1 (s3 - s2) - v3 (s1 - s2)
-    // (candidate 2 minus the point value, and F1 - F2, F3 - F2 as third differences),
-    // evaluated in double-float on the FP32 pipe.  The interface values are never
-    // formed in FP64: the Roe flux needs only
-    //   du    = g2 + dR - dL       (fhat_R - fhat_L, for the u-scalars; double-float)
-    //   fhat_L + fhat_R = 2 P2 + (g2 + dL + dR)   (for the flux scalars; FP64)
+    // fhat_L = P2 + (2 g2 + g1)/6 + oL, fhat_R = P3 - (2 g2 + g3)/6 - oR: candidate 2 and the
+    // nonlinear offsets of df2_offset3 (oR with its sign reversed, so that both use +T), from the
+    // third differences T_f, T_{f+1}, T_{f+2} of phase B.  Evaluated in double-float on the FP32
+    // pipe.  The interface values are never formed in FP64, and the linear parts combine:
+    //   fhat_R - fhat_L = T_{f+1}/6 - (oL + oR)                          (u-scalars; double-float)
+    //   fhat_L + fhat_R = 2 P2 + [g2 + (g1 - g3)/6 + (oL - oR)]          (flux scalars; FP64)
     // One item per line pair, in two-lane double-float arithmetic.
     float2* rf = reinterpret_cast<float2*>(sm + PL::OFF_R);
     auto phase_c = [&](auto scaled) {
@@ -402,21 +431,18 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         auto ldS = [&](int w) { return df2_from4(S[tile_idx<D, W2>(w, lp, NW)]); };
         auto ldG = [&](int j) { return df2_from4(G[tile_idx<D, W2>(j, lp, PL::NG)]); };
         auto ld = [&](int k, int w) { return df2_from4(b[k * NW * W2 + tile_idx<D, W2>(w, lp, NW)]); };
-        // third differences (phase B): s0 - s1 = T_f, s1 - s2 = T_{f+1}, s3 - s2 = -T_{f+2}
-        const df2 t0 = ldS(f), tC = ldS(f + 1), t2 = df2_neg(ldS(f + 2));
-        const df2 g1 = ldG(f + 1), g2 = ldG(f + 2), g3 = ldG(f + 3);
-        const df2 g22 = df2_twice(g2);
-        const df2 dL = df2_offset<SCALE>(ld(0, f), ld(1, f + 1), ld(2, f + 2), df2_add_fast(g22, g1), t0, tC);
-        const df2 dR = df2_offset<SCALE>(ld(2, f + 3), ld(1, f + 2), ld(0, f + 1), df2_neg(df2_add_fast(g22, g3)), t2,
-                                         df2_neg(tC));
+        const df2 T1 = ldS(f + 1);
+        const df2 oL = df2_offset3<SCALE>(ld(0, f), ld(1, f + 1), ld(2, f + 2), ldS(f), T1);
+        const df2 oR = df2_offset3<SCALE>(ld(2, f + 3), ld(1, f + 2), ld(0, f + 1), ldS(f + 2), T1);
         const int o0 = tile_idx<D, W>(f, 2 * lp, NI), o1 = tile_idx<D, W>(f, 2 * lp + 1, NI);
         if (m < 5) {
-          const df2 du = df2_add_fast(g2, df2_add_fast(dR, df2_neg(dL)));
+          const df2 du = df2_add_fast(T1, df2_neg(df2_add_fast(oL, oR)));
           rf[m * NI * W + o0] = make_float2(du.hi.x, du.lo.x);
           rf[m * NI * W + o1] = make_float2(du.hi.y, du.lo.y);
         }
-        if (m >= 4) {  // flux scalar: fhat_L + fhat_R = 2 P2 + (g2 + dL + dR), P2 copied in phase A2
-          const df2 t = df2_add_fast(g2, df2_add_fast(dL, dR));
+        if (m >= 4) {  // flux scalar; P2 copied in phase A2
+          const df2 lin = df2_add_fast(ldG(f + 2), df2_mul_u(df2_add_fast(ldG(f + 1), df2_neg(ldG(f + 3))), df2_sixth()));
+          const df2 t = df2_add_fast(lin, df2_add_fast(oL, df2_neg(oR)));
           double* F = sm + PL::OFF_R + (1 + m) * NI * W;
           F[o0] = fma(2.0, F[o0], f2d_bits(t.hi.x)) + f2d_bits(t.lo.x);
           F[o1] = fma(2.0, F[o1], f2d_bits(t.hi.y)) + f2d_bits(t.lo.y);
@@ -486,7 +512,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         }
         const df ra = ldr(0, sa), rb = ldr(0, sb);
         const df rsum = df_add_pos(ra, rb);
-        const df rs = df_div(df{1.0f, 0.0f}, rsum);
+        const df rs = df_div_r(df{1.0f, 0.0f}, rsum);  // refined, as 1/c and c below: at jumps their errors lead
         const df wa = df_mul_u(ra, rs), wb = df_mul_u(rb, rs);
         df V[3];
 #pragma unroll
@@ -497,8 +523,8 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         const df c2 = df_mul(df_add_fast(H, df_neg(q2h)), df{a.gm1_hi, a.gm1_lo});
         bad |= !(c2.hi > 0.0f);
         range_bad |= !(c2.hi > 1e-30f && c2.hi < 1e30f && rsum.hi > 1e-30f && rsum.hi < 1e30f);
-        const df c = df_sqrt(c2);
-        const df rc = df_div(df{1.0f, 0.0f}, c);
+        const df c = df_sqrt_r(c2);
+        const df rc = df_div_r(df{1.0f, 0.0f}, c);
         constexpr int T1 = (D == 0) ? 1 : 0;
         constexpr int T2 = (D == 2) ? 1 : 2;
         const df un = V[D], vt1 = V[T1], vt2 = V[T2];
