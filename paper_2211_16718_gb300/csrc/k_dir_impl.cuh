@@ -57,14 +57,15 @@ constexpr int NQ = 9;             // reconstructed scalars
 //   MODE 0: Q [NQ][NP*W] point values, ROE [5][NP*W] sqrt(rho), u, v, w, H,
 //           FV [4][NP*W] viscous flux, B [NQ][3][NW*W] squared indicators,
 //           R [18][NI*W] interface values, later [5][NI*W] interface fluxes.
-//   MODE 1: Q [NQ][NP*W], dead after phase A2: ROE [5][NP*W] and FV [4][NP*W] then
-//           arrive there by cp.async (as FP64) while phases B and C run;
-//           B [NQ][3][NW*W/2] squared indicators, dead after phase C: the epilogue
-//           operands then arrive there; S [NQ][NW*W/2] third differences;
+//   MODE 1: Q [NQ][NP*W], dead after phase A2: ROE [5][NR*W] then arrives there by cp.async (as
+//           FP64) while phases B and C run, and phase C puts T [5][NI*W] behind it, the double-float
+//           part of fhat_L + fhat_R of the five flux scalars;
+//           B [NQ][3][NW*W/2] squared indicators, dead after phase C: the epilogue operands and
+//           FV [4][NV*W] then arrive there; S [NQ][NW*W/2] third differences;
 //           G [NQ][NG*W/2] first differences (B, S, G: double-float values of the two
 //           lines of a line pair side by side, 16 bytes (hi0, hi1, lo0, lo1), indexed
 //           like the lines with W/2 line pairs); R [10][NI*W]: jumps du of u_0..u_4
-//           (double-float, slots 0-4) and the sums of the five flux scalars
+//           (double-float, slots 0-4) and the left point values of the five flux scalars
 //           (FP64, slots 5-9), later [5][NI*W] interface fluxes.
 //   The MODE 1 plan of a 24 x 4 tile is 57.2 KB, so that four CTAs of 256 threads
 //   (64 registers) share an SM.  MODE 1 tiles have an even number of lines.
@@ -78,17 +79,26 @@ struct Plan {
   static constexpr int NW = TP + 4;                 // 3-point windows centred at -2 .. TP+1
   static constexpr int NI = TP + 1;                 // interfaces -1/2 .. TP-1/2
   static constexpr int NG = NP - 1;                 // first differences
+  static constexpr int NR = (MODE == 1) ? TP + 2 : NP;  // Roe-average inputs: the interfaces' own points
+  static constexpr int NV = (MODE == 1) ? TP + 4 : NP;  // viscous flux: 2-point halo
   static constexpr int OFF_Q = 0;
   static constexpr int OFF_ROE = (MODE == 1) ? OFF_Q : OFF_Q + NQ * NP * W;
-  static constexpr int OFF_FV = OFF_ROE + 5 * NP * W;
-  static constexpr int OFF_B = (MODE == 1) ? OFF_Q + NQ * NP * W : OFF_FV + 4 * NP * W;
+  static constexpr int OFF_T = OFF_ROE + 5 * NR * W;    // MODE 1
+  static constexpr int END_T = OFF_T + 5 * NI * W;
+  static constexpr int OFF_B = (MODE == 0)          ? OFF_ROE + (5 + 4) * NP * W
+                               : (END_T > NQ * NP * W) ? (END_T + 1) / 2 * 2
+                                                       : OFF_Q + NQ * NP * W;
+  static constexpr int OFF_FV = (MODE == 1) ? OFF_B + 15 * TP * W : OFF_ROE + 5 * NP * W;
   static constexpr int OFF_S = OFF_B + NQ * 3 * NW * W;  // MODE 1: third differences
   static constexpr int OFF_G = OFF_S + (MODE == 1 ? NQ * NW * W : 0);
   static constexpr int OFF_R = OFF_G + (MODE == 1 ? NQ * NG * W : 0);
   static constexpr int R_SLOTS = (MODE == 1) ? 10 : 18;
   static constexpr int WORDS = OFF_R + R_SLOTS * NI * W;
   static constexpr int BYTES = WORDS * 8;
-  static_assert(MODE == 0 || OFF_FV + 4 * NP * W <= OFF_B, "ROE and FV fit the dead point values");
+  static_assert(MODE == 0 || OFF_FV + 4 * NV * W <= OFF_S, "epilogue operands and FV fit the dead indicators");
+  // MODE 1: the threads that fetch the epilogue operands and FV while the others run phase D
+  static constexpr int FETCH0 = THREADS / 2;
+  static_assert(MODE == 0 || (NI * W <= FETCH0 && NV * W <= THREADS - FETCH0), "phase D and the fetches side by side");
 };
 
 // Index of conserved component c among the reconstructed scalars.  MODE 0 keeps
@@ -243,7 +253,9 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
 
   // ---- A2 (MODE 1): first differences g_j = q_{j+1} - q_j in FP64, kept as double-float,
   //      and the point values q_j of the five flux scalars copied to interface j - 2
-  const int pf = tid - (PL::THREADS - np * W);  // prefetched point of this thread (MODE 1; none if negative)
+  constexpr int NR = PL::NR, NV = PL::NV;
+  const int nr = len + 2;                       // points 2 .. np - 3: both sides of every interface
+  const int pf = tid - (PL::THREADS - nr * W);  // prefetched point of this thread (MODE 1; none if negative)
   static_assert(MODE == 0 || NP * W <= PL::THREADS, "one prefetched point per thread");
   if constexpr (MODE == 1) {
     constexpr int NG = PL::NG;
@@ -268,26 +280,20 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       }
     }
     __syncthreads();
-    // the point values are dead: fetch the Roe-average inputs and the viscous flux into
-    // their space while phases B and C run.  One point per thread, on the last NP*W
-    // threads (those with the fewest phase-C items), which also convert their Roe
-    // inputs to double-float in place before the barrier that ends phase C.
+    // the point values are dead: fetch the Roe-average inputs into their space while phases B
+    // and C run.  One point per thread, on the last nr*W threads (those with the fewest phase-C
+    // items), which also convert their Roe inputs to double-float in place before the barrier
+    // that ends phase C.
     if (pf >= 0) {
       int pos, line;
-      item_split<D, W>(pf, np, c_rcp20.v[np], pos, line);
-      const long long p = flat(wrap(s0 - 3 + pos), min(a0 + line, na - 1));
-      const int sp = tile_idx<D, W>(pos, line, NP);
-      double* r = sm + PL::OFF_ROE + sp;
-      cp_async8(r + 0 * NP * W, a.pm + PM_SR * N + p);
-      cp_async8(r + 1 * NP * W, a.pm + PM_U * N + p);
-      cp_async8(r + 2 * NP * W, a.pm + PM_V * N + p);
-      cp_async8(r + 3 * NP * W, a.pm + PM_W * N + p);
-      cp_async8(r + 4 * NP * W, a.pm + PM_H * N + p);
-      if (a.fv != nullptr) {
-        double* f = sm + PL::OFF_FV + sp;
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) cp_async8(f + cc * NP * W, a.fv + (long long)(a.fv_dstride * D + cc) * N + p);
-      }
+      item_split<D, W>(pf, nr, c_rcp20.v[nr], pos, line);
+      const long long p = flat(wrap(s0 - 1 + pos), min(a0 + line, na - 1));
+      double* r = sm + PL::OFF_ROE + tile_idx<D, W>(pos, line, NR);
+      cp_async8(r + 0 * NR * W, a.pm + PM_SR * N + p);
+      cp_async8(r + 1 * NR * W, a.pm + PM_U * N + p);
+      cp_async8(r + 2 * NR * W, a.pm + PM_V * N + p);
+      cp_async8(r + 3 * NR * W, a.pm + PM_W * N + p);
+      cp_async8(r + 4 * NR * W, a.pm + PM_H * N + p);
     }
     cp_async_commit();
   }
@@ -416,7 +422,8 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
     // third differences T_f, T_{f+1}, T_{f+2} of phase B.  Evaluated in double-float on the FP32
     // pipe.  The interface values are never formed in FP64, and the linear parts combine:
     //   fhat_R - fhat_L = T_{f+1}/6 - (oL + oR)                          (u-scalars; double-float)
-    //   fhat_L + fhat_R = 2 P2 + [g2 + (g1 - g3)/6 + (oL - oR)]          (flux scalars; FP64)
+    //   fhat_L + fhat_R = 2 P2 + [g2 + (g1 - g3)/6 + (oL - oR)]          (flux scalars; the bracket
+    //                                                                    in double-float)
     // One item per line pair, in two-lane double-float arithmetic.
     float2* rf = reinterpret_cast<float2*>(sm + PL::OFF_R);
     auto phase_c = [&](auto scaled) {
@@ -443,9 +450,9 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         if (m >= 4) {  // flux scalar; P2 copied in phase A2
           const df2 lin = df2_add_fast(ldG(f + 2), df2_mul_u(df2_add_fast(ldG(f + 1), df2_neg(ldG(f + 3))), df2_sixth()));
           const df2 t = df2_add_fast(lin, df2_add_fast(oL, df2_neg(oR)));
-          double* F = sm + PL::OFF_R + (1 + m) * NI * W;
-          F[o0] = fma(2.0, F[o0], f2d_bits(t.hi.x)) + f2d_bits(t.lo.x);
-          F[o1] = fma(2.0, F[o1], f2d_bits(t.hi.y)) + f2d_bits(t.lo.y);
+          float2* F = reinterpret_cast<float2*>(sm + PL::OFF_T) + (m - 4) * NI * W;
+          F[o0] = make_float2(t.hi.x, t.lo.x);
+          F[o1] = make_float2(t.hi.y, t.lo.y);
         }
       }
     };
@@ -453,33 +460,42 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       phase_c(std::true_type{});
     else
       phase_c(std::false_type{});
-    cp_async_wait_all();  // this thread's ROE / FV copies; the barrier publishes them
+    cp_async_wait_all();  // this thread's ROE copies; the barrier publishes them
     if (pf >= 0) {  // velocities to double-float, in place (sqrt(rho) and H arrive as
                        // double-float: planes of the NS3D_FP64 primitive layout)
       int pos, line;
-      item_split<D, W>(pf, np, c_rcp20.v[np], pos, line);
-      double* r = sm + PL::OFF_ROE + tile_idx<D, W>(pos, line, NP);
+      item_split<D, W>(pf, nr, c_rcp20.v[nr], pos, line);
+      double* r = sm + PL::OFF_ROE + tile_idx<D, W>(pos, line, NR);
 #pragma unroll
       for (int k = 1; k < 4; ++k) {
-        const df x = d2df_bits(r[k * NP * W]);
-        reinterpret_cast<float2*>(r)[k * NP * W] = make_float2(x.hi, x.lo);
+        const df x = d2df_bits(r[k * NR * W]);
+        reinterpret_cast<float2*>(r)[k * NR * W] = make_float2(x.hi, x.lo);
       }
     }
   }
   __syncthreads();
 
-  // ---- epilogue operands: fetched asynchronously into the (now unused) indicator
-  //      space while phase D runs; each thread later reads only its own point's slots.
+  // ---- epilogue operands, and in MODE 1 the viscous flux: fetched asynchronously into the (now
+  //      unused) indicator space while phase D runs; in MODE 1 by the threads that have no interface.
   //      cp.async.ca reads through L1 like a plain load, so in the persistent kernel (NC
   //      false), where the operands were written by other CTAs before the last grid-wide
   //      barrier, it sees them exactly as the plain loads it replaces would.
   static_assert(PL::TP * PL::W <= PL::THREADS, "one epilogue point per thread");
   static_assert(15 * PL::TP * PL::W <= NQ * 3 * PL::NW * PL::W, "prefetch slots fit the indicator space");
-  double* pre = sm + PL::OFF_B + 15 * tid;
-  if (tid < len * W) {
+  double* pre = sm + PL::OFF_B + 15 * tid;  // of this thread's point of phase E
+  const int ft = (MODE == 1) ? tid - PL::FETCH0 : tid;
+  if (ft >= 0 && ft < len * W) {
     int pp, line;
-    item_split<D, W>(tid, len, c_rcp20.v[len], pp, line);
-    if (a0 + line < na) epilogue_prefetch(a, flat(s0 + pp, a0 + line), pre);
+    item_split<D, W>(ft, len, c_rcp20.v[len], pp, line);
+    if (a0 + line < na) epilogue_prefetch(a, flat(s0 + pp, a0 + line), sm + PL::OFF_B + 15 * ft);
+  }
+  if (MODE == 1 && a.fv != nullptr && ft >= 0 && ft < nw * W) {  // points 1 .. np - 2
+    int pos, line;
+    item_split<D, W>(ft, nw, c_rcp20.v[nw], pos, line);
+    const long long p = flat(wrap(s0 - 2 + pos), min(a0 + line, na - 1));
+    double* f = sm + PL::OFF_FV + tile_idx<D, W>(pos, line, NV);
+#pragma unroll
+    for (int cc = 0; cc < 4; ++cc) cp_async8(f + cc * NV * W, a.fv + (long long)(a.fv_dstride * D + cc) * N + p);
   }
   cp_async_commit();
 
@@ -493,22 +509,21 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       int f, line;
       item_split<D, W>(item, ni, c_rcp20.v[ni], f, line);
       const int o = tile_idx<D, W>(f, line, NI);
-      const int sa = tile_idx<D, W>(f + 2, line, NP), sb = tile_idx<D, W>(f + 3, line, NP);
+      const int ia = (MODE == 1) ? f : f + 2;  // the interface's left point among the Roe inputs
+      const int sa = tile_idx<D, W>(ia, line, NR), sb = tile_idx<D, W>(ia + 1, line, NR);
       if (MODE == 1) {
         // Roe dissipation X|Lambda|X^{-1} du in double-float from the double-float jumps
         // du of phase C and the double-float Roe-average inputs; the flux, already divided
-        // by dx for phase E, is (fhat_L + fhat_R)/(2 dx) - diss/(2 dx): two FP64 operations
-        // per component
+        // by dx for phase E, is P2/dx + (t - diss)/(2 dx), t the double-float part of
+        // fhat_L + fhat_R = 2 P2 + t: two FP64 operations per component
         const float2* rf = reinterpret_cast<const float2*>(r);
-        auto ldr = [&](int k, int sp) { const float2 v = rf[k * NP * W + sp]; return df{v.x, v.y}; };
+        auto ldr = [&](int k, int sp) { const float2 v = rf[k * NR * W + sp]; return df{v.x, v.y}; };
         const float2* rj = reinterpret_cast<const float2*>(rec);
         df du[5];
-        double fs[5];  // fhat_L + fhat_R of the five flux components (f_0 = u_{1+D})
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
           const float2 j = rj[scalar_of<MODE, D>(v) * NI * W + o];
           du[v] = df{j.x, j.y};
-          fs[v] = rec[(5 + v) * NI * W + o];
         }
         const df ra = ldr(0, sa), rb = ldr(0, sb);
         const df rsum = df_add_pos(ra, rb);
@@ -555,11 +570,13 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         diss[1 + T2] = df_add_fast(df_mul_u(d0, vt2), A4);
         diss[4] = df_add_fast(df_add_fast(df_mul_u(S, H), df_mul_u(cD, un)),
                               df_add_fast(df_mul_u(A2, q2h), df_add_fast(df_mul_u(A3, vt1), df_mul_u(A4, vt2))));
-        const df mhr = df_neg(d2df_bits(a.g.hrh[D]));
+        const df hr = d2df_bits(a.g.hrh[D]);
+        const float2* ts = reinterpret_cast<const float2*>(sm + PL::OFF_T);
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          const df t = df_mul(diss[v], mhr);
-          rec[v * NI * W + o] = fma(a.g.hrh[D], fs[v], f2d_bits(t.hi)) + f2d_bits(t.lo);
+        for (int v = 0; v < 5; ++v) {  // flux component 0 is u_{1+D}
+          const float2 tv = ts[v * NI * W + o];
+          const df t = df_mul(df_add_fast(df{tv.x, tv.y}, df_neg(diss[v])), hr);
+          rec[v * NI * W + o] = fma(a.g.rh[D], rec[(5 + v) * NI * W + o], f2d_bits(t.hi)) + f2d_bits(t.lo);
         }
         continue;
       }
@@ -635,10 +652,10 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
     if (__any_sync(0xffffffffu, bad) && (tid & 31) == 0) atomicOr(a.status, ST_NONPHYS);
     if (MODE == 1 && __any_sync(0xffffffffu, range_bad) && (tid & 31) == 0) atomicOr(a.status, ST_DF_RANGE);
   }
+  cp_async_wait_all();
   __syncthreads();
 
   // ---- E: conservative difference + viscous divergence + epilogue ----------------
-  cp_async_wait_all();
   {
     const double rdx = a.g.rh[D];
     const double r12 = a.g.r12h[D];
@@ -657,9 +674,9 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
           const df r12d = d2df_bits(r12);
 #pragma unroll
           for (int cc = 0; cc < 4; ++cc) {
-            const float2* fc = reinterpret_cast<const float2*>(fvs + cc * NP * W);
-            auto ld = [&](int j) { const float2 v = fc[tile_idx<D, W>(j, line, NP)]; return df{v.x, v.y}; };
-            const df t = d4_dfv(ld(pp + 1), ld(pp + 2), ld(pp + 4), ld(pp + 5), r12d);
+            const float2* fc = reinterpret_cast<const float2*>(fvs + cc * NV * W);
+            auto ld = [&](int j) { const float2 v = fc[tile_idx<D, W>(j, line, NV)]; return df{v.x, v.y}; };
+            const df t = d4_dfv(ld(pp), ld(pp + 1), ld(pp + 3), ld(pp + 4), r12d);
             cv[1 + cc] = (cv[1 + cc] + f2d_bits(t.hi)) + f2d_bits(t.lo);
           }
         }
