@@ -112,7 +112,7 @@ __device__ __forceinline__ float weno_safe(float B1, float B2, float B3, float c
 }
 
 // Accumulation / RK epilogue with its operands from the prefetch slots: kp = k, ops = U_n then
-// acc or the stage input; the arithmetic of dir_epilogue.
+// acc or the stage input; the arithmetic of dir_epilogue_pre.
 __device__ __forceinline__ void dir_epilogue_pre32(const DirArgs& a, long long p, const double cv[5], const double* kp,
                                                    const double* ops) {
   const long long N = a.g.N;
@@ -176,12 +176,6 @@ __device__ __forceinline__ void dir_epilogue_pre32(const DirArgs& a, long long p
     default:
       break;
   }
-}
-
-// 16-byte asynchronous global -> shared copy (both addresses 16-byte aligned), L2 only.
-__device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 
 // dir_epilogue_pre32 for two x-adjacent points p and p + 1 (p even), their operands and results

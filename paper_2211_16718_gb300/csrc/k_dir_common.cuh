@@ -93,72 +93,6 @@ __device__ __forceinline__ long long tile_flat(const Grid& g, int c, int la, int
   return ((long long)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
 }
 
-// Accumulate this direction's contribution cv[5] at point p, or finish the RHS /
-// RK stage (last direction), according to a.epi.
-__device__ __forceinline__ void dir_epilogue(const DirArgs& a, long long p, const double cv[5]) {
-  const long long N = a.g.N;
-  switch (a.epi) {
-    case EPI_ACC_WRITE:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) a.k[v * N + p] = cv[v];
-      break;
-    case EPI_ACC_ADD:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) a.k[v * N + p] += cv[v];
-      break;
-    case EPI_RHS_OUT:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) a.out[v * N + p] = a.k[v * N + p] + cv[v];
-      break;
-    case EPI_RK4_FIRST:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = a.k[v * N + p] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, a.un[v * N + p]);
-        a.acc[v * N + p] = K;
-      }
-      break;
-    case EPI_RK4_MID:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = a.k[v * N + p] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, a.un[v * N + p]);
-        a.acc[v * N + p] = fma(2.0, K, a.acc[v * N + p]);
-      }
-      break;
-    case EPI_RK4_LAST:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = a.k[v * N + p] + cv[v];
-        a.out[v * N + p] = fma(a.a, a.acc[v * N + p] + K, a.un[v * N + p]);
-      }
-      break;
-    case EPI_SSP_1:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = a.k[v * N + p] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, a.un[v * N + p]);
-      }
-      break;
-    case EPI_SSP_2:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = a.k[v * N + p] + cv[v];
-        a.out[v * N + p] = 0.75 * a.un[v * N + p] + 0.25 * fma(a.a, K, a.u[v * N + p]);
-      }
-      break;
-    case EPI_SSP_3:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = a.k[v * N + p] + cv[v];
-        a.out[v * N + p] = (1.0 / 3.0) * a.un[v * N + p] + (2.0 / 3.0) * fma(a.a, K, a.u[v * N + p]);
-      }
-      break;
-    default:
-      break;
-  }
-}
-
 // Number of FP64 operands per point the epilogue reads (k, then U_n, then acc or the stage input).
 __host__ __device__ __forceinline__ int epilogue_operands(int epi) {
   switch (epi) {
@@ -179,26 +113,41 @@ __device__ __forceinline__ void cp_async8(double* dst_smem, const double* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Start fetching the epilogue operands of point p into pre[0 .. epilogue_operands(a.epi)).
+// 16-byte asynchronous global -> shared copy (both addresses 16-byte aligned), L2 only.
+__device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+// One double (PAIR false), or two adjacent ones from 16-byte aligned addresses.
+template <bool PAIR>
+__device__ __forceinline__ void cp_async_d(double* dst_smem, const double* src) {
+  if (PAIR) cp_async16(dst_smem, src);
+  else cp_async8(dst_smem, src);
+}
+
+// Start fetching the epilogue operands of point p (PAIR: of p and p + 1) into pre[v * TS],
+// v < epilogue_operands(a.epi).
+template <bool PAIR, int TS>
 __device__ __forceinline__ void epilogue_prefetch(const DirArgs& a, long long p, double* pre) {
   const long long N = a.g.N;
   const int n = epilogue_operands(a.epi);
   if (n == 0) return;
 #pragma unroll
-  for (int v = 0; v < 5; ++v) cp_async8(pre + v, a.k + v * N + p);
+  for (int v = 0; v < 5; ++v) cp_async_d<PAIR>(pre + v * TS, a.k + v * N + p);
   if (n >= 10) {
 #pragma unroll
-    for (int v = 0; v < 5; ++v) cp_async8(pre + 5 + v, a.un + v * N + p);
+    for (int v = 0; v < 5; ++v) cp_async_d<PAIR>(pre + (5 + v) * TS, a.un + v * N + p);
   }
   if (n == 15) {
     const double* third = (a.epi == EPI_SSP_2 || a.epi == EPI_SSP_3) ? a.u : a.acc;
 #pragma unroll
-    for (int v = 0; v < 5; ++v) cp_async8(pre + 10 + v, third + v * N + p);
+    for (int v = 0; v < 5; ++v) cp_async_d<PAIR>(pre + (10 + v) * TS, third + v * N + p);
   }
 }
 
-// dir_epilogue with the operands read from pre (filled by epilogue_prefetch) instead of
-// global memory; the same arithmetic, so the same bits.
+// Accumulate this direction's contribution cv[5] at point p, or finish the RHS / RK stage (last
+// direction), according to a.epi; the operands in pre[v * TS] (filled by epilogue_prefetch).
+template <int TS>
 __device__ __forceinline__ void dir_epilogue_pre(const DirArgs& a, long long p, const double cv[5],
                                                  const double* pre) {
   const long long N = a.g.N;
@@ -209,54 +158,54 @@ __device__ __forceinline__ void dir_epilogue_pre(const DirArgs& a, long long p, 
       break;
     case EPI_ACC_ADD:
 #pragma unroll
-      for (int v = 0; v < 5; ++v) a.k[v * N + p] = pre[v] + cv[v];
+      for (int v = 0; v < 5; ++v) a.k[v * N + p] = pre[v * TS] + cv[v];
       break;
     case EPI_RHS_OUT:
 #pragma unroll
-      for (int v = 0; v < 5; ++v) a.out[v * N + p] = pre[v] + cv[v];
+      for (int v = 0; v < 5; ++v) a.out[v * N + p] = pre[v * TS] + cv[v];
       break;
     case EPI_RK4_FIRST:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, pre[5 + v]);
+        const double K = pre[v * TS] + cv[v];
+        a.out[v * N + p] = fma(a.a, K, pre[(5 + v) * TS]);
         a.acc[v * N + p] = K;
       }
       break;
     case EPI_RK4_MID:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, pre[5 + v]);
-        a.acc[v * N + p] = fma(2.0, K, pre[10 + v]);
+        const double K = pre[v * TS] + cv[v];
+        a.out[v * N + p] = fma(a.a, K, pre[(5 + v) * TS]);
+        a.acc[v * N + p] = fma(2.0, K, pre[(10 + v) * TS]);
       }
       break;
     case EPI_RK4_LAST:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, pre[10 + v] + K, pre[5 + v]);
+        const double K = pre[v * TS] + cv[v];
+        a.out[v * N + p] = fma(a.a, pre[(10 + v) * TS] + K, pre[(5 + v) * TS]);
       }
       break;
     case EPI_SSP_1:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, pre[5 + v]);
+        const double K = pre[v * TS] + cv[v];
+        a.out[v * N + p] = fma(a.a, K, pre[(5 + v) * TS]);
       }
       break;
     case EPI_SSP_2:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v] + cv[v];
-        a.out[v * N + p] = 0.75 * pre[5 + v] + 0.25 * fma(a.a, K, pre[10 + v]);
+        const double K = pre[v * TS] + cv[v];
+        a.out[v * N + p] = 0.75 * pre[(5 + v) * TS] + 0.25 * fma(a.a, K, pre[(10 + v) * TS]);
       }
       break;
     case EPI_SSP_3:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v] + cv[v];
-        a.out[v * N + p] = (1.0 / 3.0) * pre[5 + v] + (2.0 / 3.0) * fma(a.a, K, pre[10 + v]);
+        const double K = pre[v * TS] + cv[v];
+        a.out[v * N + p] = (1.0 / 3.0) * pre[(5 + v) * TS] + (2.0 / 3.0) * fma(a.a, K, pre[(10 + v) * TS]);
       }
       break;
     default:

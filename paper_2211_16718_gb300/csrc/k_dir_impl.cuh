@@ -482,20 +482,37 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
   //      barrier, it sees them exactly as the plain loads it replaces would.
   static_assert(PL::TP * PL::W <= PL::THREADS, "one epilogue point per thread");
   static_assert(15 * PL::TP * PL::W <= NQ * 3 * PL::NW * PL::W, "prefetch slots fit the indicator space");
-  double* pre = sm + PL::OFF_B + 15 * tid;  // of this thread's point of phase E
+  //      The z pass with nx even takes two x-adjacent points (lines 2j, 2j + 1 of the tile: their flat
+  //      index is even) per 16-byte copy, past L1: half the copies.  U_n and the stage input may be
+  //      the caller's and only 8-byte aligned; the rest is the library's.  z pass with the RK4
+  //      epilogue at 128^3: 502 -> 471 us (16-byte copies through L1: 505).  Not so the y pass, which
+  //      has 9 operands instead of up to 19 (415 -> 425 us), nor the Roe inputs above (phase A has
+  //      just read three of their five planes through L1).
+  const bool pair16 = D == 2 && W % 2 == 0 && (na & 1) == 0 && (((uintptr_t)a.un | (uintptr_t)a.u) & 15) == 0;
+  constexpr int TS = TP * W;
+  double* pre = sm + PL::OFF_B;  // [15][TP*W]
   const int ft = (MODE == 1) ? tid - PL::FETCH0 : tid;
-  if (ft >= 0 && ft < len * W) {
-    int pp, line;
-    item_split<D, W>(ft, len, c_rcp20.v[len], pp, line);
-    if (a0 + line < na) epilogue_prefetch(a, flat(s0 + pp, a0 + line), sm + PL::OFF_B + 15 * ft);
-  }
-  if (MODE == 1 && a.fv != nullptr && ft >= 0 && ft < nw * W) {  // points 1 .. np - 2
-    int pos, line;
-    item_split<D, W>(ft, nw, c_rcp20.v[nw], pos, line);
-    const long long p = flat(wrap(s0 - 2 + pos), min(a0 + line, na - 1));
-    double* f = sm + PL::OFF_FV + tile_idx<D, W>(pos, line, NV);
+  auto fetch_epilogue = [&](auto pair) {
+    constexpr bool PAIR = decltype(pair)::value;
+    constexpr int S = PAIR ? 2 : 1;
+    if (ft < len * (W / S)) {
+      int pp, l;
+      item_split<D, W / S>(ft, len, c_rcp20.v[len], pp, l);
+      if (a0 + S * l < na) epilogue_prefetch<PAIR, TS>(a, flat(s0 + pp, a0 + S * l), pre + S * ft);
+    }
+    if (MODE == 1 && a.fv != nullptr && ft < nw * (W / S)) {  // points 1 .. np - 2
+      int pos, l;
+      item_split<D, W / S>(ft, nw, c_rcp20.v[nw], pos, l);
+      const long long p = flat(wrap(s0 - 2 + pos), min(a0 + S * l, na - S));
+      double* f = sm + PL::OFF_FV + tile_idx<D, W>(pos, S * l, NV);
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) cp_async8(f + cc * NV * W, a.fv + (long long)(a.fv_dstride * D + cc) * N + p);
+      for (int cc = 0; cc < 4; ++cc)
+        cp_async_d<PAIR>(f + cc * NV * W, a.fv + (long long)(a.fv_dstride * D + cc) * N + p);
+    }
+  };
+  if (ft >= 0) {
+    if (D == 2 && pair16) fetch_epilogue(std::bool_constant<D == 2>{});
+    else fetch_epilogue(std::false_type{});
   }
   cp_async_commit();
 
@@ -680,7 +697,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
             cv[1 + cc] = (cv[1 + cc] + f2d_bits(t.hi)) + f2d_bits(t.lo);
           }
         }
-        dir_epilogue_pre(a, flat(s0 + pp, a0 + line), cv, pre);
+        dir_epilogue_pre<TS>(a, flat(s0 + pp, a0 + line), cv, pre + item);
         continue;
       }
 #pragma unroll
@@ -695,7 +712,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         }
       }
       const long long p = flat(s0 + pp, a0 + line);
-      dir_epilogue_pre(a, p, cv, pre);
+      dir_epilogue_pre<TS>(a, p, cv, pre + item);
     }
   }
 }

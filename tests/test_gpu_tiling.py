@@ -97,3 +97,20 @@ def test_balanced_tiles(ns3d, orc, nx, ny, nz):
             assert rel_err(out[-1], ref) <= 1e-12, (prec, v)
             assert np.array_equal(out[0], out[-1]), (prec, v)
 
+
+
+@pytest.mark.parametrize("nx", [24, 26, 27])
+def test_step_of_a_state_on_8_byte_boundaries(ns3d, nx):
+    """The z pass takes 16-byte copies only where U_n allows it: the same bits either way."""
+    import torch
+    u = _gpu(I.random_smooth(nx, 10, 30, seed=8, amp=0.1, mach=0.4))
+    buf = torch.empty(u.numel() + 1, dtype=torch.float64, device="cuda")
+    v = buf[1:].view(u.shape)
+    v.copy_(u)
+    assert v.data_ptr() % 16 == 8
+    s = ns3d.Solver(nx, 10, 30, mu_eff=0.003)
+    s.rk_step(u, 0.01, 2)
+    s.rk_step(v, 0.01, 2)
+    s.check()
+    s.close()
+    assert torch.equal(u, v)
