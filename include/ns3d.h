@@ -77,7 +77,7 @@ enum { NS3D_RK4 = 0, NS3D_SSPRK3 = 1 };           /* time integrators (Sec. 2.2)
  *                   conserved to FP64 rounding); state, RK accumulation and reductions in
  *                   FP64.  Relative RHS error ~1e-7 of the flux scale max|f|/dx.
  *                   Requires weno_eps >= 1e-15.
- *  NS3D_FP64_STRICT every operation in FP64 (one FP64 division per reconstruction). */
+ *  NS3D_FP64_STRICT every operation in FP64 (one FP64 reciprocal per reconstruction). */
 enum { NS3D_FP64 = 0, NS3D_FP32_BULK = 1, NS3D_FP64_STRICT = 2 };
 /* Storage of the viscous flux vectors (same results, bitwise, in every mode):
  *  NS3D_STORAGE_FULL  all three directions' fluxes at once, 12*N doubles;

@@ -23,7 +23,14 @@
 // The three squared indicators of a window serve the left-biased reconstruction
 // at one interface and the right-biased one at another, so each is computed once.
 //
-// MODE 0 (all FP64): fhat = sum_k omega_k F_k with one FP64 division.
+// Since sum omega = 1, fhat = F_2 + omega_1 (F_1 - F_2) + omega_3 (F_3 - F_2): the reconstructions
+// are candidate 2 and an offset from third differences of the data.
+// MODE 0 (all FP64): bound by the FP64 pipe (2 lanes per SM and clock), so written for its operation
+// count: with D = B_2/6 the offset is D [B_3 (F_1 - F_2) + 3 B_1 (F_3 - F_2)] / [D B_3 + B_1 (B_3 + 3 D)],
+// six operations and a reciprocal; jump and sum of the two reconstructions share their linear parts.
+// 495 FP64 operations per point and pass where candidates, IEEE divisions and separate left and right
+// values took 726: 96^3 pass 1.26 / 1.31 / 1.35 -> 0.91 / 0.92 / 0.95 ms (x / y / z, FP64 pipe 87 %
+// busy), the error of a right-hand side against 64 bits 13-19 % smaller.
 // MODE 1 (FP64 values, double-float weights): since sum omega = 1,
 //   fhat = F_2 + omega_1 (F_1 - F_2) + omega_3 (F_3 - F_2),
 // where F_1 - F_2 and F_3 - F_2 are third differences of the data and the weights, which only multiply these small
@@ -55,8 +62,10 @@ constexpr int NQ = 9;             // reconstructed scalars
 // Tile plan of a direction pass: TP points along the pencil times W lines.
 // Shared memory in 8-byte words (doubles, or double-float pairs in MODE 1):
 //   MODE 0: Q [NQ][NP*W] point values, ROE [5][NP*W] sqrt(rho), u, v, w, H,
-//           FV [4][NP*W] viscous flux, B [NQ][3][NW*W] squared indicators,
-//           R [18][NI*W] interface values, later [5][NI*W] interface fluxes.
+//           FV [4][NP*W] viscous flux, B [NQ][4][NW*W] per window B_1, B_2/6, B_3 and a third
+//           of its third difference (later the epilogue operands), R [10][NI*W]: jumps of u_0..u_4
+//           (slots 0-4) and sums of the flux components (slots 5-9), later [5][NI*W] interface fluxes.
+//           73.9 KB for 32 x 4: three CTAs of 256 threads share an SM.
 //   MODE 1: Q [NQ][NP*W], dead after phase A2: ROE [5][NR*W] then arrives there by cp.async (as
 //           FP64) while phases B and C run, and phase C puts T [5][NI*W] behind it, the double-float
 //           part of fhat_L + fhat_R of the five flux scalars;
@@ -73,7 +82,7 @@ template <int MODE, int TP_, int W_>
 struct Plan {
   static constexpr int TP = TP_;                    // points per tile along the pencil
   static constexpr int W = W_;                      // lines per tile
-  static constexpr int THREADS = (MODE == 0) ? 128 : 256;  // MODE 1: 8 warps share the tile (latency hiding)
+  static constexpr int THREADS = 256;  // 8 warps share the tile (latency hiding)
   static constexpr int MIN_CTAS = (MODE == 0) ? 3 : 4;     // resident CTAs per SM the registers allow
   static constexpr int NP = TP + 6;                 // points incl. 3-point halo each side
   static constexpr int NW = TP + 4;                 // 3-point windows centred at -2 .. TP+1
@@ -89,14 +98,14 @@ struct Plan {
                                : (END_T > NQ * NP * W) ? (END_T + 1) / 2 * 2
                                                        : OFF_Q + NQ * NP * W;
   static constexpr int OFF_FV = (MODE == 1) ? OFF_B + 15 * TP * W : OFF_ROE + 5 * NP * W;
-  static constexpr int OFF_S = OFF_B + NQ * 3 * NW * W;  // MODE 1: third differences
+  static constexpr int OFF_S = OFF_B + NQ * (MODE == 0 ? 4 : 3) * NW * W;  // MODE 1: third differences
   static constexpr int OFF_G = OFF_S + (MODE == 1 ? NQ * NW * W : 0);
   static constexpr int OFF_R = OFF_G + (MODE == 1 ? NQ * NG * W : 0);
-  static constexpr int R_SLOTS = (MODE == 1) ? 10 : 18;
+  static constexpr int R_SLOTS = 10;
   static constexpr int WORDS = OFF_R + R_SLOTS * NI * W;
   static constexpr int BYTES = WORDS * 8;
   static_assert(MODE == 0 || OFF_FV + 4 * NV * W <= OFF_S, "epilogue operands and FV fit the dead indicators");
-  // MODE 1: the threads that fetch the epilogue operands and FV while the others run phase D
+  // the threads that fetch the epilogue operands (MODE 1: and FV) while the others run phase D
   static constexpr int FETCH0 = THREADS / 2;
   static_assert(MODE == 0 || (NI * W <= FETCH0 && NV * W <= THREADS - FETCH0), "phase D and the fetches side by side");
 };
@@ -112,13 +121,23 @@ __host__ __device__ constexpr int scalar_of(int c) {
   return (c == 1 + D) ? 4 : (c == 1 + T1) ? 1 : (c == 1 + T2) ? 2 : 3;
 }
 
-__device__ __forceinline__ double weno_combine(double B1, double B2, double B3, double F1, double F2, double F3) {
-  const double p23 = B2 * B3;
-  const double t13 = 6.0 * (B1 * B3);
-  const double t12 = 3.0 * (B1 * B2);
-  const double num = fma(p23, F1, fma(t13, F2, t12 * F3));
-  const double den = p23 + t13 + t12;
-  return num / den;
+// FP64 reciprocal and reciprocal square root from the special-function unit's approximations (PTX
+// rcp / rsqrt.approx.ftz.f64, about 20 correct bits) and one cubic correction: three and five FP64
+// operations where the IEEE division and square root take nine and ten, error below 1 ulp.
+// Reciprocals of magnitudes outside [2^-1021, 2^1020) and of non-finite values are IEEE divisions.
+__device__ __forceinline__ double rcp_cubic(double x) {
+  const uint32_t e11 = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
+  if (e11 - 2u >= 2041u) return 1.0 / x;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double rsqrt_cubic(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x * r, r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
 }
 
 // Range of the scaled indicators b_k inside which df2_offset3 needs no rescaling of the B_k = b_k^2:
@@ -301,26 +320,39 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
   // ---- B: squared scaled smoothness indicators of every window ----------------
   int need_scale = 0;
   if constexpr (MODE == 0) {
+    // one item per line and four adjacent windows, which share differences
     const double* q = sm + PL::OFF_Q;
-    const unsigned rcp_nw = c_rcp20.v[nw];
-    for (int item = tid; item < NQ * nw * W; item += PL::THREADS) {
-      int m, w, line;
-      item_split<D, W>(item, nw, rcp_nw, m, w, line);
-      const int o = tile_idx<D, W>(w, line, NW);
+    const int nw4 = (nw + 3) / 4;
+    const unsigned rcp_nw4 = c_rcp20.v[nw4];
+    for (int item = tid; item < NQ * nw4 * W; item += PL::THREADS) {
+      int m, w4, line;
+      item_split<D, W>(item, nw4, rcp_nw4, m, w4, line);
       const double* qm = q + m * NP * W;
-      const double x = qm[tile_idx<D, W>(w, line, NP)];
-      const double y = qm[tile_idx<D, W>(w + 1, line, NP)];
-      const double z = qm[tile_idx<D, W>(w + 2, line, NP)];
-      const double gm = y - x, gp = z - y, s = gp - gm;
-      double* bw = sm + PL::OFF_B;
-      const double aa = fma((13.0 / 3.0) * s, s, a.eps4);
-      const double u1 = fma(3.0, gp, -gm);   // x - 4y + 3z
-      const double u2 = gm + gp;             // z - x
-      const double u3 = fma(-3.0, gm, gp);   // 3x - 4y + z
-      const double b1 = fma(u1, u1, aa), b2 = fma(u2, u2, aa), b3 = fma(u3, u3, aa);
-      bw[(m * 3 + 0) * NW * W + o] = b1 * b1;
-      bw[(m * 3 + 1) * NW * W + o] = b2 * b2;
-      bw[(m * 3 + 2) * NW * W + o] = b3 * b3;
+      double* bw = sm + PL::OFF_B + m * 4 * NW * W;
+      auto ldq = [&](int j) { return qm[tile_idx<D, W>(min(j, np - 1), line, NP)]; };
+      double q1 = ldq(4 * w4 + 1), q2 = ldq(4 * w4 + 2);
+      double gm = q1 - ldq(4 * w4), gp = q2 - q1, s0 = gp - gm;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int w = 4 * w4 + k;
+        if (w >= nw) break;
+        const int o = tile_idx<D, W>(w, line, NW);
+        // the third difference of the last window needs a point beyond the tile and is never read
+        const double q3 = ldq(w + 3), gn = q3 - q2, s1 = gn - gp;
+        bw[3 * NW * W + o] = (1.0 / 3.0) * (s0 - s1);
+        const double aa = fma((13.0 / 3.0) * s0, s0, a.eps4);
+        const double u1 = fma(3.0, gp, -gm);   // x - 4y + 3z
+        const double u2 = gm + gp;             // z - x
+        const double u3 = fma(-3.0, gm, gp);   // 3x - 4y + z
+        const double b1 = fma(u1, u1, aa), b2 = fma(u2, u2, aa), b3 = fma(u3, u3, aa);
+        bw[0 * NW * W + o] = b1 * b1;
+        bw[1 * NW * W + o] = b2 * ((1.0 / 6.0) * b2);
+        bw[2 * NW * W + o] = b3 * b3;
+        q2 = q3;
+        gm = gp;
+        gp = gn;
+        s0 = s1;
+      }
     }
   } else {
     // one item per line pair and two adjacent windows: two-lane double-float arithmetic (packed FP32
@@ -390,31 +422,33 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
 
   // ---- C: left/right WENO5 reconstructions at every interface -------------------
   if constexpr (MODE == 0) {
+    // F_1 - F_2 = T_f/3, 3 (F_3 - F_2) = T_{f+1}/2 (left), the mirror image with -T (right); as in
+    // MODE 1 the jump is T_{f+1}/6 + oR - oL, the sum [7 (P2 + P3) - (P1 + P4)]/6 + oL + oR
     const double* q = sm + PL::OFF_Q;
     double* rec = sm + PL::OFF_R;
     const unsigned rcp_ni = c_rcp20.v[ni];
     for (int item = tid; item < NQ * ni * W; item += PL::THREADS) {
       int m, f, line;
       item_split<D, W>(item, ni, rcp_ni, m, f, line);
-      const double* qm = q + m * NP * W;
-      const double P0 = qm[tile_idx<D, W>(f, line, NP)], P1 = qm[tile_idx<D, W>(f + 1, line, NP)];
-      const double P2 = qm[tile_idx<D, W>(f + 2, line, NP)], P3 = qm[tile_idx<D, W>(f + 3, line, NP)];
-      const double P4 = qm[tile_idx<D, W>(f + 4, line, NP)], P5 = qm[tile_idx<D, W>(f + 5, line, NP)];
-      // third-order candidates at the interface between P2 and P3
-      const double xR = fma(11.0 / 6.0, P2, fma(-7.0 / 6.0, P1, (1.0 / 3.0) * P0));
-      const double eR = fma(1.0 / 3.0, P3, fma(5.0 / 6.0, P2, (-1.0 / 6.0) * P1));
-      const double eL = fma(-1.0 / 6.0, P4, fma(5.0 / 6.0, P3, (1.0 / 3.0) * P2));
-      const double xL = fma(1.0 / 3.0, P5, fma(-7.0 / 6.0, P4, (11.0 / 6.0) * P3));
-      const double* b = sm + PL::OFF_B + m * 3 * NW * W;
-      const double B1f = b[0 * NW * W + tile_idx<D, W>(f, line, NW)];
-      const double B2f1 = b[1 * NW * W + tile_idx<D, W>(f + 1, line, NW)];
-      const double B3f2 = b[2 * NW * W + tile_idx<D, W>(f + 2, line, NW)];
-      const double B3f3 = b[2 * NW * W + tile_idx<D, W>(f + 3, line, NW)];
-      const double B2f2 = b[1 * NW * W + tile_idx<D, W>(f + 2, line, NW)];
-      const double B1f1 = b[0 * NW * W + tile_idx<D, W>(f + 1, line, NW)];
+      const double* b = sm + PL::OFF_B + m * 4 * NW * W;
+      auto ld = [&](int k, int w) { return b[k * NW * W + tile_idx<D, W>(w, line, NW)]; };
+      const double Tc = ld(3, f + 1), T2 = 1.5 * Tc;
+      auto offset = [&](double B1, double D2, double B3, double T3, double& num, double& r) {
+        num = D2 * fma(B3, T3, B1 * T2);
+        r = rcp_cubic(fma(B1, fma(3.0, D2, B3), D2 * B3));
+      };
+      double nL, rL, nR, rR;  // oL = nL rL, oR = -nR rR
+      offset(ld(0, f), ld(1, f + 1), ld(2, f + 2), ld(3, f), nL, rL);
+      offset(ld(2, f + 3), ld(1, f + 2), ld(0, f + 1), ld(3, f + 2), nR, rR);
       const int o = tile_idx<D, W>(f, line, NI);
-      rec[(2 * m) * NI * W + o] = weno_combine(B1f, B2f1, B3f2, xR, eR, eL);
-      rec[(2 * m + 1) * NI * W + o] = weno_combine(B3f3, B2f2, B1f1, xL, eL, eR);
+      if (m < 5) rec[m * NI * W + o] = fma(-nR, rR, fma(-nL, rL, 0.5 * Tc));
+      if (m >= 5 || m == 1 + D) {  // f_0 = u_{1+D}
+        const double* qm = q + m * NP * W;
+        const double P1 = qm[tile_idx<D, W>(f + 1, line, NP)], P2 = qm[tile_idx<D, W>(f + 2, line, NP)];
+        const double P3 = qm[tile_idx<D, W>(f + 3, line, NP)], P4 = qm[tile_idx<D, W>(f + 4, line, NP)];
+        const double lin = fma(7.0 / 6.0, P2 + P3, (-1.0 / 6.0) * (P1 + P4));
+        rec[(m < 5 ? 5 : m + 1) * NI * W + o] = fma(-nR, rR, fma(nL, rL, lin));
+      }
     }
   } else {
     // fhat_L = P2 + (2 g2 + g1)/6 + oL, fhat_R = P3 - (2 g2 + g3)/6 - oR: candidate 2 and the
@@ -476,7 +510,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
   __syncthreads();
 
   // ---- epilogue operands, and in MODE 1 the viscous flux: fetched asynchronously into the (now
-  //      unused) indicator space while phase D runs; in MODE 1 by the threads that have no interface.
+  //      unused) indicator space while phase D runs, by the threads that have no interface.
   //      cp.async.ca reads through L1 like a plain load, so in the persistent kernel (NC
   //      false), where the operands were written by other CTAs before the last grid-wide
   //      barrier, it sees them exactly as the plain loads it replaces would.
@@ -491,7 +525,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
   const bool pair16 = D == 2 && W % 2 == 0 && (na & 1) == 0 && (((uintptr_t)a.un | (uintptr_t)a.u) & 15) == 0;
   constexpr int TS = TP * W;
   double* pre = sm + PL::OFF_B;  // [15][TP*W]
-  const int ft = (MODE == 1) ? tid - PL::FETCH0 : tid;
+  const int ft = tid - PL::FETCH0;
   auto fetch_epilogue = [&](auto pair) {
     constexpr bool PAIR = decltype(pair)::value;
     constexpr int S = PAIR ? 2 : 1;
@@ -597,24 +631,11 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         }
         continue;
       }
-      double uL[5], uR[5], fL[5], fR[5];
+      double du[5];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        uL[v] = rec[(2 * v) * NI * W + o];
-        uR[v] = rec[(2 * v + 1) * NI * W + o];
-      }
-#pragma unroll
-      for (int v = 1; v < 5; ++v) {
-        fL[v] = rec[(2 * (4 + v)) * NI * W + o];
-        fR[v] = rec[(2 * (4 + v) + 1) * NI * W + o];
-      }
-      fL[0] = uL[1 + D];
-      fR[0] = uR[1 + D];
+      for (int v = 0; v < 5; ++v) du[v] = rec[v * NI * W + o];
       const double ra = r[sa], rb = r[sb];
-      const double rsum = ra + rb;
-      // MODE 1: FP32-seeded Newton reciprocals (FP64 accurate, ~4 FP64 operations
-      // instead of ~9 for the IEEE division); MODE 0: IEEE division and square root
-      const double rs = (MODE == 1) ? rcp_newton(rsum) : 1.0 / rsum;
+      const double rs = rcp_cubic(ra + rb);
       const double wa = ra * rs, wb = rb * rs;
       double V[3];
 #pragma unroll
@@ -623,19 +644,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       const double q2h = 0.5 * fma(V[0], V[0], fma(V[1], V[1], V[2] * V[2]));
       const double c2 = gm1 * (H - q2h);
       bad |= !(c2 > 0.0);
-      double c, rc;
-      if (MODE == 1) {
-        // the float seeds need c^2 and sqrt(rho_a) + sqrt(rho_b) inside the float range
-        range_bad |= !(c2 > 1e-36 && c2 < 1e36 && rsum > 1e-36 && rsum < 1e36);
-        rc = rsqrt_newton(c2);
-        c = c2 * rc;
-      } else {
-        c = sqrt(c2);
-        rc = 1.0 / c;
-      }
-      double du[5];
-#pragma unroll
-      for (int v = 0; v < 5; ++v) du[v] = uR[v] - uL[v];
+      const double rc = rsqrt_cubic(c2), c = c2 * rc;
       constexpr int T1 = (D == 0) ? 1 : 0;
       constexpr int T2 = (D == 2) ? 1 : 2;
       const double un = V[D], vt1 = V[T1], vt2 = V[T2];
@@ -664,7 +673,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       diss[1 + T2] = fma(d0, vt2, A4);
       diss[4] = fma(S, H, fma(cD, un, fma(A2, q2h, fma(A3, vt1, A4 * vt2))));
 #pragma unroll
-      for (int v = 0; v < 5; ++v) rec[v * NI * W + o] = 0.5 * (fL[v] + fR[v] - diss[v]);
+      for (int v = 0; v < 5; ++v) rec[v * NI * W + o] = a.g.hrh[D] * (rec[(5 + v) * NI * W + o] - diss[v]);  // / dx
     }
     if (__any_sync(0xffffffffu, bad) && (tid & 31) == 0) atomicOr(a.status, ST_NONPHYS);
     if (MODE == 1 && __any_sync(0xffffffffu, range_bad) && (tid & 31) == 0) atomicOr(a.status, ST_DF_RANGE);
@@ -674,7 +683,6 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
 
   // ---- E: conservative difference + viscous divergence + epilogue ----------------
   {
-    const double rdx = a.g.rh[D];
     const double r12 = a.g.r12h[D];
     const double* F = sm + PL::OFF_R;
     const double* fvs = sm + PL::OFF_FV;
@@ -701,7 +709,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         continue;
       }
 #pragma unroll
-      for (int v = 0; v < 5; ++v) cv[v] = (F[v * NI * W + om] - F[v * NI * W + op]) * rdx;
+      for (int v = 0; v < 5; ++v) cv[v] = F[v * NI * W + om] - F[v * NI * W + op];
       if (a.fv != nullptr) {
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) {
