@@ -575,57 +575,90 @@ __global__ void __launch_bounds__(APL::THREADS, 2) k_adj_dir(const AdjArgs a) {
 
 // ============================================================================================
 // NS3D_FP64 form: the reconstruction adjoints in double-float arithmetic on the FP32 pipe.
-// Everything the WENO5 derivative needs is a function of the first differences g_j of the
-// data: s_k (second differences), v_k, b_k = 4 eps + 13/3 s_k^2 + v_k^2, the weights, the
-// candidate differences q_0 - q_1 = (s_0 - s_1)/3 and q_2 - q_1 = (s_1 - s_2)/6, and
-// q_k - q = (q_k - q_1) - M with M = omega_0 (q_0 - q_1) + omega_2 (q_2 - q_1).  The value
-// itself is q = P_c + (2 g_2 + g_1)/6 + M (P_c the stencil centre), the same offset form as
-// the forward pass.  The Roe-flux adjoint is double-float too (one interface per item); the
-// window terms, weights, reconstruction adjoints and the per-point gather take the tile's two
-// lines at once with the packed FP32 instructions (df2.cuh).  The per-point sums of the
-// reconstruction contributions are converted back to FP64 once.  To keep double-float values inside the float range whatever the scale of
-// the adjoint input, each tile divides lambda by the power of two of its largest magnitude
-// and multiplies its results back (exact).
+// Everything the WENO5 derivative needs is a function of the first differences g_j of the data.
+// With T_w = s_w - s_{w+1} the third difference of the windows w, w + 1 (s_w = g_{w+1} - g_w),
+//   value^L = P2 + (2 g2 + g1)/6 + M^L,   M^L = omega_0 T_f/3 + omega_2 T_{f+1}/6,
+//   value^R = P3 - (2 g2 + g3)/6 - M^R,   M^R the same with T_{f+2}, T_{f+1} (mirrored),
+// so that the jump is T_{f+1}/6 - (M^L + M^R), and an adjoint y of a value flows into
+//  - the window terms b_k: y omega_k (M - E_k) (-> 2/b_k), E = (T_f/3, 0, T_{f+1}/6);
+//  - the third differences: y omega_0/3 into T_f, y omega_2/6 into T_{f+1};
+//  - the linear part: for the conserved variables (y^R = -y^L = gamma) it is gamma T_{f+1}/6; for the
+//    flux components (y^L = y^R = h) its sum over a point's interfaces is the 4th-order central
+//    difference of lambda, taken from the interface differences when the point gathers.
+// Each b_k of a window is used by two reconstructions and each T by six, so their adjoints are
+// summed per window before they are multiplied by the derivatives (phase E2), which halves the
+// work of carrying every reconstruction's derivative to its five points.
+// The window terms, weights, reconstruction adjoints and the per-point gather take the tile's two
+// lines at once with the packed FP32 instructions (df2.cuh), the Roe-flux adjoint one interface of
+// one line per thread, beside the flux components' reconstruction adjoints, which do not need it.
+// The per-point sums are converted back to FP64 once.  To keep double-float values inside the float
+// range whatever the scale of the adjoint input, each tile divides the interface differences of
+// lambda by the power of two of lambda's largest magnitude and multiplies its results back (exact).
+// What bounds it: latency at 16 warps per SM (128 registers; 103 KB of shared memory).  355 warp
+// instructions per point where carrying every reconstruction to its points took 488: 128^3 pass
+// 2.15 / 2.24 / 2.13 -> 1.63 / 1.85 / 1.81 ms (x / y / z).  More warps with fewer registers lose: the
+// Roe adjoint's chain then spills 430 bytes (384 threads of 80 registers: 2.18 / 2.28 / 2.23 ms).
 // ============================================================================================
-template <int TP_, int W_, int THREADS_, int MIN_CTAS_>
+template <int TP_, int THREADS_, int MIN_CTAS_>
 struct AdjPlanDF {
-  static constexpr int TP = TP_;
-  static constexpr int W = W_;
+  static constexpr int TP = TP_;      // points per tile along the pencil, at most (balanced tiles)
+  static constexpr int W = 2;         // lines: one pair
   static constexpr int THREADS = THREADS_;
   static constexpr int MIN_CTAS = MIN_CTAS_;
   static constexpr int NP = TP + 10;  // points incl. a halo of 5 each side
   static constexpr int NI = TP + 5;   // interfaces
   static constexpr int NW = TP + 8;   // 3-point windows starting at 0 .. NW-1
-  static constexpr int OFF_Q = 0;                        // [9][NP*W] doubles
+  // 8-byte words; a record is 16 bytes, a double-float of both lines (hi0, hi1, lo0, lo1)
+  static constexpr int OFF_Q = 0;                        // [9][NP*W] FP64 u_0..u_4, f_1..f_4
   static constexpr int OFF_RI = OFF_Q + 9 * NP * W;      // [8][NP*W] double-float sqrt(rho), u, v, w, H;
                                                          //   FP64 p; double-float rho, e
-  static constexpr int OFF_L = OFF_RI + 8 * NP * W;      // [5][NP*W] lambda / 2^E
-  static constexpr int OFF_G = OFF_L + 5 * NP * W;       // [9][NP] first differences of both lines
-  static constexpr int OFF_B = OFF_G + 9 * NP * W;       // [9][3][NW] 1/b_k of every window, both lines
-  static constexpr int OFF_REC = OFF_B + 27 * NW * W;    // [10][NI*W] doubles: u^L, u^R of u_0..u_4
-  static constexpr int OFF_RD = OFF_REC + 10 * NI * W;   // [15][NI*W] double-float Roe adjoints
-  static constexpr int OFF_WC = OFF_RD + 15 * NI * W;    // [9][6][NI] stencil contributions, both lines
-  static constexpr int WORDS = OFF_WC + 54 * NI * W;
+  static constexpr int OFF_L = OFF_RI + 8 * NP * W;      // [5][NP*W] FP64 lambda
+  static constexpr int OFF_LH = OFF_L + 5 * NP * W;      // [5][NI] records: adjoint of the interface flux
+  static constexpr int OFF_G = OFF_LH + 5 * NI * W;      // [9][NP] records: first differences; later the
+                                                         //   gathered FP64 sums [9][TP*W]
+  static constexpr int OFF_T = OFF_G + 9 * NP * W;       // [9][NW] records: T/6
+  static constexpr int OFF_B = OFF_T + 9 * NW * W;       // [9][3][NW] records: 1/b_k, later the window adjoints
+  static constexpr int OFF_REC = OFF_B + 27 * NW * W;    // [5][NI] records: jumps of u_0..u_4
+  static constexpr int OFF_RD = OFF_REC + 5 * NI * W;    // [15][NI] records: Roe adjoints
+  static constexpr int OFF_WC = OFF_RD + 15 * NI * W;    // [9][9][NI] records: weights, then contributions
+  static constexpr int WORDS = OFF_WC + 81 * NI * W;
   static constexpr int BYTES = WORDS * 8;
+  static_assert(OFF_LH % 2 == 0 && OFF_G % 2 == 0 && OFF_B % 2 == 0 && OFF_RD % 2 == 0, "records are 16-byte aligned");
+  // phase D: the interfaces of both lines on whole warps, the flux components beside them
+  static constexpr int D_THREADS = (NI * W + 31) / 32 * 32;
 };
-using APF = AdjPlanDF<32, 2, 256, 2>;
+using APF = AdjPlanDF<32, 256, 2>;
 
 __device__ __forceinline__ df df_sub(df x, df y) { return df_add_fast(x, df_neg(y)); }
 __device__ __forceinline__ float2 df_pack(df x) { return make_float2(x.hi, x.lo); }
 __device__ __forceinline__ df df_unpack(float2 v) { return df{v.x, v.y}; }
 
-struct DFConst {
-  df third, sixth, c263;  // 1/3, 1/6, 26/3
-};
+// Lane `line` of a record.
+__device__ __forceinline__ df rec_lane(const float4* r, int line) {
+  const float* f = reinterpret_cast<const float*>(r);
+  return df{f[line], f[2 + line]};
+}
+__device__ __forceinline__ void set_rec_lane(float4* r, int line, df x) {
+  float* f = reinterpret_cast<float*>(r);
+  f[line] = x.hi;
+  f[2 + line] = x.lo;
+}
 
 // The WENO pieces below take the two lines of a tile at once (two-lane double-float,
 // df2.cuh: each lane computes what one line would).
 // Products and positive sums in this section are left unnormalised where they feed another
 // double-float operation (df2_mul_u and friends: the same values, |lo| a few ulp(hi)).
-struct DF2Const {
-  df2 third, sixth, c263;
-};
 __device__ __forceinline__ df2 df2_sub(df2 x, df2 y) { return df2_add_fast(x, df2_neg(y)); }
+
+// 1/y for a normalised y, refined seed, unnormalised result (df2_div_ru with x = 1).
+__device__ __forceinline__ df2 df2_rcp_ru(df2 y) {
+  const float2 one = f2splat(1.0f);
+  float2 r = make_float2(rcp_seed(y.hi.x), rcp_seed(y.hi.y));
+  r = f2fma(r, f2fma(f2neg(y.hi), r, one), r);
+  const df2 p = two_prod2(r, y.hi);
+  const float2 rem = f2fma(f2neg(r), y.lo, f2sub(f2sub(one, p.hi), p.lo));
+  return df2{r, f2mul(rem, r)};
+}
 
 // The three weights of one reconstruction from the reciprocals r_k = 1/b_k of its window
 // terms (candidate order 0, 1, 2; optimal weights 1, 6, 3 over 10):
@@ -635,59 +668,29 @@ __device__ __forceinline__ void df2_omega(df2 r0, df2 r1, df2 r2, df2 om[3]) {
   const df2 a0 = df2_sqr_u(r0);
   const df2 a1 = df2_mul_f_u(df2_sqr_u(r1), 6.0f);
   const df2 a2 = df2_mul_f_u(df2_sqr_u(r2), 3.0f);
-  const df2 r = df2_div(df2{f2splat(1.0f), f2splat(0.0f)}, df2_add_pos_u(a0, df2_add_pos_u(a1, a2)));
+  const df2 sum = df2_add_pos_u(a0, df2_add_pos_u(a1, a2));
+  const df2 r = df2_rcp_ru(fast_two_sum2(sum.hi, sum.lo));
   om[0] = df2_mul_u(a0, r);
   om[1] = df2_mul_u(a1, r);
   om[2] = df2_mul_u(a2, r);
 }
 
-// Offset M of the reconstruction from its candidate 1, and the candidate differences.
-__device__ __forceinline__ df2 df2_adj_offset(df2 g0, df2 g1, df2 g2, df2 g3, const df2 om[3], const DF2Const& k,
-                                              df2& E0, df2& E2, df2 s[3]) {
-  s[0] = df2_sub(g1, g0);
-  s[1] = df2_sub(g2, g1);
-  s[2] = df2_sub(g3, g2);
-  E0 = df2_mul_u(df2_sub(s[0], s[1]), k.third);
-  E2 = df2_mul_u(df2_sub(s[1], s[2]), k.sixth);
-  return df2_add_fast(df2_mul_u(om[0], E0), df2_mul_u(om[2], E2));
+// M (M^R with the mirrored windows' third differences): ta6 = T_f/6 (T_{f+2}/6), tb6 = T_{f+1}/6.
+__device__ __forceinline__ df2 df2_adj_offset(const df2 om[3], df2 ta6, df2 tb6) {
+  return df2_add_fast(df2_twice(df2_mul_u(om[0], ta6)), df2_mul_u(om[2], tb6));
 }
 
-// y * d(value)/d(q_t), t = 0..4, of the reconstruction of stencil differences g0..g3 with
-// the reciprocals rb0..rb2 of its window terms and weights om (as weno_adjoint, in
-// double-float).
-__device__ __forceinline__ void df2_recon_adjoint(df2 g0, df2 g1, df2 g2, df2 g3, df2 rb0, df2 rb1, df2 rb2,
-                                                  const df2 om[3], df2 y, const DF2Const& k, df2 out[5]) {
-  df2 s[3], E0, E2;
-  const df2 M = df2_adj_offset(g0, g1, g2, g3, om, k, E0, E2, s);
-  const df2 v0 = df2_sub(df2_mul_f_u(g1, 3.0f), g0);
-  const df2 v1 = df2_add_fast(g1, g2);
-  const df2 v2 = df2_sub(g3, df2_mul_f_u(g2, 3.0f));
+// Adjoint y of one reconstruction value (sign: of +M): half the adjoints of its window terms b_k
+// (r_k = 1/b_k) into kb[3], those of ta6 and tb6 into ta, tb.
+__device__ __forceinline__ void df2_recon_adjoint(const df2 om[3], df2 r0, df2 r1, df2 r2, df2 ta6, df2 tb6, df2 y,
+                                                  df2 kb[3], df2& ta, df2& tb) {
+  const df2 M = df2_adj_offset(om, ta6, tb6);
   const df2 y0 = df2_mul_u(y, om[0]), y1 = df2_mul_u(y, om[1]), y2 = df2_mul_u(y, om[2]);
-  // adjoints of b_k: -2 y_k (q_k - q) / b_k with q_0 - q = E0 - M, q_1 - q = -M, q_2 - q = E2 - M
-  const df2 k0 = df2_twice(df2_mul(df2_mul_u(y0, df2_sub(M, E0)), rb0));
-  const df2 k1 = df2_twice(df2_mul(df2_mul_u(y1, M), rb1));
-  const df2 k2 = df2_twice(df2_mul(df2_mul_u(y2, df2_sub(M, E2)), rb2));
-  // direct term sum_k y_k dq_k/dq_t
-  out[0] = df2_mul_u(y0, k.third);
-  out[1] = df2_neg(df2_mul_u(df2_add_fast(df2_mul_f_u(y0, 7.0f), y1), k.sixth));
-  out[2] = df2_mul_u(df2_add_fast(df2_mul_f_u(y0, 11.0f), df2_add_fast(df2_mul_f_u(y1, 5.0f), df2_twice(y2))), k.sixth);
-  out[3] = df2_mul_u(df2_add_fast(df2_twice(y1), df2_mul_f_u(y2, 5.0f)), k.sixth);
-  out[4] = df2_neg(df2_mul_u(y2, k.sixth));
-  // db/d(x, y, z) of a window = 26/3 s (1, -2, 1) + 2 v dv/d(x, y, z)
-  df2 t = df2_mul_u(df2_mul_u(s[0], k0), k.c263), r = df2_twice(df2_mul_u(v0, k0));  // dv = (1, -4, 3)
-  out[0] = df2_add_fast(out[0], df2_add_fast(t, r));
-  out[1] = df2_sub(out[1], df2_add_fast(df2_twice(t), df2_twice(df2_twice(r))));
-  out[2] = df2_add_fast(out[2], df2_add_fast(t, df2_mul_f_u(r, 3.0f)));
-  t = df2_mul_u(df2_mul_u(s[1], k1), k.c263);
-  r = df2_twice(df2_mul_u(v1, k1));  // dv = (-1, 0, 1)
-  out[1] = df2_add_fast(out[1], df2_sub(t, r));
-  out[2] = df2_sub(out[2], df2_twice(t));
-  out[3] = df2_add_fast(out[3], df2_add_fast(t, r));
-  t = df2_mul_u(df2_mul_u(s[2], k2), k.c263);
-  r = df2_twice(df2_mul_u(v2, k2));  // dv = (3, -4, 1)
-  out[2] = df2_add_fast(out[2], df2_add_fast(t, df2_mul_f_u(r, 3.0f)));
-  out[3] = df2_sub(out[3], df2_add_fast(df2_twice(t), df2_twice(df2_twice(r))));
-  out[4] = df2_add_fast(out[4], df2_add_fast(t, r));
+  kb[0] = df2_mul(df2_mul_u(y0, df2_sub(M, df2_twice(ta6))), r0);
+  kb[1] = df2_mul(df2_mul_u(y1, M), r1);
+  kb[2] = df2_mul(df2_mul_u(y2, df2_sub(M, tb6)), r2);
+  ta = df2_twice(y0);
+  tb = y2;
 }
 
 __device__ __forceinline__ double pow2d(int k) { return __hiloint2double((k + 1023) << 20, 0); }
@@ -869,7 +872,9 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
   const int nD = a.g.n[D];
   const int na = a.g.n[AX];
   const long long N = a.g.N;
-  const int s0 = blockIdx.x * TP;
+  int s0, len;
+  tile_span(D, nD, a.tile_u, a.tile_r, blockIdx.x, s0, len);
+  const int np = len + 10, ni = len + 5, nw = len + 8;  // this tile's points with halo, interfaces, windows
   const int a0 = blockIdx.y * W;
   const int bz = blockIdx.z;
   const int tid = threadIdx.x;
@@ -877,32 +882,26 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
   double* q = sm + APF::OFF_Q;
   double* ri = sm + APF::OFF_RI;
   double* lm = sm + APF::OFF_L;
-  // G, Bw and wc hold the two lines of the tile side by side (hi0, hi1, lo0, lo1)
-  static_assert(W == 2, "the two-lane phases take the tile's two lines together");
+  float4* LH4 = reinterpret_cast<float4*>(sm + APF::OFF_LH);  // [5][NI]
   float4* G4 = reinterpret_cast<float4*>(sm + APF::OFF_G);    // [9][NP]
+  float4* T4 = reinterpret_cast<float4*>(sm + APF::OFF_T);    // [9][NW]
   float4* Bw4 = reinterpret_cast<float4*>(sm + APF::OFF_B);   // [9][3][NW]
-  double* rec = sm + APF::OFF_REC;
-  double* rd = sm + APF::OFF_RD;
-  float4* wc4 = reinterpret_cast<float4*>(sm + APF::OFF_WC);  // [9][6][NI]
-  DFConst kc;
-  {
-    const double third = 1.0 / 3.0, sixth = 1.0 / 6.0, c263 = 26.0 / 3.0;
-    kc.third = df{(float)third, (float)(third - (double)(float)third)};
-    kc.sixth = df{(float)sixth, (float)(sixth - (double)(float)sixth)};
-    kc.c263 = df{(float)c263, (float)(c263 - (double)(float)c263)};
-  }
-  const DF2Const kc2{df2_splat(kc.third), df2_splat(kc.sixth), df2_splat(kc.c263)};
-  const df eps4{(float)a.eps4, (float)(a.eps4 - (double)(float)a.eps4)};
-  const df c133{(float)(13.0 / 3.0), (float)(13.0 / 3.0 - (double)(float)(13.0 / 3.0))};
+  float4* J4 = reinterpret_cast<float4*>(sm + APF::OFF_REC);  // [5][NI]
+  float4* RD4 = reinterpret_cast<float4*>(sm + APF::OFF_RD);  // [15][NI]
+  float4* wc4 = reinterpret_cast<float4*>(sm + APF::OFF_WC);  // [9][9][NI]
+  constexpr float sx_hi = (float)(1.0 / 6.0), sx_lo = (float)(1.0 / 6.0 - (double)sx_hi);
+  constexpr float c133_hi = (float)(13.0 / 3.0), c133_lo = (float)(13.0 / 3.0 - (double)c133_hi);
+  const df2 sixth = df2_splat(df{sx_hi, sx_lo}), c133 = df2_splat(df{c133_hi, c133_lo});
   if (tid == 0) s_emax = -2000;
   __syncthreads();
 
   // ---- A: load; largest binary exponent of lambda in the tile ----------------------------
   int emax = -2000;
-  for (int item = tid; item < NP * W; item += APF::THREADS) {
+  for (int item = tid; item < np * W; item += APF::THREADS) {
     int pos, line;
-    tile_split<D, W>(item, NP, pos, line);
-    const int c = wrap_idx(s0 - 5 + pos, nD);
+    item_split<D, W>(item, np, c_rcp20.v[np], pos, line);
+    int c = s0 - 5 + pos;
+    if (c < 0 || c >= nD) c = wrap_idx(c, nD);
     const int la = min(a0 + line, na - 1);
     const long long p = tile_flat<D>(a.g, c, la, bz);
     double U[5];
@@ -938,102 +937,148 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
   emax = __reduce_max_sync(0xffffffffu, emax);
   if ((tid & 31) == 0) atomicMax(&s_emax, emax);
   __syncthreads();
-  // E = exponent of the largest |lambda| (0 if lambda vanishes on the tile); lambda / 2^E
+  // E = exponent of the largest |lambda| (0 if lambda vanishes on the tile)
   const int E = (s_emax == -2000) ? 0 : max(-1000, min(1000, s_emax));
-  const double down = pow2d(-E);
   int range_bad = 0;
-  for (int item = tid; item < NP * W; item += APF::THREADS) {
-    int pos, line;
-    tile_split<D, W>(item, NP, pos, line);
-    const int s = tile_idx<D, W>(pos, line, NP);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) lm[v * NP * W + s] *= down;
-  }
   // first differences of the 9 scalars, FP64, kept as double-float; both lines of the tile
-  // per item, stored side by side (hi0, hi1, lo0, lo1) for the two-lane phases below
-  for (int item = tid; item < 9 * (NP - 1); item += APF::THREADS) {
-    const int m = item / (NP - 1);
-    const int j = item - m * (NP - 1);
+  // per item, stored side by side for the two-lane phases below
+  const int ng = np - 1;
+  const unsigned rcp_ng = c_rcp20.v[ng], rcp_ni = c_rcp20.v[ni];
+  for (int item = tid; item < 9 * ng; item += APF::THREADS) {
+    const int m = (int)(((unsigned)item * rcp_ng) >> 20);
+    const int j = item - m * ng;
     const double* qm = q + m * NP * W;
     const double d0 = qm[tile_idx<D, W>(j + 1, 0, NP)] - qm[tile_idx<D, W>(j, 0, NP)];
     const double d1 = qm[tile_idx<D, W>(j + 1, 1, NP)] - qm[tile_idx<D, W>(j, 1, NP)];
     G4[m * NP + j] = df2_to4(df2_pack(d2df_bits(d0), d2df_bits(d1)));
   }
+  // adjoint of the interface fluxes, (lambda_{i+1} - lambda_i) / dx / 2^E
+  {
+    const double sc = rdx * pow2d(-E);
+    for (int item = APF::THREADS - 1 - tid; item < 5 * ni; item += APF::THREADS) {
+      const int v = (int)(((unsigned)item * rcp_ni) >> 20);
+      const int f = item - v * ni;
+      const double* l = lm + v * NP * W;
+      const double d0 = (l[tile_idx<D, W>(f + 3, 0, NP)] - l[tile_idx<D, W>(f + 2, 0, NP)]) * sc;
+      const double d1 = (l[tile_idx<D, W>(f + 3, 1, NP)] - l[tile_idx<D, W>(f + 2, 1, NP)]) * sc;
+      LH4[v * NI + f] = df2_to4(df2_pack(d2df_bits(d0), d2df_bits(d1)));
+    }
+  }
   __syncthreads();
 
-  // ---- B: window terms b_k of every window, stored as 1/b_k (both lines at once) -----------------
+  // ---- B: window terms b_k of every window, stored as 1/b_k, and T/6 (both lines at once) ---------
   {
-    const df2 c133_2 = df2_splat(c133), eps4_2 = df2_splat(eps4);
-    const df2 one{f2splat(1.0f), f2splat(0.0f)};
-    for (int item = tid; item < 9 * NW; item += APF::THREADS) {
-      const int m = item / NW;
-      const int w = item - m * NW;
+    const df2 eps4 = df2_splat(df{(float)a.eps4, (float)(a.eps4 - (double)(float)a.eps4)});
+    const float2 four = f2splat(4.0f);
+    const unsigned rcp_nw = c_rcp20.v[nw];
+    for (int item = tid; item < 9 * nw; item += APF::THREADS) {
+      const int m = (int)(((unsigned)item * rcp_nw) >> 20);
+      const int w = item - m * nw;
       const float4* Gm = G4 + m * NP;
-      const df2 g0 = df2_from4(Gm[w]), g1 = df2_from4(Gm[w + 1]);
+      const df2 g0 = df2_from4(Gm[w]), g1 = df2_from4(Gm[w + 1]), g2 = df2_from4(Gm[min(w + 2, ng - 1)]);
       const df2 sw = df2_sub(g1, g0);
-      const df2 aa = df2_add_pos_u(df2_mul_u(df2_sqr_u(sw), c133_2), eps4_2);
-      const df2 b0 = df2_add_pos_u(df2_sqr_u(df2_sub(df2_mul_f_u(g1, 3.0f), g0)), aa);
-      const df2 b1 = df2_add_pos_u(df2_sqr_u(df2_add_fast(g0, g1)), aa);
-      const df2 b2 = df2_add_pos_u(df2_sqr_u(df2_sub(g1, df2_mul_f_u(g0, 3.0f))), aa);
+      // (the last window's T needs a difference beyond the tile and is never read)
+      T4[m * NW + w] = df2_to4(df2_mul_u(df2_sub(sw, df2_sub(g2, g1)), sixth));
+      // b_1 = u^2 + aa, b_{0,2} = (b_1 + 4 s^2) +- 4 u s with u = g0 + g1, aa = (13/3) s^2 + 4 eps
+      const df2 s2 = df2_sqr_u(sw);
+      const df2 u2 = df2_add_fast(g0, g1);
+      const df2 b1 = df2_add_pos_u(df2_sqr_u(u2), df2_add_pos_u(df2_mul_u(s2, c133), eps4));
+      const df2 pq = df2_add_ordered_u(b1, df2_scale(s2, four));
+      const df2 r4 = df2_scale(df2_mul_u(u2, sw), four);
+      const df2 b0 = df2_add_ordered(pq, r4), b2 = df2_add_ordered(pq, df2_neg(r4));
       // their reciprocals: the weights (c_k / b_k^2) and the adjoints of b_k (omega_k / b_k) need only those
-      Bw4[(m * 3 + 0) * NW + w] = df2_to4(df2_div(one, b0));
-      Bw4[(m * 3 + 1) * NW + w] = df2_to4(df2_div(one, b1));
-      Bw4[(m * 3 + 2) * NW + w] = df2_to4(df2_div(one, b2));
+      Bw4[(m * 3 + 0) * NW + w] = df2_to4(df2_rcp_ru(b0));
+      Bw4[(m * 3 + 1) * NW + w] = df2_to4(df2_rcp_ru(fast_two_sum2(b1.hi, b1.lo)));
+      Bw4[(m * 3 + 2) * NW + w] = df2_to4(df2_rcp_ru(b2));
       // b^2 must stay inside the float range (differences of the data up to ~1e9)
       range_bad |= !(fmaxf(b0.hi.x, fmaxf(b1.hi.x, b2.hi.x)) < 1e18f) || !(fmaxf(b0.hi.y, fmaxf(b1.hi.y, b2.hi.y)) < 1e18f);
     }
   }
   __syncthreads();
 
-  // ---- C: jumps of the u reconstructions (for the Roe adjoint), both lines at once -----------
-  for (int item = tid; item < 5 * NI; item += APF::THREADS) {
-    const int m = item / NI;
-    const int f = item - m * NI;
-    const float4* Gm = G4 + m * NP;
-    df2 g[5];
+  auto ldB = [&](int m, int k, int w) { return df2_from4(Bw4[(m * 3 + k) * NW + w]); };
+  auto ldT = [&](int m, int w) { return df2_from4(T4[m * NW + w]); };
+
+  // ---- C: weights and jumps of the u reconstructions (for the Roe adjoint), both lines at once ------
+  for (int item = tid; item < 5 * ni; item += APF::THREADS) {
+    const int m = (int)(((unsigned)item * rcp_ni) >> 20);
+    const int f = item - m * ni;
+    float4* wm = wc4 + m * 9 * NI + f;
+    df2 om[3];
+    const df2 T1 = ldT(m, f + 1);
+    df2_omega(ldB(m, 0, f), ldB(m, 1, f + 1), ldB(m, 2, f + 2), om);
+    const df2 ML = df2_adj_offset(om, ldT(m, f), T1);
 #pragma unroll
-    for (int j = 0; j < 5; ++j) g[j] = df2_from4(Gm[f + j]);
-    const float4* B = Bw4 + m * 3 * NW;
-    auto ldb = [&](int k, int w) { return df2_from4(B[k * NW + w]); };
-    df2 omL[3], omR[3], s[3], E0, E2;
-    df2_omega(ldb(0, f), ldb(1, f + 1), ldb(2, f + 2), omL);
-    const df2 ML = df2_adj_offset(g[0], g[1], g[2], g[3], omL, kc2, E0, E2, s);
-    df2_omega(ldb(2, f + 3), ldb(1, f + 2), ldb(0, f + 1), omR);
-    const df2 MR = df2_adj_offset(df2_neg(g[4]), df2_neg(g[3]), df2_neg(g[2]), df2_neg(g[1]), omR, kc2, E0, E2, s);
-    // the jump ûR - ûL = (P3 - P2) - (2 g2 + g3)/6 + MR - (2 g2 + g1)/6 - ML, in double-float
-    // (the values themselves are not needed)
-    const df2 g22 = df2_twice(g[2]);
-    const df2 lin = df2_mul_u(df2_add_fast(df2_add_fast(g22, g[1]), df2_add_fast(g22, g[3])), kc2.sixth);
-    const df2 du = df2_add_fast(df2_add_fast(g[2], df2_neg(lin)), df2_add_fast(MR, df2_neg(ML)));
-    float2* rj = reinterpret_cast<float2*>(rec) + m * NI * W;
-    rj[tile_idx<D, W>(f, 0, NI)] = df_pack(df2_lane0(du));
-    rj[tile_idx<D, W>(f, 1, NI)] = df_pack(df2_lane1(du));
-    // the weights, for phase E (which overwrites these slots with its contributions)
-    float4* wm = wc4 + m * 6 * NI;
+    for (int k = 0; k < 3; ++k) wm[k * NI] = df2_to4(om[k]);  // for phase E1, which overwrites these slots
+    df2_omega(ldB(m, 2, f + 3), ldB(m, 1, f + 2), ldB(m, 0, f + 1), om);
+    const df2 MR = df2_adj_offset(om, ldT(m, f + 2), T1);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      wm[k * NI + f] = df2_to4(omL[k]);
-      wm[(3 + k) * NI + f] = df2_to4(omR[k]);
-    }
+    for (int k = 0; k < 3; ++k) wm[(3 + k) * NI] = df2_to4(om[k]);
+    J4[m * NI + f] = df2_to4(df2_sub(T1, df2_add_fast(ML, MR)));
   }
   __syncthreads();
 
-  // ---- D: adjoint of the Roe flux, in double-float -----------------------------------------
-  {
+  // ---- E1 (one scalar and interface, both lines): adjoints of the two reconstructions -> half the
+  //      adjoints of their six window terms (slots 0-2 left, 3-5 right) and those of T_f/6, T_{f+1}/6,
+  //      T_{f+2}/6 (slots 6-8)
+  auto recon = [&](int m, int f) {
+    float4* wm = wc4 + m * 9 * NI + f;
+    const df2 T0 = ldT(m, f), T1 = ldT(m, f + 1), T2 = ldT(m, f + 2);
+    const df2 l0 = ldB(m, 0, f), l1 = ldB(m, 1, f + 1), l2 = ldB(m, 2, f + 2);
+    const df2 r0 = ldB(m, 2, f + 3), r1 = ldB(m, 1, f + 2), r2 = ldB(m, 0, f + 1);
+    df2 yL, yR, om[3], kb[3], ta, tb, tc;
+    if (m < 5) {
+      yR = df2_from4(RD4[m * NI + f]);
+      yL = df2_neg(yR);
+      tc = yR;  // linear part of the jump
+      if (m == 1 + D) {  // mass flux f_0 = u_{1+D}: (f^L + f^R)/2 part
+        const df2 h0 = df2_scale(df2_from4(LH4[f]), f2splat(0.5f));
+        yL = df2_add_fast(yL, h0);
+        yR = df2_add_fast(yR, h0);
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) om[k] = df2_from4(wm[k * NI]);
+    } else {
+      yL = yR = df2_scale(df2_from4(LH4[(m - 4) * NI + f]), f2splat(0.5f));
+      df2_omega(l0, l1, l2, om);
+    }
+    range_bad |= !(fabsf(yL.hi.x) < 1e30f && fabsf(yR.hi.x) < 1e30f && fabsf(yL.hi.y) < 1e30f && fabsf(yR.hi.y) < 1e30f);
+    df2_recon_adjoint(om, l0, l1, l2, T0, T1, yL, kb, ta, tb);
+    if (m < 5) tb = df2_add_fast(tb, tc);
+    wm[0 * NI] = df2_to4(kb[0]);
+    wm[1 * NI] = df2_to4(kb[1]);
+    wm[2 * NI] = df2_to4(kb[2]);
+    wm[6 * NI] = df2_to4(ta);
+    if (m < 5) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) om[k] = df2_from4(wm[(3 + k) * NI]);
+    } else {
+      df2_omega(r0, r1, r2, om);
+    }
+    df2 tbR;
+    df2_recon_adjoint(om, r0, r1, r2, T2, T1, df2_neg(yR), kb, ta, tbR);  // value^R = ... - M^R
+    wm[3 * NI] = df2_to4(kb[0]);
+    wm[4 * NI] = df2_to4(kb[1]);
+    wm[5 * NI] = df2_to4(kb[2]);
+    wm[7 * NI] = df2_to4(df2_add_fast(tb, tbR));
+    wm[8 * NI] = df2_to4(ta);
+  };
+
+  // ---- D: adjoint of the Roe flux, in double-float, on the first warps; the flux components'
+  //      reconstruction adjoints on the others
+  if (tid < APF::D_THREADS) {
     int bad = 0;
-    const df gam = d2df_bits(a.gamma), gm1 = d2df_bits(a.gamma - 1.0), hd = d2df_bits(a.hdelta);
-    const float2* rf = reinterpret_cast<const float2*>(ri);
-    float2* rdf = reinterpret_cast<float2*>(rd);
-    for (int item = tid; item < NI * W; item += APF::THREADS) {
+    if (tid < ni * W) {
+      const df gam = d2df_bits(a.gamma), gm1 = d2df_bits(a.gamma - 1.0), hd = d2df_bits(a.hdelta);
+      const float2* rf = reinterpret_cast<const float2*>(ri);
       int f, line;
-      tile_split<D, W>(item, NI, f, line);
-      const int o = tile_idx<D, W>(f, line, NI);
+      item_split<D, W>(tid, ni, rcp_ni, f, line);
       const int sa = tile_idx<D, W>(f + 2, line, NP), sb = tile_idx<D, W>(f + 3, line, NP);
       df du[5], Lh[5], Va[3], Vb[3];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        du[v] = df_unpack(reinterpret_cast<const float2*>(rec)[v * NI * W + o]);
-        Lh[v] = d2df_bits((lm[v * NP * W + sb] - lm[v * NP * W + sa]) * rdx);
+        du[v] = rec_lane(J4 + v * NI + f, line);
+        Lh[v] = rec_lane(LH4 + v * NI + f, line);
       }
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
@@ -1041,111 +1086,100 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
         Vb[m] = df_unpack(rf[(1 + m) * NP * W + sb]);
       }
       df dub[5], ga[5], gb[5];
-      bad |= roe_adjoint_df<D>(du, Lh, df_unpack(rf[sa]), df_unpack(rf[sb]), Va, Vb, df_unpack(rf[4 * NP * W + sa]),
-                               df_unpack(rf[4 * NP * W + sb]), df_unpack(rf[6 * NP * W + sa]),
-                               df_unpack(rf[7 * NP * W + sa]), df_unpack(rf[6 * NP * W + sb]),
-                               df_unpack(rf[7 * NP * W + sb]), gam, gm1, hd, dub, ga, gb);
+      bad = roe_adjoint_df<D>(du, Lh, df_unpack(rf[sa]), df_unpack(rf[sb]), Va, Vb, df_unpack(rf[4 * NP * W + sa]),
+                              df_unpack(rf[4 * NP * W + sb]), df_unpack(rf[6 * NP * W + sa]),
+                              df_unpack(rf[7 * NP * W + sa]), df_unpack(rf[6 * NP * W + sb]),
+                              df_unpack(rf[7 * NP * W + sb]), gam, gm1, hd, dub, ga, gb);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        rdf[v * NI * W + o] = df_pack(dub[v]);
-        rdf[(5 + v) * NI * W + o] = df_pack(ga[v]);
-        rdf[(10 + v) * NI * W + o] = df_pack(gb[v]);
+        set_rec_lane(RD4 + v * NI + f, line, dub[v]);
+        set_rec_lane(RD4 + (5 + v) * NI + f, line, ga[v]);
+        set_rec_lane(RD4 + (10 + v) * NI + f, line, gb[v]);
       }
     }
     if (__any_sync(0xffffffffu, bad & 1) && (tid & 31) == 0) atomicOr(a.status, ST_NONPHYS);
     range_bad |= bad & 2;
+  } else {
+    for (int item = tid - APF::D_THREADS; item < 4 * ni; item += APF::THREADS - APF::D_THREADS) {
+      const int m = (int)(((unsigned)item * rcp_ni) >> 20);
+      recon(5 + m, item - m * ni);
+    }
   }
   __syncthreads();
 
-  // ---- E: reconstruction adjoints -> six stencil contributions per scalar and interface, -----
-  //      both lines at once
-  for (int item = tid; item < 9 * NI; item += APF::THREADS) {
-    const int m = item / NI;
-    const int f = item - m * NI;
-    df y2[2][2];  // [line][left, right]
-#pragma unroll
-    for (int line = 0; line < 2; ++line) {
-      const int o = tile_idx<D, W>(f, line, NI);
-      const int sa = tile_idx<D, W>(f + 2, line, NP), sb = tile_idx<D, W>(f + 3, line, NP);
-      df yL, yR;
-      if (m < 5) {
-        const df gdu = df_unpack(reinterpret_cast<const float2*>(rd)[m * NI * W + o]);
-        yL = df_neg(gdu);
-        yR = gdu;
-        if (m == 1 + D) {  // mass flux f_0 = u_{1+D}: (f^L + f^R)/2 part
-          const df h0 = d2df_bits(0.5 * ((lm[sb] - lm[sa]) * rdx));
-          yL = df_add_fast(yL, h0);
-          yR = df_add_fast(yR, h0);
-        }
-      } else {
-        yL = yR = d2df_bits(0.5 * ((lm[(m - 4) * NP * W + sb] - lm[(m - 4) * NP * W + sa]) * rdx));
-      }
-      range_bad |= !(fabsf(yL.hi) < 1e30f && fabsf(yR.hi) < 1e30f);
-      y2[line][0] = yL;
-      y2[line][1] = yR;
-    }
-    const float4* Gm = G4 + m * NP;
-    df2 g[5];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) g[j] = df2_from4(Gm[f + j]);
-    const float4* B = Bw4 + m * 3 * NW;
-    auto ldb = [&](int k, int w) { return df2_from4(B[k * NW + w]); };
-    float4* wm = wc4 + m * 6 * NI;
-    df2 omL[3], omR[3];
-    if (m < 5) {  // stored by phase C
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        omL[k] = df2_from4(wm[k * NI + f]);
-        omR[k] = df2_from4(wm[(3 + k) * NI + f]);
-      }
-    } else {
-      df2_omega(ldb(0, f), ldb(1, f + 1), ldb(2, f + 2), omL);
-      df2_omega(ldb(2, f + 3), ldb(1, f + 2), ldb(0, f + 1), omR);
-    }
-    df2 cL[5], cR[5];
-    df2_recon_adjoint(g[0], g[1], g[2], g[3], ldb(0, f), ldb(1, f + 1), ldb(2, f + 2), omL,
-                             df2_pack(y2[0][0], y2[1][0]), kc2, cL);
-    df2_recon_adjoint(df2_neg(g[4]), df2_neg(g[3]), df2_neg(g[2]), df2_neg(g[1]), ldb(2, f + 3),
-                             ldb(1, f + 2), ldb(0, f + 1), omR, df2_pack(y2[0][1], y2[1][1]), kc2, cR);
-    wm[0 * NI + f] = df2_to4(cL[0]);
-#pragma unroll
-    for (int j = 1; j < 5; ++j) wm[j * NI + f] = df2_to4(df2_add_fast(cL[j], cR[5 - j]));
-    wm[5 * NI + f] = df2_to4(cR[0]);
+  // ---- E1 of the conserved variables
+  for (int item = tid; item < 5 * ni; item += APF::THREADS) {
+    const int m = (int)(((unsigned)item * rcp_ni) >> 20);
+    recon(m, item - m * ni);
   }
   if (__any_sync(0xffffffffu, range_bad) && (tid & 31) == 0) atomicOr(a.status, ST_DF_RANGE);
+  __syncthreads();
+
+  // ---- E2 (one scalar and window 2 .. len+4, both lines): the window's adjoint sums -> a quarter of the
+  //      adjoints A, B of its two first differences (slots 0, 1) and the adjoint of T/6 (slot 2), into the
+  //      dead reciprocals.  With k_j half the adjoint of b_j and K their sum,
+  //      A/4 = -(13/3) s K - v_0 k_0 + v_1 k_1 - 3 v_2 k_2,  B/4 = (13/3) s K + 3 v_0 k_0 + v_1 k_1 + v_2 k_2
+  {
+    const int nv = len + 3;
+    const unsigned rcp_nv = c_rcp20.v[nv];
+    for (int item = tid; item < 9 * nv; item += APF::THREADS) {
+      const int m = (int)(((unsigned)item * rcp_nv) >> 20);
+      const int w = 2 + item - m * nv;
+      const float4* wm = wc4 + m * 9 * NI;
+      auto ldw = [&](int k, int f) { return df2_from4(wm[k * NI + f]); };
+      Bw4[(m * 3 + 2) * NW + w] = df2_to4(df2_add_fast(df2_add_fast(ldw(6, w), ldw(7, w - 1)), ldw(8, w - 2)));
+      if (w < 3) continue;  // only its T is used
+      const df2 k0 = df2_add_fast(ldw(0, w), ldw(5, w - 1));
+      const df2 k1 = df2_add_fast(ldw(1, w - 1), ldw(4, w - 2));
+      const df2 k2 = df2_add_fast(ldw(2, w - 2), ldw(3, w - 3));
+      const df2 g0 = df2_from4(G4[m * NP + w]), g1 = df2_from4(G4[m * NP + w + 1]);
+      const df2 ps = df2_mul_u(df2_mul_u(df2_sub(g1, g0), df2_add_fast(k0, df2_add_fast(k1, k2))), c133);
+      const df2 p0 = df2_mul_u(df2_sub(df2_mul_f_u(g1, 3.0f), g0), k0);
+      const df2 p1 = df2_mul_u(df2_add_fast(g0, g1), k1);
+      const df2 p2 = df2_mul_u(df2_sub(g1, df2_mul_f_u(g0, 3.0f)), k2);
+      Bw4[(m * 3 + 0) * NW + w] = df2_to4(df2_sub(df2_sub(p1, ps), df2_add_fast(p0, df2_mul_f_u(p2, 3.0f))));
+      Bw4[(m * 3 + 1) * NW + w] = df2_to4(df2_add_fast(df2_add_fast(p1, ps), df2_add_fast(p2, df2_mul_f_u(p0, 3.0f))));
+    }
+  }
   __syncthreads();
 
   // ---- F: gather, adjoint of the point fluxes, scale back, epilogue ----------------------------
   const double up = pow2d(E);
   const double gm1 = a.gamma - 1.0;
-  // F1: the gather, one (scalar, point, line) per item, into the dead window-term space
-  static_assert(9 * TP * W <= 27 * NW * W, "gathered sums fit the window-term space");
-  double* gsm = sm + APF::OFF_B;  // [9][TP*W]
+  // F1: the gather, one scalar and point of both lines per item, into the dead first differences:
+  //   (A_{p-1} - A_p) + (B_{p-2} - B_{p-1}) + [T_p - T_{p-3} + 3 (T_{p-2} - T_{p-1})]/6
+  //   + [7 (h_{p-2} + h_{p-3}) - (h_{p-1} + h_{p-4})]/6 (flux components), h half the interface adjoint
+  //   + the Roe-average adjoints of the point's two interfaces (conserved variables)
+  static_assert(TP * W <= NP * W, "gathered sums fit the space of the first differences");
+  double* gsm = sm + APF::OFF_G;  // [9][TP*W]
   {
-    const float* wcf = reinterpret_cast<const float*>(wc4);  // lane `line` of a pair: hi at +line, lo at +2+line
-    const float2* rdf = reinterpret_cast<const float2*>(rd);
-    for (int item = tid; item < 9 * TP * W; item += APF::THREADS) {
-      const int m = item / (TP * W);
-      int pp, line;
-      tile_split<D, W>(item - m * TP * W, TP, pp, line);
-      const int pos = pp + 5;
-      auto ldw = [&](int slot) { return df{wcf[4 * slot + line], wcf[4 * slot + 2 + line]}; };
-      df acc = ldw(m * 6 * NI + pos);
-#pragma unroll
-      for (int j = 1; j < 6; ++j) acc = df_add_fast(acc, ldw((m * 6 + j) * NI + pos - j));
-      if (m < 5) {  // the Roe-average adjoints of the two interfaces next to the point
-        const int oa = tile_idx<D, W>(pos - 2, line, NI), ob = tile_idx<D, W>(pos - 3, line, NI);
-        acc = df_add_fast(acc, df_add_fast(df_unpack(rdf[(5 + m) * NI * W + oa]), df_unpack(rdf[(10 + m) * NI * W + ob])));
+    const unsigned rcp_len = c_rcp20.v[len];
+    for (int item = tid; item < 9 * len; item += APF::THREADS) {
+      const int m = (int)(((unsigned)item * rcp_len) >> 20);
+      const int pp = item - m * len;
+      const int p = pp + 5;
+      auto ldw = [&](int k, int w) { return df2_from4(Bw4[(m * 3 + k) * NW + w]); };
+      const df2 ab = df2_add_fast(df2_sub(ldw(0, p - 1), ldw(0, p)), df2_sub(ldw(1, p - 2), ldw(1, p - 1)));
+      df2 lin = df2_add_fast(df2_sub(ldw(2, p), ldw(2, p - 3)), df2_mul_f_u(df2_sub(ldw(2, p - 2), ldw(2, p - 1)), 3.0f));
+      if (m >= 5 || m == 1 + D) {
+        const float4* lh = LH4 + (m < 5 ? 0 : m - 4) * NI;
+        const df2 in = df2_add_fast(df2_from4(lh[p - 2]), df2_from4(lh[p - 3]));
+        const df2 ex = df2_add_fast(df2_from4(lh[p - 1]), df2_from4(lh[p - 4]));
+        lin = df2_add_fast(lin, df2_sub(df2_mul_f_u(in, 3.5f), df2_scale(ex, f2splat(0.5f))));
       }
-      gsm[m * TP * W + tile_idx<D, W>(pp, line, TP)] = f2d_bits(acc.hi) + f2d_bits(acc.lo);
+      df2 acc = df2_add_fast(df2_scale(ab, f2splat(4.0f)), df2_mul_u(lin, sixth));
+      if (m < 5)
+        acc = df2_add_fast(acc, df2_add_fast(df2_from4(RD4[(5 + m) * NI + p - 2]), df2_from4(RD4[(10 + m) * NI + p - 3])));
+      gsm[m * TP * W + tile_idx<D, W>(pp, 0, TP)] = f2d_bits(acc.hi.x) + f2d_bits(acc.lo.x);
+      gsm[m * TP * W + tile_idx<D, W>(pp, 1, TP)] = f2d_bits(acc.hi.y) + f2d_bits(acc.lo.y);
     }
   }
   __syncthreads();
   // F2: adjoint of the point fluxes, scale back, epilogue (one point per item)
-  for (int item = tid; item < TP * W; item += APF::THREADS) {
+  for (int item = tid; item < len * W; item += APF::THREADS) {
     int pp, line;
-    tile_split<D, W>(item, TP, pp, line);
-    if (s0 + pp >= nD || a0 + line >= na) continue;
+    item_split<D, W>(item, len, c_rcp20.v[len], pp, line);
+    if (a0 + line >= na) continue;
     const int pos = pp + 5;
     double gsum[9], cv[5];
 #pragma unroll
@@ -1552,10 +1586,12 @@ cudaError_t launch_adj_dir(int d, const AdjArgs& a, cudaStream_t s) {
   const int BXd = (d == 2) ? 1 : 2;
   if (a.mode == 1) {
     dim3 grid((a.g.n[d] + APF::TP - 1) / APF::TP, (a.g.n[AXd] + APF::W - 1) / APF::W, a.g.n[BXd]);
+    AdjArgs r = a;
+    tile_split_units(d, a.g.n[d], grid.x, r.tile_u, r.tile_r);
     switch (d) {
-      case 0: k_adj_dir_df<0><<<grid, APF::THREADS, APF::BYTES, s>>>(a); break;
-      case 1: k_adj_dir_df<1><<<grid, APF::THREADS, APF::BYTES, s>>>(a); break;
-      default: k_adj_dir_df<2><<<grid, APF::THREADS, APF::BYTES, s>>>(a); break;
+      case 0: k_adj_dir_df<0><<<grid, APF::THREADS, APF::BYTES, s>>>(r); break;
+      case 1: k_adj_dir_df<1><<<grid, APF::THREADS, APF::BYTES, s>>>(r); break;
+      default: k_adj_dir_df<2><<<grid, APF::THREADS, APF::BYTES, s>>>(r); break;
     }
     return cudaGetLastError();
   }

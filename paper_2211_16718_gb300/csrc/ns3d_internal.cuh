@@ -145,6 +145,7 @@ struct AdjArgs {
   double gamma, eps4, hdelta;
   int* status;
   int mode;           // 0: all FP64; 1: reconstruction adjoints in double-float (NS3D_FP64)
+  int tile_u, tile_r; // cut of the pencil into tiles (tile_split_units), filled in by the launch (mode 1)
 };
 
 constexpr int ADJ_SCRATCH_PLANES = 16;  // viscous-adjoint scratch: grad adjoint 12, velocity 3, rho 1
