@@ -594,10 +594,13 @@ __global__ void __launch_bounds__(APL::THREADS, 2) k_adj_dir(const AdjArgs a) {
 // The per-point sums are converted back to FP64 once.  To keep double-float values inside the float
 // range whatever the scale of the adjoint input, each tile divides the interface differences of
 // lambda by the power of two of lambda's largest magnitude and multiplies its results back (exact).
-// What bounds it: latency at 16 warps per SM (128 registers; 103 KB of shared memory).  355 warp
+// What bounds it: latency at 16 warps per SM (128 registers; 103 KB of shared memory).  365 warp
 // instructions per point where carrying every reconstruction to its points took 488: 128^3 pass
 // 2.15 / 2.24 / 2.13 -> 1.63 / 1.85 / 1.81 ms (x / y / z).  More warps with fewer registers lose: the
 // Roe adjoint's chain then spills 430 bytes (384 threads of 80 registers: 2.18 / 2.28 / 2.23 ms).
+// The Roe adjoint with pairs on the packed lanes (its phase 14.6k -> 7.9k cycles per tile), the flux
+// components' whole chain beside it, and the point-flux adjoint by component with its epilogue
+// operands prefetched (8.2k -> 4.1k cycles): 1.48 / 1.56 / 1.60 ms.
 // ============================================================================================
 template <int TP_, int THREADS_, int MIN_CTAS_>
 struct AdjPlanDF {
@@ -717,151 +720,205 @@ __device__ __forceinline__ df harten_df(df lam, df delta, df& dl, df& dd) {
 // Adjoint of the Roe flux at one interface in double-float arithmetic on the FP32 pipe: the
 // algebra of roe_adjoint (Sec. 2.2, Eq. Roe, wave strengths, Harten's fix, Roe average of the
 // grid-point states a = i, b = i+1), every quantity as a double-float (~48 bits) instead of
-// FP64.  du: the jump of the conserved reconstructions, Lh: the adjoint of the interface flux;
-// returns dub (adjoint of du) and ga, gb (adjoints of the two conserved point states).  Returns
-// 1 for a non-physical Roe state, 2 for values outside the float range of the double-float
-// arithmetic.
+// FP64.  One interface per thread; what comes in twos runs on the two lanes of the packed
+// operations (df2.cuh): the states (a, b), the tangential directions (T1, T2), the acoustic fields
+// (1, 5) and pairs of sums with a common factor.  The phase is one thread's chain of dependent
+// operations, so their number is its time (about 1.2k instead of 2.0k).
+// du: the jump of the conserved reconstructions, Lh: the adjoint of the interface flux; sr, Vab, Hab,
+// rho, e: sqrt(rho), velocity, H, rho, e of (a, b).  Returns dub (adjoint of du) and gab (adjoints of
+// the two conserved point states); 1 for a non-physical Roe state, 2 for values outside the float
+// range of the double-float arithmetic.
 template <int D>
-__device__ __forceinline__ int roe_adjoint_df(const df du[5], const df Lh[5], df ra, df rb, const df Va[3],
-                                              const df Vb[3], df Ha, df Hb, df rho_a, df e_a, df rho_b, df e_b,
-                                              df gamma, df gm1, df hdelta, df dub[5], df ga[5], df gb[5]) {
+__device__ __forceinline__ int roe_adjoint_df2(const df du[5], const df Lh[5], df2 sr, const df2 Vab[3], df2 Hab,
+                                               df2 rho, df2 e, df gamma, df gm1, df hdelta, df dub[5], df2 gab[5]) {
   constexpr int T1 = (D == 0) ? 1 : 0;
   constexpr int T2 = (D == 2) ? 1 : 2;
-  const df one{1.0f, 0.0f}, zero{0.0f, 0.0f};
-  const df rsum = df_add_pos(ra, rb);
-  const df rs = df_div(one, rsum);
-  const df wa = df_mul(ra, rs), wb = df_mul(rb, rs);
-  df V[3];
-#pragma unroll
-  for (int m = 0; m < 3; ++m) V[m] = df_add_fast(df_mul_u(wa, Va[m]), df_mul_u(wb, Vb[m]));
-  const df H = df_add_pos(df_mul_u(wa, Ha), df_mul_u(wb, Hb));
-  const df q2 = df_add_pos_u(df_sqr_u(V[0]), df_add_pos_u(df_sqr_u(V[1]), df_sqr_u(V[2])));
+  const df one{1.0f, 0.0f};
+  auto l0 = [](df2 x) { return df2_lane0(x); };
+  auto l1 = [](df2 x) { return df2_lane1(x); };
+  auto sp = [](df x) { return df2_splat(x); };
+  auto pk = [](df x, df y) { return df2_pack(x, y); };
+  auto fma2 = [](df2 x, df2 y, df2 z) { return df2_add_fast(df2_mul_u(x, y), z); };
+  auto half2 = [](df2 x) { return df2_scale(x, f2splat(0.5f)); };
+  const df rsum = df_add_pos(l0(sr), l1(sr));
+  const df rs = df_div_r(one, rsum);
+  const df2 w = df2_mul(sr, sp(rs));
+  const df2 xt1 = df2_mul_u(w, Vab[T1]), xt2 = df2_mul_u(w, Vab[T2]);
+  const df2 xn = df2_mul_u(w, Vab[D]), xh = df2_mul_u(w, Hab);
+  const df2 vt = df2_add_fast(pk(l0(xt1), l0(xt2)), pk(l1(xt1), l1(xt2)));  // (V_T1, V_T2)
+  const df2 uH = df2_add_fast(pk(l0(xn), l0(xh)), pk(l1(xn), l1(xh)));      // (V_D, H)
+  const df un = l0(uH), H = l1(uH);
+  const df2 vt_sq = df2_sqr_u(vt);
+  const df q2 = df_add_pos_u(df_sqr_u(un), df_add_pos_u(l0(vt_sq), l1(vt_sq)));
   const df q2h = fast_two_sum(0.5f * q2.hi, 0.5f * q2.lo);
   const df c2 = df_mul(df_sub(H, q2h), gm1);
   int flags = (c2.hi > 0.0f) ? 0 : 1;
-  flags |= (c2.hi > 1e-30f && c2.hi < 1e30f && rsum.hi > 1e-30f && rsum.hi < 1e30f && rho_a.hi > 1e-30f &&
-            rho_a.hi < 1e30f && rho_b.hi > 1e-30f && rho_b.hi < 1e30f && fabsf(H.hi) < 1e30f)
+  flags |= (c2.hi > 1e-30f && c2.hi < 1e30f && rsum.hi > 1e-30f && rsum.hi < 1e30f && rho.hi.x > 1e-30f &&
+            rho.hi.x < 1e30f && rho.hi.y > 1e-30f && rho.hi.y < 1e30f && fabsf(H.hi) < 1e30f)
                ? 0
                : 2;
-  const df c = df_sqrt(c2);
-  const df rc = df_div(one, c);
-  const df un = V[D], vt1 = V[T1], vt2 = V[T2];
+  const df c = df_sqrt_r(c2);
+  const df rc = df_div_r(one, c);
   const df rc2 = df_sqr(rc);
   const df b1 = df_mul(gm1, rc2);
-  const df vdm = df_add_fast(df_mul_u(V[0], du[1]), df_add_fast(df_mul_u(V[1], du[2]), df_mul_u(V[2], du[3])));
+  const df2 dut = pk(du[1 + T1], du[1 + T2]);
+  const df2 vd = df2_mul_u(vt, dut);
+  const df vdm = df_add_fast(df_mul_u(un, du[1 + D]), df_add_fast(l0(vd), l1(vd)));
   const df Y = df_sub(df_fma(q2h, du[0], du[4]), vdm);
   const df phi = df_mul(b1, Y);
   const df X = df_sub(df_mul_u(un, du[0]), du[1 + D]);
   const df ach = df_half(df_mul(X, rc));
   const df a2 = df_sub(du[0], phi);
-  const df a3 = df_sub(du[1 + T1], df_mul_u(vt1, du[0]));
-  const df a4 = df_sub(du[1 + T2], df_mul_u(vt2, du[0]));
-  const df phh = df_half(phi);
-  const df a1 = df_add_fast(phh, ach), a5 = df_sub(phh, ach);
+  const df2 a34 = df2_sub(dut, df2_mul_u(vt, sp(du[0])));
+  const df2 a15 = df2_add_fast(sp(df_half(phi)), pk(ach, df_neg(ach)));
   const df delta = df_mul(hdelta, c);
   df dl1, dd1, dl5, dd5;
-  const df l1 = harten_df(df_sub(un, c), delta, dl1, dd1);
-  const df l5 = harten_df(df_add_fast(un, c), delta, dl5, dd5);
+  const df2 lam15 = df2_add_fast(sp(un), pk(df_neg(c), c));
+  const df h1 = harten_df(l0(lam15), delta, dl1, dd1), h5 = harten_df(l1(lam15), delta, dl5, dd5);
+  const df2 l15 = pk(h1, h5);
   const df l2 = df_abs(un);
   const float sg2 = (un.hi > 0.0f) ? 1.0f : ((un.hi < 0.0f) ? -1.0f : 0.0f);
-  const df A1 = df_mul(l1, a1), A2 = df_mul(l2, a2), A3 = df_mul(l2, a3), A4 = df_mul(l2, a4), A5 = df_mul(l5, a5);
-  const df S = df_add_fast(A1, A5), d0 = df_add_fast(S, A2), cD = df_mul(c, df_sub(A5, A1));
+  const df2 A15 = df2_mul(l15, a15), A34 = df2_mul(sp(l2), a34);
+  const df A2 = df_mul(l2, a2);
+  const df S = df_add_fast(l0(A15), l1(A15)), dA = df_sub(l1(A15), l0(A15));
+  const df d0 = df_add_fast(S, A2), cD = df_mul(c, dA);
   // backward: the adjoint of the dissipation vector is -Lhat/2
   df Db[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) Db[v] = df{-0.5f * Lh[v].hi, -0.5f * Lh[v].lo};
-  const df d0b = df_fma(Db[1 + D], un, df_fma(Db[1 + T1], vt1, df_fma(Db[1 + T2], vt2, Db[0])));
+  const df2 Dbt = pk(Db[1 + T1], Db[1 + T2]), D4 = sp(Db[4]);
+  const df2 dv = df2_mul_u(Dbt, vt);
+  const df d0b = df_fma(Db[1 + D], un, df_add_fast(df_add_fast(l0(dv), l1(dv)), Db[0]));
   const df cDb = df_fma(Db[4], un, Db[1 + D]);
-  const df Sb = df_fma(Db[4], H, d0b);
-  const df A2b = df_fma(Db[4], q2h, d0b);
-  const df A3b = df_fma(Db[4], vt1, Db[1 + T1]);
-  const df A4b = df_fma(Db[4], vt2, Db[1 + T2]);
+  const df2 SA = fma2(D4, pk(H, q2h), sp(d0b));  // adjoints of S and A_2
+  const df Sb = l0(SA), A2b = l1(SA);
+  const df2 A34b = fma2(D4, vt, Dbt);
   const df ccDb = df_mul(c, cDb);
-  const df A1b = df_sub(Sb, ccDb), A5b = df_add_fast(Sb, ccDb);
+  const df2 A15b = df2_add_fast(sp(Sb), pk(df_neg(ccDb), ccDb));
   df unb = df_add_fast(df_mul_u(Db[1 + D], d0), df_mul_u(Db[4], cD));
-  df vt1b = df_add_fast(df_mul_u(Db[1 + T1], d0), df_mul_u(Db[4], A3));
-  df vt2b = df_add_fast(df_mul_u(Db[1 + T2], d0), df_mul_u(Db[4], A4));
-  df Hbar = df_mul(Db[4], S);
-  df q2hb = df_mul(Db[4], A2);
-  df cb = df_mul(cDb, df_sub(A5, A1));
+  df2 vtb = df2_add_fast(df2_mul_u(Dbt, sp(d0)), df2_mul_u(D4, A34));
+  df2 Hq = df2_mul(D4, pk(S, A2));  // adjoints of H and |V|^2/2
+  df cb = df_mul(cDb, dA);
   // A_k = l_k a_k
-  const df a1b = df_mul(A1b, l1), a2b = df_mul(A2b, l2), a3b = df_mul(A3b, l2), a4b = df_mul(A4b, l2);
-  const df a5b = df_mul(A5b, l5);
-  const df l1b = df_mul(A1b, a1), l5b = df_mul(A5b, a5);
-  const df l2b = df_fma(A2b, a2, df_fma(A3b, a3, df_mul_u(A4b, a4)));
-  const df t1 = df_mul_u(dl1, l1b), t5 = df_mul_u(dl5, l5b);
-  unb = df_add_fast(df_add_fast(t1, t5), df_add_fast(df{sg2 * l2b.hi, sg2 * l2b.lo}, unb));
-  cb = df_add_fast(df_add_fast(df_sub(t5, t1), df_mul_u(hdelta, df_fma(dd1, l1b, df_mul_u(dd5, l5b)))), cb);
+  const df2 a15b = df2_mul(A15b, l15), a34b = df2_mul(A34b, sp(l2)), l15b = df2_mul(A15b, a15);
+  const df a2b = df_mul(A2b, l2);
+  const df2 la = df2_mul_u(A34b, a34);
+  const df l2b = df_fma(A2b, a2, df_add_fast(l0(la), l1(la)));
+  const df2 t15 = df2_mul_u(pk(dl1, dl5), l15b);
+  const df2 tsd = df2_add_fast(sp(l1(t15)), pk(l0(t15), df_neg(l0(t15))));  // t5 +- t1
+  unb = df_add_fast(l0(tsd), df_add_fast(df{sg2 * l2b.hi, sg2 * l2b.lo}, unb));
+  cb = df_add_fast(l1(tsd), cb);
+  if (dd1.hi != 0.0f || dd5.hi != 0.0f)  // Harten's branch: the width depends on c
+    cb = df_add_fast(df_mul_u(hdelta, df_fma(dd1, l0(l15b), df_mul_u(dd5, l1(l15b)))), cb);
   // wave strengths
-  const df phib = df_sub(df_half(df_add_fast(a1b, a5b)), a2b);
-  const df achb = df_sub(a1b, a5b);
-  dub[0] = df_sub(a2b, df_add_fast(df_mul_u(vt1, a3b), df_mul_u(vt2, a4b)));
-  dub[1 + T1] = a3b;
-  dub[1 + T2] = a4b;
-  vt1b = df_sub(vt1b, df_mul_u(a3b, du[0]));
-  vt2b = df_sub(vt2b, df_mul_u(a4b, du[0]));
-  const df Xb = df_half(df_mul(rc, achb));
-  df rcb = df_half(df_mul(X, achb));
-  unb = df_fma(Xb, du[0], unb);
-  dub[0] = df_fma(Xb, un, dub[0]);
-  dub[1 + D] = df_neg(Xb);
-  const df b1b = df_mul(phib, Y);
-  const df Yb = df_mul(phib, b1);
-  q2hb = df_fma(Yb, du[0], q2hb);
-  dub[0] = df_fma(Yb, q2h, dub[0]);
-  dub[4] = Yb;
-  df Vbar[3];
-  Vbar[D] = unb;
-  Vbar[T1] = vt1b;
-  Vbar[T2] = vt2b;
-#pragma unroll
-  for (int m = 0; m < 3; ++m) {
-    Vbar[m] = df_sub(Vbar[m], df_mul_u(Yb, du[1 + m]));  // vdm = V . du_m
-    dub[1 + m] = df_sub(dub[1 + m], df_mul_u(Yb, V[m]));
-  }
-  rcb = df_fma(b1b, df_twice(df_mul(gm1, rc)), rcb);
+  const df2 psd = df2_add_fast(sp(l0(a15b)), pk(l1(a15b), df_neg(l1(a15b))));  // a1b +- a5b
+  const df phib = df_sub(df_half(l0(psd)), a2b);
+  const df achb = l1(psd);
+  const df2 va = df2_mul_u(vt, a34b);
+  df dub0 = df_sub(a2b, df_add_fast(l0(va), l1(va)));
+  vtb = df2_sub(vtb, df2_mul_u(a34b, sp(du[0])));
+  const df2 XR = half2(df2_mul(pk(rc, X), sp(achb)));  // adjoints of X and (through X rc / 2) of rc
+  const df Xb = l0(XR);
+  df rcb = l1(XR);
+  const df2 ud = fma2(sp(Xb), pk(du[0], un), pk(unb, dub0));
+  const df2 bY = df2_mul(sp(phib), pk(Y, b1));  // adjoints of b1 and Y
+  const df2 Yb = sp(l1(bY));
+  const df2 qd = fma2(Yb, pk(du[0], q2h), pk(l1(Hq), l1(ud)));
+  dub[0] = l1(qd);
+  dub[4] = l1(bY);
+  const df2 nD = df2_sub(pk(l0(ud), df_neg(Xb)), df2_mul_u(Yb, pk(du[1 + D], un)));  // vdm = V . du_m
+  dub[1 + D] = l1(nD);
+  vtb = df2_sub(vtb, df2_mul_u(Yb, dut));
+  const df2 dT = df2_sub(a34b, df2_mul_u(Yb, vt));
+  dub[1 + T1] = l0(dT);
+  dub[1 + T2] = l1(dT);
+  rcb = df_fma(l0(bY), df_twice(df_mul(gm1, rc)), rcb);
   cb = df_sub(cb, df_mul_u(rcb, rc2));
   // c = sqrt(gm1 (H - q2h))
-  const df c2b = df_half(df_mul(cb, rc));
-  Hbar = df_fma(gm1, c2b, Hbar);
-  q2hb = df_sub(q2hb, df_mul_u(gm1, c2b));
+  const df gc = df_mul_u(gm1, df_half(df_mul(cb, rc)));
+  Hq = df2_add_fast(pk(l0(Hq), l0(qd)), pk(gc, df_neg(gc)));
+  const df Hbar = l0(Hq), q2hb = l1(Hq);
+  vtb = fma2(sp(q2hb), vt, vtb);
+  df2 Vbar[3];
+  Vbar[T1] = sp(l0(vtb));
+  Vbar[T2] = sp(l1(vtb));
+  Vbar[D] = sp(df_fma(q2hb, un, l0(nD)));
+  const df2 Vroe[3] = {sp(D == 0 ? un : l0(vt)), sp(D == 1 ? un : (D == 0 ? l0(vt) : l1(vt))), sp(D == 2 ? un : l1(vt))};
+  // Roe average of the point states, (a, b) on the lanes
+  df2 rr = df2_mul_u(sp(Hbar), df2_sub(Hab, sp(H)));
 #pragma unroll
-  for (int m = 0; m < 3; ++m) Vbar[m] = df_fma(q2hb, V[m], Vbar[m]);
-  // Roe average of the point states a, b
-  df rab = df_mul_u(Hbar, df_sub(Ha, H)), rbb = df_mul_u(Hbar, df_sub(Hb, H));
+  for (int m = 0; m < 3; ++m) rr = fma2(Vbar[m], df2_sub(Vab[m], Vroe[m]), rr);
+  rr = df2_mul(rr, sp(rs));
+  // point primitives: V = m/rho, H = gamma e/rho - gm1 |V|^2/2, sqrt(rho)
+  const df2 ri = df2_div(df2_splat(one), rho);
+  const df2 Hb = df2_mul(w, sp(Hbar));
+  const df2 gH = df2_mul(Hb, sp(gm1)), Hg = df2_mul(Hb, sp(gamma));
+  df2 vdot = df2_mul_u(Hg, df2_mul(e, ri));
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
-    rab = df_fma(Vbar[m], df_sub(Va[m], V[m]), rab);
-    rbb = df_fma(Vbar[m], df_sub(Vb[m], V[m]), rbb);
+    const df2 Vt = df2_sub(df2_mul_u(w, Vbar[m]), df2_mul_u(gH, Vab[m]));
+    vdot = fma2(Vt, Vab[m], vdot);
+    gab[1 + m] = df2_mul(Vt, ri);
   }
-  rab = df_mul(rab, rs);
-  rbb = df_mul(rbb, rs);
-  // point primitives: V = m/rho, H = gamma e/rho - gm1 |V|^2/2, sqrt(rho)
-#pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    const df wgt = side ? wb : wa;
-    const df* Vp = side ? Vb : Va;
-    const df rho = side ? rho_b : rho_a, e = side ? e_b : e_a, sr = side ? rb : ra;
-    const df rr = df_div(one, rho);
-    const df Hb_ = df_mul(wgt, Hbar);
-    const df gH = df_mul(Hb_, gm1);
-    const df srb = side ? rbb : rab;
-    df Vt[3], vdot = zero;
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {
-      Vt[m] = df_sub(df_mul_u(wgt, Vbar[m]), df_mul_u(gH, Vp[m]));
-      vdot = df_fma(Vt[m], Vp[m], vdot);
-    }
-    df* gs = side ? gb : ga;
-    const df Hg = df_mul(Hb_, gamma);
-    gs[4] = df_mul(Hg, rr);
-    // d sqrt(rho)/d rho = 1/(2 sqrt(rho)) = sqrt(rho) / (2 rho)
-    gs[0] = df_sub(df_mul_u(df_half(srb), df_mul(sr, rr)), df_mul_u(df_fma(Hg, df_mul(e, rr), vdot), rr));
-#pragma unroll
-    for (int m = 0; m < 3; ++m) gs[1 + m] = df_mul(Vt[m], rr);
-  }
+  gab[4] = df2_mul(Hg, ri);
+  // d sqrt(rho)/d rho = 1/(2 sqrt(rho)) = sqrt(rho) / (2 rho)
+  gab[0] = df2_sub(df2_mul_u(half2(rr), df2_mul(sr, ri)), df2_mul_u(vdot, ri));
   return flags;
 }
+
+// Operands of the adjoint epilogue besides k: how many, and their planes.
+__device__ __forceinline__ int adj_epilogue_operands(const AdjArgs& a, const double*& o1, const double*& o2) {
+  o1 = o2 = nullptr;
+  switch (a.epi) {
+    case AEPI_RK4_4:
+    case AEPI_SSP_3: o1 = a.ubs; return 1;
+    case AEPI_RK4_M: o1 = a.ubs; o2 = a.gout; return 2;
+    case AEPI_ACC: o1 = a.gout; return 1;
+    case AEPI_SSP_2: o1 = a.sb; o2 = a.gout; return 2;
+    default: return 0;
+  }
+}
+
+// adj_epilogue of component v at index i = v N + p, its operands fetched: kp = k, x1, x2 as
+// adj_epilogue_operands orders them; the same arithmetic.
+__device__ __forceinline__ void adj_epilogue_pre(const AdjArgs& a, long long i, double cv, double kp, double x1,
+                                                 double x2) {
+  switch (a.epi) {
+    case AEPI_WRITE: a.k[i] = cv; break;
+    case AEPI_ADD: a.k[i] = kp + cv; break;
+    case AEPI_OUT: a.gout[i] = kp + cv; break;
+    case AEPI_RK4_4: {
+      const double K = kp + cv;
+      a.gout[i] = x1 + K;
+      a.lnext[i] = fma(a.c1, x1, a.c2 * K);
+      break;
+    }
+    case AEPI_RK4_M: {
+      const double K = kp + cv;
+      a.gout[i] = x2 + K;
+      a.lnext[i] = fma(a.c1, x1, a.c2 * K);
+      break;
+    }
+    case AEPI_ACC: a.gout[i] = x1 + (kp + cv); break;
+    case AEPI_SSP_3: {
+      const double s = fma(2.0 / 3.0, x1, kp + cv);
+      a.gout[i] = fma(1.0 / 3.0, x1, 0.75 * s);
+      a.lnext[i] = (0.25 * a.c2) * s;
+      a.sb[i] = 0.25 * s;
+      break;
+    }
+    case AEPI_SSP_2: {
+      const double s = x1 + (kp + cv);
+      a.gout[i] = x2 + s;
+      a.lnext[i] = a.c2 * s;
+      break;
+    }
+    default: break;
+  }
+}
+
+// Barrier of the n threads (whole warps) that use barrier `id`.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 template <int D>
 __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(const AdjArgs a) {
@@ -966,6 +1023,22 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
   }
   __syncthreads();
 
+  // epilogue operands: asynchronously, k into the dead lambda now, the others after phase E2
+  static_assert(5 * TP * W <= 5 * NP * W && 10 * TP * W <= 81 * NI * W, "epilogue operands fit");
+  double* pre_k = sm + APF::OFF_L;   // [5][TP*W]
+  double* pre_x = sm + APF::OFF_WC;  // [10][TP*W]
+  auto fetch = [&](double* dst, const double* src) {
+    for (int item = tid; item < 5 * len * W; item += APF::THREADS) {
+      const int v = (int)(((unsigned)(item / W) * c_rcp20.v[len]) >> 20);
+      const int pt = item - v * (len * W);
+      int pp, line;
+      item_split<D, W>(pt, len, c_rcp20.v[len], pp, line);
+      if (a0 + line < na) cp_async8(dst + v * TP * W + pt, src + v * N + tile_flat<D>(a.g, s0 + pp, a0 + line, bz));
+    }
+  };
+  if (a.epi != AEPI_WRITE) fetch(pre_k, a.k);
+  cp_async_commit();
+
   // ---- B: window terms b_k of every window, stored as 1/b_k, and T/6 (both lines at once) ---------
   {
     const df2 eps4 = df2_splat(df{(float)a.eps4, (float)(a.eps4 - (double)(float)a.eps4)});
@@ -1064,8 +1137,57 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
     wm[8 * NI] = df2_to4(ta);
   };
 
-  // ---- D: adjoint of the Roe flux, in double-float, on the first warps; the flux components'
-  //      reconstruction adjoints on the others
+  // ---- E2 (one scalar and window 2 .. len+4, both lines): the window's adjoint sums -> a quarter of the
+  //      adjoints A, B of its two first differences (slots 0, 1) and the adjoint of T/6 (slot 2), into the
+  //      dead reciprocals.  With k_j half the adjoint of b_j and K their sum,
+  //      A/4 = -(13/3) s K - v_0 k_0 + v_1 k_1 - 3 v_2 k_2,  B/4 = (13/3) s K + 3 v_0 k_0 + v_1 k_1 + v_2 k_2
+  auto window = [&](int m, int w) {
+    const float4* wm = wc4 + m * 9 * NI;
+    auto ldw = [&](int k, int f) { return df2_from4(wm[k * NI + f]); };
+    Bw4[(m * 3 + 2) * NW + w] = df2_to4(df2_add_fast(df2_add_fast(ldw(6, w), ldw(7, w - 1)), ldw(8, w - 2)));
+    if (w < 3) return;  // only its T is used
+    const df2 k0 = df2_add_fast(ldw(0, w), ldw(5, w - 1));
+    const df2 k1 = df2_add_fast(ldw(1, w - 1), ldw(4, w - 2));
+    const df2 k2 = df2_add_fast(ldw(2, w - 2), ldw(3, w - 3));
+    const df2 g0 = df2_from4(G4[m * NP + w]), g1 = df2_from4(G4[m * NP + w + 1]);
+    const df2 ps = df2_mul_u(df2_mul_u(df2_sub(g1, g0), df2_add_fast(k0, df2_add_fast(k1, k2))), c133);
+    const df2 p0 = df2_mul_u(df2_sub(df2_mul_f_u(g1, 3.0f), g0), k0);
+    const df2 p1 = df2_mul_u(df2_add_fast(g0, g1), k1);
+    const df2 p2 = df2_mul_u(df2_sub(g1, df2_mul_f_u(g0, 3.0f)), k2);
+    Bw4[(m * 3 + 0) * NW + w] = df2_to4(df2_sub(df2_sub(p1, ps), df2_add_fast(p0, df2_mul_f_u(p2, 3.0f))));
+    Bw4[(m * 3 + 1) * NW + w] = df2_to4(df2_add_fast(df2_add_fast(p1, ps), df2_add_fast(p2, df2_mul_f_u(p0, 3.0f))));
+  };
+  // ---- F1: the gather, one scalar and point of both lines per item:
+  //   (A_{p-1} - A_p) + (B_{p-2} - B_{p-1}) + [T_p - T_{p-3} + 3 (T_{p-2} - T_{p-1})]/6
+  //   + [7 (h_{p-2} + h_{p-3}) - (h_{p-1} + h_{p-4})]/6 (flux components), h half the interface adjoint
+  //   + the Roe-average adjoints of the point's two interfaces (conserved variables)
+  // into the dead first differences (conserved variables) and point fluxes (flux components)
+  static_assert(5 * TP * W <= 9 * NP * W && 4 * TP * W <= 4 * NP * W, "gathered sums fit");
+  double* gsm_u = sm + APF::OFF_G;                // [5][TP*W]
+  double* gsm_f = sm + APF::OFF_Q + 5 * NP * W;   // [4][TP*W]
+  auto gather = [&](int m, int pp) {
+    const int p = pp + 5;
+    auto ldw = [&](int k, int w) { return df2_from4(Bw4[(m * 3 + k) * NW + w]); };
+    const df2 ab = df2_add_fast(df2_sub(ldw(0, p - 1), ldw(0, p)), df2_sub(ldw(1, p - 2), ldw(1, p - 1)));
+    df2 lin = df2_add_fast(df2_sub(ldw(2, p), ldw(2, p - 3)), df2_mul_f_u(df2_sub(ldw(2, p - 2), ldw(2, p - 1)), 3.0f));
+    if (m >= 5 || m == 1 + D) {
+      const float4* lh = LH4 + (m < 5 ? 0 : m - 4) * NI;
+      const df2 in = df2_add_fast(df2_from4(lh[p - 2]), df2_from4(lh[p - 3]));
+      const df2 ex = df2_add_fast(df2_from4(lh[p - 1]), df2_from4(lh[p - 4]));
+      lin = df2_add_fast(lin, df2_sub(df2_mul_f_u(in, 3.5f), df2_scale(ex, f2splat(0.5f))));
+    }
+    df2 acc = df2_add_fast(df2_scale(ab, f2splat(4.0f)), df2_mul_u(lin, sixth));
+    if (m < 5)
+      acc = df2_add_fast(acc, df2_add_fast(df2_from4(RD4[(5 + m) * NI + p - 2]), df2_from4(RD4[(10 + m) * NI + p - 3])));
+    double* g = (m < 5) ? gsm_u + m * TP * W : gsm_f + (m - 5) * TP * W;
+    g[tile_idx<D, W>(pp, 0, TP)] = f2d_bits(acc.hi.x) + f2d_bits(acc.lo.x);
+    g[tile_idx<D, W>(pp, 1, TP)] = f2d_bits(acc.hi.y) + f2d_bits(acc.lo.y);
+  };
+  const int nv = len + 3;
+  const unsigned rcp_nv = c_rcp20.v[nv], rcp_len = c_rcp20.v[len];
+
+  // ---- D: adjoint of the Roe flux, in double-float, on the first warps; the flux components' adjoints,
+  //      which do not need it, through E1, E2 and F1 on the others (a barrier of their own)
   if (tid < APF::D_THREADS) {
     int bad = 0;
     if (tid < ni * W) {
@@ -1074,154 +1196,120 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
       int f, line;
       item_split<D, W>(tid, ni, rcp_ni, f, line);
       const int sa = tile_idx<D, W>(f + 2, line, NP), sb = tile_idx<D, W>(f + 3, line, NP);
-      df du[5], Lh[5], Va[3], Vb[3];
+      auto ab = [&](int k) { return df2_pack(df_unpack(rf[k * NP * W + sa]), df_unpack(rf[k * NP * W + sb])); };
+      df du[5], Lh[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         du[v] = rec_lane(J4 + v * NI + f, line);
         Lh[v] = rec_lane(LH4 + v * NI + f, line);
       }
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        Va[m] = df_unpack(rf[(1 + m) * NP * W + sa]);
-        Vb[m] = df_unpack(rf[(1 + m) * NP * W + sb]);
-      }
-      df dub[5], ga[5], gb[5];
-      bad = roe_adjoint_df<D>(du, Lh, df_unpack(rf[sa]), df_unpack(rf[sb]), Va, Vb, df_unpack(rf[4 * NP * W + sa]),
-                              df_unpack(rf[4 * NP * W + sb]), df_unpack(rf[6 * NP * W + sa]),
-                              df_unpack(rf[7 * NP * W + sa]), df_unpack(rf[6 * NP * W + sb]),
-                              df_unpack(rf[7 * NP * W + sb]), gam, gm1, hd, dub, ga, gb);
+      const df2 Vab[3] = {ab(1), ab(2), ab(3)};
+      df dub[5];
+      df2 gab[5];
+      bad = roe_adjoint_df2<D>(du, Lh, ab(0), Vab, ab(4), ab(6), ab(7), gam, gm1, hd, dub, gab);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         set_rec_lane(RD4 + v * NI + f, line, dub[v]);
-        set_rec_lane(RD4 + (5 + v) * NI + f, line, ga[v]);
-        set_rec_lane(RD4 + (10 + v) * NI + f, line, gb[v]);
+        set_rec_lane(RD4 + (5 + v) * NI + f, line, df2_lane0(gab[v]));
+        set_rec_lane(RD4 + (10 + v) * NI + f, line, df2_lane1(gab[v]));
       }
     }
     if (__any_sync(0xffffffffu, bad & 1) && (tid & 31) == 0) atomicOr(a.status, ST_NONPHYS);
     range_bad |= bad & 2;
   } else {
-    for (int item = tid - APF::D_THREADS; item < 4 * ni; item += APF::THREADS - APF::D_THREADS) {
+    constexpr int NT = APF::THREADS - APF::D_THREADS;
+    for (int item = tid - APF::D_THREADS; item < 4 * ni; item += NT) {
       const int m = (int)(((unsigned)item * rcp_ni) >> 20);
       recon(5 + m, item - m * ni);
+    }
+    bar_sync(1, NT);
+    for (int item = tid - APF::D_THREADS; item < 4 * nv; item += NT) {
+      const int m = (int)(((unsigned)item * rcp_nv) >> 20);
+      window(5 + m, 2 + item - m * nv);
+    }
+    bar_sync(1, NT);
+    for (int item = tid - APF::D_THREADS; item < 4 * len; item += NT) {
+      const int m = (int)(((unsigned)item * rcp_len) >> 20);
+      gather(5 + m, item - m * len);
     }
   }
   __syncthreads();
 
-  // ---- E1 of the conserved variables
+  // ---- the conserved variables
   for (int item = tid; item < 5 * ni; item += APF::THREADS) {
     const int m = (int)(((unsigned)item * rcp_ni) >> 20);
     recon(m, item - m * ni);
   }
   if (__any_sync(0xffffffffu, range_bad) && (tid & 31) == 0) atomicOr(a.status, ST_DF_RANGE);
   __syncthreads();
-
-  // ---- E2 (one scalar and window 2 .. len+4, both lines): the window's adjoint sums -> a quarter of the
-  //      adjoints A, B of its two first differences (slots 0, 1) and the adjoint of T/6 (slot 2), into the
-  //      dead reciprocals.  With k_j half the adjoint of b_j and K their sum,
-  //      A/4 = -(13/3) s K - v_0 k_0 + v_1 k_1 - 3 v_2 k_2,  B/4 = (13/3) s K + 3 v_0 k_0 + v_1 k_1 + v_2 k_2
-  {
-    const int nv = len + 3;
-    const unsigned rcp_nv = c_rcp20.v[nv];
-    for (int item = tid; item < 9 * nv; item += APF::THREADS) {
-      const int m = (int)(((unsigned)item * rcp_nv) >> 20);
-      const int w = 2 + item - m * nv;
-      const float4* wm = wc4 + m * 9 * NI;
-      auto ldw = [&](int k, int f) { return df2_from4(wm[k * NI + f]); };
-      Bw4[(m * 3 + 2) * NW + w] = df2_to4(df2_add_fast(df2_add_fast(ldw(6, w), ldw(7, w - 1)), ldw(8, w - 2)));
-      if (w < 3) continue;  // only its T is used
-      const df2 k0 = df2_add_fast(ldw(0, w), ldw(5, w - 1));
-      const df2 k1 = df2_add_fast(ldw(1, w - 1), ldw(4, w - 2));
-      const df2 k2 = df2_add_fast(ldw(2, w - 2), ldw(3, w - 3));
-      const df2 g0 = df2_from4(G4[m * NP + w]), g1 = df2_from4(G4[m * NP + w + 1]);
-      const df2 ps = df2_mul_u(df2_mul_u(df2_sub(g1, g0), df2_add_fast(k0, df2_add_fast(k1, k2))), c133);
-      const df2 p0 = df2_mul_u(df2_sub(df2_mul_f_u(g1, 3.0f), g0), k0);
-      const df2 p1 = df2_mul_u(df2_add_fast(g0, g1), k1);
-      const df2 p2 = df2_mul_u(df2_sub(g1, df2_mul_f_u(g0, 3.0f)), k2);
-      Bw4[(m * 3 + 0) * NW + w] = df2_to4(df2_sub(df2_sub(p1, ps), df2_add_fast(p0, df2_mul_f_u(p2, 3.0f))));
-      Bw4[(m * 3 + 1) * NW + w] = df2_to4(df2_add_fast(df2_add_fast(p1, ps), df2_add_fast(p2, df2_mul_f_u(p0, 3.0f))));
-    }
+  for (int item = tid; item < 5 * nv; item += APF::THREADS) {
+    const int m = (int)(((unsigned)item * rcp_nv) >> 20);
+    window(m, 2 + item - m * nv);
   }
   __syncthreads();
+  const double *x1 = nullptr, *x2 = nullptr;
+  const int nx = adj_epilogue_operands(a, x1, x2);
+  if (nx >= 1) fetch(pre_x, x1);
+  if (nx == 2) fetch(pre_x + 5 * TP * W, x2);
+  cp_async_commit();
+  for (int item = tid; item < 5 * len; item += APF::THREADS) {
+    const int m = (int)(((unsigned)item * rcp_len) >> 20);
+    gather(m, item - m * len);
+  }
+  cp_async_wait_all();
+  __syncthreads();
 
-  // ---- F: gather, adjoint of the point fluxes, scale back, epilogue ----------------------------
+  // ---- F2: adjoint of the point fluxes, scale back, epilogue; one component of one point per item, the
+  //      two long ones (0 and 1 + D) first, so that the FP64 work is spread over all warps
   const double up = pow2d(E);
   const double gm1 = a.gamma - 1.0;
-  // F1: the gather, one scalar and point of both lines per item, into the dead first differences:
-  //   (A_{p-1} - A_p) + (B_{p-2} - B_{p-1}) + [T_p - T_{p-3} + 3 (T_{p-2} - T_{p-1})]/6
-  //   + [7 (h_{p-2} + h_{p-3}) - (h_{p-1} + h_{p-4})]/6 (flux components), h half the interface adjoint
-  //   + the Roe-average adjoints of the point's two interfaces (conserved variables)
-  static_assert(TP * W <= NP * W, "gathered sums fit the space of the first differences");
-  double* gsm = sm + APF::OFF_G;  // [9][TP*W]
-  {
-    const unsigned rcp_len = c_rcp20.v[len];
-    for (int item = tid; item < 9 * len; item += APF::THREADS) {
-      const int m = (int)(((unsigned)item * rcp_len) >> 20);
-      const int pp = item - m * len;
-      const int p = pp + 5;
-      auto ldw = [&](int k, int w) { return df2_from4(Bw4[(m * 3 + k) * NW + w]); };
-      const df2 ab = df2_add_fast(df2_sub(ldw(0, p - 1), ldw(0, p)), df2_sub(ldw(1, p - 2), ldw(1, p - 1)));
-      df2 lin = df2_add_fast(df2_sub(ldw(2, p), ldw(2, p - 3)), df2_mul_f_u(df2_sub(ldw(2, p - 2), ldw(2, p - 1)), 3.0f));
-      if (m >= 5 || m == 1 + D) {
-        const float4* lh = LH4 + (m < 5 ? 0 : m - 4) * NI;
-        const df2 in = df2_add_fast(df2_from4(lh[p - 2]), df2_from4(lh[p - 3]));
-        const df2 ex = df2_add_fast(df2_from4(lh[p - 1]), df2_from4(lh[p - 4]));
-        lin = df2_add_fast(lin, df2_sub(df2_mul_f_u(in, 3.5f), df2_scale(ex, f2splat(0.5f))));
-      }
-      df2 acc = df2_add_fast(df2_scale(ab, f2splat(4.0f)), df2_mul_u(lin, sixth));
-      if (m < 5)
-        acc = df2_add_fast(acc, df2_add_fast(df2_from4(RD4[(5 + m) * NI + p - 2]), df2_from4(RD4[(10 + m) * NI + p - 3])));
-      gsm[m * TP * W + tile_idx<D, W>(pp, 0, TP)] = f2d_bits(acc.hi.x) + f2d_bits(acc.lo.x);
-      gsm[m * TP * W + tile_idx<D, W>(pp, 1, TP)] = f2d_bits(acc.hi.y) + f2d_bits(acc.lo.y);
-    }
-  }
-  __syncthreads();
-  // F2: adjoint of the point fluxes, scale back, epilogue (one point per item)
-  for (int item = tid; item < len * W; item += APF::THREADS) {
+  const int nl = len * W;
+#pragma unroll 1
+  for (int round = 0; round < 2; ++round) {
+    // the second round (component T2) goes to warps that had a short component in the first
+    const int item = round == 0 ? tid : APF::THREADS + (tid ^ (APF::THREADS / 2));
+    if (item >= 5 * nl) continue;
+    const int part = (int)(((unsigned)(item / W) * rcp_len) >> 20);
+    const int pt = item - part * nl;
     int pp, line;
-    item_split<D, W>(item, len, c_rcp20.v[len], pp, line);
+    item_split<D, W>(pt, len, rcp_len, pp, line);
     if (a0 + line >= na) continue;
-    const int pos = pp + 5;
-    double gsum[9], cv[5];
-#pragma unroll
-    for (int m = 0; m < 9; ++m) gsum[m] = gsm[m * TP * W + tile_idx<D, W>(pp, line, TP)];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) cv[v] = gsum[v];
-    const int s = tile_idx<D, W>(pos, line, NP);
-    const double rho = q[s], e = q[4 * NP * W + s], pr = ri[5 * NP * W + s];
+    constexpr int T1 = (D == 0) ? 1 : 0, T2 = (D == 2) ? 1 : 2;
+    const int v = (part == 0) ? 0 : (part == 1) ? 1 + D : (part == 2) ? 4 : (part == 3) ? 1 + T1 : 1 + T2;
+    const int s = tile_idx<D, W>(pp + 5, line, NP), gi = tile_idx<D, W>(pp, line, TP);
     const float2* rfs = reinterpret_cast<const float2*>(ri) + s;
-    double V[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    auto vel = [&](int k) {
       const float2 vk = rfs[(1 + k) * NP * W];
-      V[k] = f2d_bits(vk.x) + f2d_bits(vk.y);
-    }
-    const double un = V[D];
-    const double Fbm[3] = {gsum[5], gsum[6], gsum[7]};
-    const double Fb4 = gsum[8];
-    const double pb = fma(Fb4, un, Fbm[D]);
-    double unb = Fb4 * (e + pr);
+      return f2d_bits(vk.x) + f2d_bits(vk.y);
+    };
+    auto Fb = [&](int k) { return gsm_f[k * TP * W + gi]; };  // adjoint of f_{1+k}
+    const double un = vel(D), Fb4 = Fb(3);
+    const double gp = gm1 * fma(Fb4, un, Fb(D));
+    double cv = gsm_u[v * TP * W + gi];
+    if (part >= 3) {
+      cv = fma(-gp, vel(v - 1), fma(Fb(v - 1), un, cv));
+    } else if (part == 2) {
+      cv = fma(Fb4, un, cv) + gp;
+    } else {
+      const double rho = q[s], e = q[4 * NP * W + s], pr = ri[5 * NP * W + s];
+      double unb = Fb4 * (e + pr);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      unb = fma(Fbm[k], q[(1 + k) * NP * W + s], unb);
-      cv[1 + k] = fma(Fbm[k], un, cv[1 + k]);
-    }
-    cv[4] = fma(Fb4, un, cv[4]);
-    const double rr = rcp_newton(rho);
-    cv[1 + D] = fma(unb, rr, cv[1 + D]);
-    cv[0] = fma(-unb * un, rr, cv[0]);
-    const double gp = gm1 * pb;
-    cv[4] += gp;
-    double v2 = 0.0;
+      for (int k = 0; k < 3; ++k) unb = fma(Fb(k), q[(1 + k) * NP * W + s], unb);
+      const double rr = rcp_newton(rho);
+      if (part == 1) {
+        cv = fma(-gp, un, fma(unb, rr, fma(Fb(D), un, cv)));
+      } else {
+        double v2 = 0.0;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      cv[1 + k] = fma(-gp, V[k], cv[1 + k]);
-      v2 = fma(V[k], V[k], v2);
+        for (int k = 0; k < 3; ++k) {
+          const double V = (k == D) ? un : vel(k);
+          v2 = fma(V, V, v2);
+        }
+        cv = fma(0.5 * gp, v2, fma(-unb * un, rr, cv));
+      }
     }
-    cv[0] = fma(0.5 * gp, v2, cv[0]);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) cv[v] *= up;
     const long long p = tile_flat<D>(a.g, s0 + pp, a0 + line, bz);
-    adj_epilogue(a, p, cv);
+    adj_epilogue_pre(a, v * N + p, cv * up, pre_k[v * TP * W + pt], pre_x[v * TP * W + pt], pre_x[(5 + v) * TP * W + pt]);
   }
 }
 

@@ -114,3 +114,19 @@ def test_step_of_a_state_on_8_byte_boundaries(ns3d, nx):
     s.check()
     s.close()
     assert torch.equal(u, v)
+
+
+# one tile, one point over one and two tiles, x lengths that are no multiple of 4, one-point lines;
+# against the all-FP64 adjoint kernels, which have their own tiles and algebra (both pinned to the
+# oracle's dense adjoint elsewhere): the tolerance of that comparison
+@pytest.mark.parametrize("nx,ny,nz", [(32, 33, 5), (65, 3, 31), (2, 66, 35), (39, 7, 64), (1, 9, 34)])
+def test_adjoint_tiles(ns3d, nx, ny, nz):
+    u = _gpu(I.random_smooth(nx, ny, nz, seed=9, amp=0.1, mach=0.5))
+    lam = _gpu(np.random.default_rng(5).normal(size=(5, nz, ny, nx)))
+    out = []
+    for prec in (0, 2):
+        s = ns3d.Solver(nx, ny, nz, mu_eff=0.003, precision=prec)
+        out.append(s.rhs_vjp(u, lam).cpu().numpy())
+        s.check()
+        s.close()
+    assert rel_err(out[0], out[1]) <= 1e-11
