@@ -952,7 +952,8 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
   if (tid == 0) s_emax = -2000;
   __syncthreads();
 
-  // ---- A: load; largest binary exponent of lambda in the tile ----------------------------
+  // ---- A: load; largest binary exponent of lambda in the tile (one point per thread: three items per
+  //      point, over the whole CTA, took 1.49 / 1.61 / 1.63 ms per pass against 1.46 / 1.55 / 1.59)
   int emax = -2000;
   for (int item = tid; item < np * W; item += APF::THREADS) {
     int pos, line;
@@ -966,6 +967,7 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
     for (int v = 0; v < 5; ++v) U[v] = __ldg(a.u + v * N + p);
     const double vx = __ldg(a.pm + PM_U * N + p), vy = __ldg(a.pm + PM_V * N + p), vz = __ldg(a.pm + PM_W * N + p);
     const double pr = __ldg(a.pm + PM_P * N + p);
+    const df sr = load_df(a.pm + PM_SR * N + p), H = load_df(a.pm + PM_H * N + p);
     const double un = (D == 0) ? vx : (D == 1) ? vy : vz;
     const int s = tile_idx<D, W>(pos, line, NP);
 #pragma unroll
@@ -975,27 +977,28 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
     q[7 * NP * W + s] = (D == 2) ? fma(U[3], un, pr) : U[3] * un;
     q[8 * NP * W + s] = (U[4] + pr) * un;
     float2* rf = reinterpret_cast<float2*>(ri);
-    rf[0 * NP * W + s] = df_pack(d2df_bits(__ldg(a.pm + PM_SR * N + p)));
+    rf[0 * NP * W + s] = df_pack(sr);
     rf[1 * NP * W + s] = df_pack(d2df_bits(vx));
     rf[2 * NP * W + s] = df_pack(d2df_bits(vy));
     rf[3 * NP * W + s] = df_pack(d2df_bits(vz));
-    rf[4 * NP * W + s] = df_pack(d2df_bits(__ldg(a.pm + PM_H * N + p)));
+    rf[4 * NP * W + s] = df_pack(H);
     ri[5 * NP * W + s] = pr;
     rf[6 * NP * W + s] = df_pack(d2df_bits(U[0]));
     rf[7 * NP * W + s] = df_pack(d2df_bits(U[4]));
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      const double l = a.lam_scale * __ldg(a.lam + v * N + p);
+      const double l = __ldg(a.lam + v * N + p);
       lm[v * NP * W + s] = l;
       const int e = ((__double2hiint(l) >> 20) & 0x7ff) - 1023;
-      if (l != 0.0 && e > emax) emax = e;
+      if ((__double_as_longlong(l) << 1) != 0 && e > emax) emax = e;
     }
   }
   emax = __reduce_max_sync(0xffffffffu, emax);
   if ((tid & 31) == 0) atomicMax(&s_emax, emax);
   __syncthreads();
-  // E = exponent of the largest |lambda| (0 if lambda vanishes on the tile)
-  const int E = (s_emax == -2000) ? 0 : max(-1000, min(1000, s_emax));
+  // E = exponent of the largest |lambda| times that of lam_scale (0 if lambda vanishes on the tile)
+  const int es = ((__double2hiint(a.lam_scale) >> 20) & 0x7ff) - 1023;
+  const int E = (s_emax == -2000) ? 0 : max(-1000, min(1000, s_emax + es));
   int range_bad = 0;
   // first differences of the 9 scalars, FP64, kept as double-float; both lines of the tile
   // per item, stored side by side for the two-lane phases below
@@ -1009,9 +1012,9 @@ __global__ void __launch_bounds__(APF::THREADS, APF::MIN_CTAS) k_adj_dir_df(cons
     const double d1 = qm[tile_idx<D, W>(j + 1, 1, NP)] - qm[tile_idx<D, W>(j, 1, NP)];
     G4[m * NP + j] = df2_to4(df2_pack(d2df_bits(d0), d2df_bits(d1)));
   }
-  // adjoint of the interface fluxes, (lambda_{i+1} - lambda_i) / dx / 2^E
+  // adjoint of the interface fluxes, (lambda_{i+1} - lambda_i) lam_scale / dx / 2^E
   {
-    const double sc = rdx * pow2d(-E);
+    const double sc = rdx * (a.lam_scale * pow2d(-E));
     for (int item = APF::THREADS - 1 - tid; item < 5 * ni; item += APF::THREADS) {
       const int v = (int)(((unsigned)item * rcp_ni) >> 20);
       const int f = item - v * ni;
@@ -1447,17 +1450,36 @@ __global__ void __launch_bounds__(256) k_visc_adj2(const Grid g, const double* _
 // to FP64 once and finishes as k_visc_adj2.  The viscous terms are ~mu |grad u| in size, so
 // the double-float rounding (2^-48) lands far below the FP64 rounding of the direction
 // adjoints they are added to, as in the forward viscous kernel.
-// Largest binary exponent of lam_scale * lambda over the planes 1..4 of lambda, into *out (which
-// holds a large negative value before; it stays so if they all vanish).
+// Largest binary exponent of lambda over the planes 1..4, plus that of lam_scale, into *out (which
+// holds a large negative value before; it stays so if they all vanish).  Integers only, one atomic per
+// block on at most 608 blocks, four loads in flight per thread: 128^3 36 -> 23 us (ncu; a product
+// and a comparison on the FP64 pipe per value, and every warp of 4096 blocks on the one address).
 __global__ void __launch_bounds__(256) k_lam_expo(const double* __restrict__ lam, long long N, double lam_scale,
                                                   int* out) {
+  __shared__ int sh[8];
   int emax = INT_MIN;
-  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < 4 * N; i += (long long)gridDim.x * 256) {
-    const double l = lam_scale * __ldg(lam + N + i);
-    if (l != 0.0) emax = max(emax, ((__double2hiint(l) >> 20) & 0x7ff) - 1023);
+  const long long n = 4 * N, stride = (long long)gridDim.x * 256;
+  auto take = [&](double x) {
+    if ((__double_as_longlong(x) << 1) != 0) emax = max(emax, ((__double2hiint(x) >> 20) & 0x7ff) - 1023);
+  };
+  long long i = blockIdx.x * 256LL + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    const double x0 = __ldg(lam + N + i), x1 = __ldg(lam + N + i + stride);
+    const double x2 = __ldg(lam + N + i + 2 * stride), x3 = __ldg(lam + N + i + 3 * stride);
+    take(x0);
+    take(x1);
+    take(x2);
+    take(x3);
   }
+  for (; i < n; i += stride) take(__ldg(lam + N + i));
   emax = __reduce_max_sync(0xffffffffu, emax);
-  if ((threadIdx.x & 31) == 0 && emax != INT_MIN) atomicMax(out, emax);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x / 32] = emax;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    emax = __reduce_max_sync(0xffffffffu, threadIdx.x < 8 ? sh[threadIdx.x] : INT_MIN);
+    const int es = ((__double2hiint(lam_scale) >> 20) & 0x7ff) - 1023;
+    if (threadIdx.x == 0 && emax != INT_MIN) atomicMax(out, emax + es);
+  }
 }
 
 // The common exponent E of the two kernels (0 if lambda vanishes), inside the FP64 range.
@@ -1484,10 +1506,12 @@ __global__ void __launch_bounds__(256) k_visc_adj1_df(const Grid g, const double
     neighbours(i, j, k, d, g, nb);
     const df r12 = d2df_bits(g.r12h[d]);
 #pragma unroll
-    for (int qv = 0; qv < 4; ++qv) {
-      const double* A = pm + (long long)((qv < 3) ? qv : PM_T) * N;
+    for (int qv = 0; qv < 3; ++qv) {
+      const double* A = pm + (long long)qv * N;
       G[qv][d] = d4_df(__ldg(A + nb[0]), __ldg(A + nb[1]), __ldg(A + nb[2]), __ldg(A + nb[3]), r12);
     }
+    const double* A = pm + (long long)PM_T * N;  // double-float plane
+    G[3][d] = d4_dfv(load_df(A + nb[0]), load_df(A + nb[1]), load_df(A + nb[2]), load_df(A + nb[3]), r12);
   }
   const df vel[3] = {d2df_bits(pm[PM_U * N + p]), d2df_bits(pm[PM_V * N + p]), d2df_bits(pm[PM_W * N + p])};
   const double two3 = 2.0 / 3.0;
@@ -1697,7 +1721,7 @@ cudaError_t launch_visc_adj1(const Grid& g, const double* pm, const double* lam,
   if (expo) {
     cudaError_t e = cudaMemsetAsync(expo, 0x80, sizeof(int), s);  // 0x80808080: below every exponent
     if (e != cudaSuccess) return e;
-    const long long blocks = std::min<long long>((4 * g.N + 255) / 256, 4096);
+    const long long blocks = std::min<long long>((4 * g.N + 1023) / 1024, 4 * 152);
     k_lam_expo<<<(int)blocks, 256, 0, s>>>(lam, g.N, lam_scale, expo);
     k_visc_adj1_df<<<plane_blocks(g), 256, 0, s>>>(g, pm, lam, lam_scale, scratch, mu, kappa, expo);
   } else

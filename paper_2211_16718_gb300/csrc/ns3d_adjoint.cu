@@ -51,11 +51,13 @@ int copy_state(ns3d_ctx* c, double* dst, const double* src, const char* what) {
 // lnext, sb, c1, c2): primitives of u, viscous adjoint (writes k), then the three
 // direction adjoints (accumulate into k; the z pass runs the epilogue).
 int vjp_pass(ns3d_ctx* c, const double* u, const double* lam, double scale, AdjArgs e) {
-  int rc = timed(c, NS3D_K_PRIM, [&] { return launch_prim(c->g, u, c->pm, c->p.gamma, c->status, c->stream); },
+  // primitives in the layout of the context's mode: both double-float adjoint kernels take T, H and
+  // sqrt(rho) as double-float (one pass of 128^3 points 48 us where the all-FP64 layout takes 120)
+  const int df = (c->p.precision == NS3D_FP64_STRICT) ? 0 : 1;
+  int rc = timed(c, NS3D_K_PRIM, [&] { return launch_prim(c->g, u, c->pm, c->p.gamma, c->status, c->stream, df); },
                  "primitive kernel");
   if (rc) return rc;
   const bool visc = c->p.mu_eff > 0.0;
-  const int df = (c->p.precision == NS3D_FP64_STRICT) ? 0 : 1;
   if (visc) {
     const double kappa = c->p.mu_eff / ((c->p.gamma - 1.0) * c->p.prandtl);
     rc = timed(c, NS3D_K_ADJ_VISC, [&] {
