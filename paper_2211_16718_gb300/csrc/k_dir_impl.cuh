@@ -576,59 +576,73 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
           const float2 j = rj[scalar_of<MODE, D>(v) * NI * W + o];
           du[v] = df{j.x, j.y};
         }
-        const df ra = ldr(0, sa), rb = ldr(0, sb);
-        const df rsum = df_add_pos(ra, rb);
+        // what comes in twos runs on the two lanes of the packed operations: the states (a, b), the
+        // tangential directions, the acoustic fields, (V_D, H), flux components 0 and 1 + D.  The phase
+        // has one item per interface on half of the warps, so its length counts: 128^3 passes
+        // 397 / 415 / 471 -> 393 / 412 / 459 us (x / y / z)
+        constexpr int T1 = (D == 0) ? 1 : 0;
+        constexpr int T2 = (D == 2) ? 1 : 2;
+        const df2 gm1d = df2_splat(df{a.gm1_hi, a.gm1_lo});
+        auto l0 = [](df2 x) { return df2_lane0(x); };
+        auto l1 = [](df2 x) { return df2_lane1(x); };
+        auto ab = [&](int k) { return df2_pack(ldr(k, sa), ldr(k, sb)); };
+        const df2 r2 = ab(0);
+        const df rsum = df_add_pos(l0(r2), l1(r2));
         const df rs = df_div_r(df{1.0f, 0.0f}, rsum);  // refined, as 1/c and c below: at jumps their errors lead
-        const df wa = df_mul_u(ra, rs), wb = df_mul_u(rb, rs);
-        df V[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m) V[m] = df_add_fast(df_mul_u(wa, ldr(1 + m, sa)), df_mul_u(wb, ldr(1 + m, sb)));
-        const df H = df_add_pos(df_mul_u(wa, ldr(4, sa)), df_mul_u(wb, ldr(4, sb)));
-        const df q2 = df_add_pos_u(df_sqr_u(V[0]), df_add_pos_u(df_sqr_u(V[1]), df_sqr_u(V[2])));
+        const df2 w = df2_mul_u(r2, df2_splat(rs));
+        const df2 xt1 = df2_mul_u(w, ab(1 + T1)), xt2 = df2_mul_u(w, ab(1 + T2));
+        const df2 vt = df2_add_fast(df2_pack(l0(xt1), l0(xt2)), df2_pack(l1(xt1), l1(xt2)));  // (V_T1, V_T2)
+        const df2 xn = df2_mul_u(w, ab(1 + D)), xh = df2_mul_u(w, ab(4));
+        const df2 uH = df2_add_fast(df2_pack(l0(xn), l0(xh)), df2_pack(l1(xn), l1(xh)));  // (V_D, H)
+        const df un = l0(uH);
+        const df2 vq = df2_sqr_u(vt);
+        const df q2 = df_add_pos_u(df_sqr_u(un), df_add_pos_u(l0(vq), l1(vq)));
         const df q2h = df{0.5f * q2.hi, 0.5f * q2.lo};
-        const df c2 = df_mul(df_add_fast(H, df_neg(q2h)), df{a.gm1_hi, a.gm1_lo});
+        const df c2 = df_mul(df_add_fast(l1(uH), df_neg(q2h)), l0(gm1d));
         bad |= !(c2.hi > 0.0f);
         range_bad |= !(c2.hi > 1e-30f && c2.hi < 1e30f && rsum.hi > 1e-30f && rsum.hi < 1e30f);
         const df c = df_sqrt_r(c2);
         const df rc = df_div_r(df{1.0f, 0.0f}, c);
-        constexpr int T1 = (D == 0) ? 1 : 0;
-        constexpr int T2 = (D == 2) ? 1 : 2;
-        const df un = V[D], vt1 = V[T1], vt2 = V[T2];
-        const df b1 = df_mul_u(df{a.gm1_hi, a.gm1_lo}, df_sqr_u(rc));
-        const df vdm = df_add_fast(df_mul_u(V[0], du[1]), df_add_fast(df_mul_u(V[1], du[2]), df_mul_u(V[2], du[3])));
-        const df phi = df_mul_u(b1, df_add_fast(df_add_fast(df_mul_u(q2h, du[0]), du[4]), df_neg(vdm)));
+        const df2 dut = df2_pack(du[1 + T1], du[1 + T2]);
+        const df2 vd = df2_mul_u(vt, dut);
+        const df2 ud = df2_mul_u(df2_pack(un, q2h), df2_pack(du[1 + D], du[0]));
+        const df vdm = df_add_fast(l0(ud), df_add_fast(l0(vd), l1(vd)));
+        const df phi = df_mul_u(df_mul_u(l0(gm1d), df_sqr_u(rc)), df_add_fast(df_add_fast(l1(ud), du[4]), df_neg(vdm)));
         const df a2 = df_add_fast(du[0], df_neg(phi));
-        const df a3 = df_add_fast(du[1 + T1], df_neg(df_mul_u(vt1, du[0])));
-        const df a4 = df_add_fast(du[1 + T2], df_neg(df_mul_u(vt2, du[0])));
-        const df ach0 = df_mul_u(df_add_fast(df_mul_u(un, du[0]), df_neg(du[1 + D])), rc);
-        const df ach = df{0.5f * ach0.hi, 0.5f * ach0.lo};
-        const df ph = df{0.5f * phi.hi, 0.5f * phi.lo};
-        const df a1 = df_add_fast(ph, ach), a5 = df_add_fast(ph, df_neg(ach));
-        df l1 = df_abs(df_add_fast(un, df_neg(c))), l5 = df_abs(df_add_fast(un, c));
-        const df l2 = df_abs(un);
+        const df2 a34 = df2_add_fast(dut, df2_neg(df2_mul_u(vt, df2_splat(du[0]))));
+        const df ach = df_mul_u(df_add_fast(df_mul_u(un, du[0]), df_neg(du[1 + D])), rc);
+        // (a1, a5) = (phi +- ach)/2
+        const df2 a15 = df2_scale(df2_add_fast(df2_splat(phi), df2_pack(ach, df_neg(ach))), f2splat(0.5f));
+        const df2 lam = df2_add_fast(df2_splat(un), df2_pack(df_neg(c), c));
+        df h1 = df_abs(l0(lam)), h5 = df_abs(l1(lam));
+        const df h2 = df_abs(un);
         const df delta = df_mul(c, df{a.hd_hi, a.hd_lo});
-        if (df_lt(l1, delta)) l1 = df_div(df_add_pos_u(df_sqr_u(l1), df_sqr_u(delta)), df_twice(delta));
-        if (df_lt(l5, delta)) l5 = df_div(df_add_pos_u(df_sqr_u(l5), df_sqr_u(delta)), df_twice(delta));
-        const df A1 = df_mul_u(l1, a1), A2 = df_mul_u(l2, a2), A3 = df_mul_u(l2, a3), A4 = df_mul_u(l2, a4);
-        const df A5 = df_mul_u(l5, a5);
-        const df S = df_add_fast(A1, A5);
+        if (df_lt(h1, delta)) h1 = df_div(df_add_pos_u(df_sqr_u(h1), df_sqr_u(delta)), df_twice(delta));
+        if (df_lt(h5, delta)) h5 = df_div(df_add_pos_u(df_sqr_u(h5), df_sqr_u(delta)), df_twice(delta));
+        const df2 A15 = df2_mul_u(df2_pack(h1, h5), a15), A34 = df2_mul_u(df2_splat(h2), a34);
+        const df A2 = df_mul_u(h2, a2);
+        const df S = df_add_fast(l0(A15), l1(A15));
         const df d0 = df_add_fast(S, A2);
-        const df cD = df_mul_u(c, df_add_fast(A5, df_neg(A1)));
-        df diss[5];
-        diss[0] = d0;
-        diss[1 + D] = df_add_fast(df_mul_u(d0, un), cD);
-        diss[1 + T1] = df_add_fast(df_mul_u(d0, vt1), A3);
-        diss[1 + T2] = df_add_fast(df_mul_u(d0, vt2), A4);
-        diss[4] = df_add_fast(df_add_fast(df_mul_u(S, H), df_mul_u(cD, un)),
-                              df_add_fast(df_mul_u(A2, q2h), df_add_fast(df_mul_u(A3, vt1), df_mul_u(A4, vt2))));
+        const df cD = df_mul_u(c, df_add_fast(l1(A15), df_neg(l0(A15))));
+        const df2 dT = df2_add_fast(df2_mul_u(df2_splat(d0), vt), A34);
+        const df dn = df_add_fast(df_mul_u(d0, un), cD);
+        const df2 e1 = df2_mul_u(df2_pack(S, cD), df2_pack(l1(uH), un));
+        const df2 e2 = df2_mul_u(A34, vt);
+        const df de = df_add_fast(df_add_fast(l0(e1), l1(e1)),
+                                  df_add_fast(df_mul_u(A2, q2h), df_add_fast(l0(e2), l1(e2))));
         const df hr = d2df_bits(a.g.hrh[D]);
         const float2* ts = reinterpret_cast<const float2*>(sm + PL::OFF_T);
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {  // flux component 0 is u_{1+D}
-          const float2 tv = ts[v * NI * W + o];
-          const df t = df_mul(df_add_fast(df{tv.x, tv.y}, df_neg(diss[v])), hr);
+        auto ldt = [&](int v) { const float2 tv = ts[v * NI * W + o]; return df{tv.x, tv.y}; };
+        auto put = [&](int v, df t) {  // flux component 0 is u_{1+D}
           rec[v * NI * W + o] = fma(a.g.rh[D], rec[(5 + v) * NI * W + o], f2d_bits(t.hi)) + f2d_bits(t.lo);
-        }
+        };
+        const df2 f0n = df2_mul(df2_add_fast(df2_pack(ldt(0), ldt(1 + D)), df2_neg(df2_pack(d0, dn))), df2_splat(hr));
+        put(0, l0(f0n));
+        put(1 + D, l1(f0n));
+        const df2 fT = df2_mul(df2_add_fast(df2_pack(ldt(1 + T1), ldt(1 + T2)), df2_neg(dT)), df2_splat(hr));
+        put(1 + T1, l0(fT));
+        put(1 + T2, l1(fT));
+        put(4, df_mul(df_add_fast(ldt(4), df_neg(de)), hr));
         continue;
       }
       double du[5];
