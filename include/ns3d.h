@@ -126,7 +126,8 @@ void ns3d_default_params(ns3d_params *p, int nx, int ny, int nz);
 
 /* Create a context: validates *p (NS3D_EINVAL), allocates the library-owned
  * device scratch (NS3D_ENOMEM): primitive variables 7*N, viscous fluxes 12*N
- * (4*N with NS3D_STORAGE_LEAN; none if mu_eff = 0), RHS accumulator 5*N doubles,
+ * (4*N with NS3D_STORAGE_LEAN; none if mu_eff = 0), RHS accumulator 5*N doubles (10*N
+ * on grids of up to 2^20 points, except NS3D_FP32_BULK and viscous lean storage),
  * reduction partials and a status word.  The first Runge-Kutta step allocates
  * two stage states 10*N (and for RK4 an accumulator 5*N) doubles.
  * cuda_stream: a cudaStream_t (NULL = legacy default stream). */
@@ -234,7 +235,7 @@ enum { NS3D_BATCH_SEQUENTIAL = 0, NS3D_BATCH_GRAPH = 1, NS3D_BATCH_PERSISTENT = 
 typedef struct ns3d_batch ns3d_batch;
 
 /* params[count] (count 1..4096, each grid <= 2^31 points); allocates the
- * per-instance scratch (~39 doubles per point).  NS3D_EINVAL / NS3D_ENOMEM. */
+ * per-instance scratch (39 doubles per point, 44 up to 2^15 points).  NS3D_EINVAL / NS3D_ENOMEM. */
 int ns3d_batch_init(const ns3d_params *params, int count, void *cuda_stream, ns3d_batch **out);
 void ns3d_batch_free(ns3d_batch *b);
 /* u_dev[count]: host array of caller-owned device states (layout as above). */

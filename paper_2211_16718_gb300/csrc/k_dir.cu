@@ -22,6 +22,48 @@ __global__ void __launch_bounds__(Plan<MODE, TP, W>::THREADS, Plan<MODE, TP, W>:
   dir_tile<D, MODE, TP, W>(a, sm, s0, len, swap ? blockIdx.x : blockIdx.y, blockIdx.z + (D == 2 ? 0 : a.t0));
 }
 
+// The x pass (blocks below nbx) and the y pass side by side in one launch: neither reads what the
+// other writes.  It fills the second pass's launch gap and the last, partly filled round of CTAs:
+// 40x25x18 right-hand side 34.8 -> 30.2 us, 32^3 RK4 step 240 -> 215 us, 64^3 passes 115 -> 112 us,
+// 96^3 all-FP64 step 8.97 -> 8.91 ms, but 128^3 passes 805 -> 816 us (the two code paths share the
+// instruction caches), so only grids of up to 2^20 points (dir_xy_merged).
+template <int MODE, int TP, int W>
+__global__ void __launch_bounds__(Plan<MODE, TP, W>::THREADS, Plan<MODE, TP, W>::MIN_CTAS) k_dir_xy(const DirArgs ax,
+                                                                                                const DirArgs ay,
+                                                                                                int nbx) {
+  extern __shared__ __align__(16) double sm[];
+  int s0, len;
+  if ((int)blockIdx.x < nbx) {
+    const int nt = (ax.g.n[0] + TP - 1) / TP, nl = (ax.g.n[1] + W - 1) / W;
+    const int r = blockIdx.x / nt, bz = r / nl;
+    tile_span(0, ax.g.n[0], ax.tile_u, ax.tile_r, blockIdx.x - r * nt, s0, len);
+    dir_tile<0, MODE, TP, W>(ax, sm, s0, len, r - bz * nl, bz);
+  } else {
+    const int b = blockIdx.x - nbx;
+    const int nt = (ay.g.n[1] + TP - 1) / TP, nl = (ay.g.n[0] + W - 1) / W;
+    const int r = b / nt, bz = r / nl;
+    tile_span(1, ay.g.n[1], ay.tile_u, ay.tile_r, b - r * nt, s0, len);
+    dir_tile<1, MODE, TP, W>(ay, sm, s0, len, r - bz * nl, bz);
+  }
+}
+
+template <int MODE, int TP, int W>
+cudaError_t launch_xy(const DirArgs& a, double* k2, cudaStream_t s) {
+  using PL = Plan<MODE, TP, W>;
+  const int* n = a.g.n;
+  const int nx = (n[0] + TP - 1) / TP, ny = (n[1] + TP - 1) / TP;
+  const long long nbx = (long long)nx * ((n[1] + W - 1) / W) * n[2], nby = (long long)ny * ((n[0] + W - 1) / W) * n[2];
+  if (nbx + nby > 0x7fffffffLL) return cudaErrorInvalidValue;
+  DirArgs x = a, y = a;
+  x.epi = y.epi = EPI_ACC_WRITE;
+  x.t0 = y.t0 = 0;
+  y.k = k2;
+  tile_split_units(0, n[0], nx, x.tile_u, x.tile_r);
+  tile_split_units(1, n[1], ny, y.tile_u, y.tile_r);
+  k_dir_xy<MODE, TP, W><<<(unsigned)(nbx + nby), PL::THREADS, PL::BYTES, s>>>(x, y, (int)nbx);
+  return cudaGetLastError();
+}
+
 // Tiles [lo, hi) along the range axis (hi < 0: all): the tiles along z for D = 2 (blockIdx.x, or
 // blockIdx.y with a.zorder), blockIdx.z (planes z) for D = 0, 1.
 template <int D, int MODE, int TP, int W>
@@ -63,6 +105,7 @@ cudaError_t set_attr() {
   cudaError_t e = set_func_attr(k_dir<0, MODE, TP, W>, bytes);
   if (e == cudaSuccess) e = set_func_attr(k_dir<1, MODE, TP, W>, bytes);
   if (e == cudaSuccess) e = set_func_attr(k_dir<2, MODE, TP, W>, bytes);
+  if (e == cudaSuccess) e = set_func_attr(k_dir_xy<MODE, TP, W>, bytes);
   return e;
 }
 
@@ -127,6 +170,16 @@ int dir_tile_start(const Grid& g, int d, int mode, int variant, int t) {
 cudaError_t launch_dir(int d, const DirArgs& a, cudaStream_t s) {
   if (a.mode == 2) return launch_dir32(d, a, s);
   return launch_dir_range(d, a, s, 0, -1);
+}
+
+cudaError_t launch_dir_xy(const DirArgs& a, double* k2, cudaStream_t s) {
+  if (a.mode == 2 || (a.fv != nullptr && a.fv_dstride == 0)) return cudaErrorInvalidValue;
+  if (a.mode == 0) return launch_xy<0, 32, 4>(a, k2, s);
+  switch (a.variant) {
+    case 1: return launch_xy<1, 16, 4>(a, k2, s);
+    case 2: return launch_xy<1, 40, 2>(a, k2, s);
+    default: return launch_xy<1, 24, 4>(a, k2, s);
+  }
 }
 
 cudaError_t launch_dir_range(int d, const DirArgs& a, cudaStream_t s, int lo, int hi) {

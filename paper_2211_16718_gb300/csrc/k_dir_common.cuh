@@ -126,7 +126,7 @@ __device__ __forceinline__ void cp_async_d(double* dst_smem, const double* src) 
 }
 
 // Start fetching the epilogue operands of point p (PAIR: of p and p + 1) into pre[v * TS],
-// v < epilogue_operands(a.epi).
+// v < epilogue_operands(a.epi), and the y contribution, if it is apart, into v = 15 .. 19.
 template <bool PAIR, int TS>
 __device__ __forceinline__ void epilogue_prefetch(const DirArgs& a, long long p, double* pre) {
   const long long N = a.g.N;
@@ -143,6 +143,10 @@ __device__ __forceinline__ void epilogue_prefetch(const DirArgs& a, long long p,
 #pragma unroll
     for (int v = 0; v < 5; ++v) cp_async_d<PAIR>(pre + (10 + v) * TS, third + v * N + p);
   }
+  if (a.k2 != nullptr) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) cp_async_d<PAIR>(pre + (15 + v) * TS, a.k2 + v * N + p);
+  }
 }
 
 // Accumulate this direction's contribution cv[5] at point p, or finish the RHS / RK stage (last
@@ -151,6 +155,7 @@ template <int TS>
 __device__ __forceinline__ void dir_epilogue_pre(const DirArgs& a, long long p, const double cv[5],
                                                  const double* pre) {
   const long long N = a.g.N;
+  auto kxy = [&](int v) { return a.k2 != nullptr ? pre[v * TS] + pre[(15 + v) * TS] : pre[v * TS]; };
   switch (a.epi) {
     case EPI_ACC_WRITE:
 #pragma unroll
@@ -162,12 +167,12 @@ __device__ __forceinline__ void dir_epilogue_pre(const DirArgs& a, long long p, 
       break;
     case EPI_RHS_OUT:
 #pragma unroll
-      for (int v = 0; v < 5; ++v) a.out[v * N + p] = pre[v * TS] + cv[v];
+      for (int v = 0; v < 5; ++v) a.out[v * N + p] = kxy(v) + cv[v];
       break;
     case EPI_RK4_FIRST:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v * TS] + cv[v];
+        const double K = kxy(v) + cv[v];
         a.out[v * N + p] = fma(a.a, K, pre[(5 + v) * TS]);
         a.acc[v * N + p] = K;
       }
@@ -175,7 +180,7 @@ __device__ __forceinline__ void dir_epilogue_pre(const DirArgs& a, long long p, 
     case EPI_RK4_MID:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v * TS] + cv[v];
+        const double K = kxy(v) + cv[v];
         a.out[v * N + p] = fma(a.a, K, pre[(5 + v) * TS]);
         a.acc[v * N + p] = fma(2.0, K, pre[(10 + v) * TS]);
       }
@@ -183,28 +188,28 @@ __device__ __forceinline__ void dir_epilogue_pre(const DirArgs& a, long long p, 
     case EPI_RK4_LAST:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v * TS] + cv[v];
+        const double K = kxy(v) + cv[v];
         a.out[v * N + p] = fma(a.a, pre[(10 + v) * TS] + K, pre[(5 + v) * TS]);
       }
       break;
     case EPI_SSP_1:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v * TS] + cv[v];
+        const double K = kxy(v) + cv[v];
         a.out[v * N + p] = fma(a.a, K, pre[(5 + v) * TS]);
       }
       break;
     case EPI_SSP_2:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v * TS] + cv[v];
+        const double K = kxy(v) + cv[v];
         a.out[v * N + p] = 0.75 * pre[(5 + v) * TS] + 0.25 * fma(a.a, K, pre[(10 + v) * TS]);
       }
       break;
     case EPI_SSP_3:
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        const double K = pre[v * TS] + cv[v];
+        const double K = kxy(v) + cv[v];
         a.out[v * N + p] = (1.0 / 3.0) * pre[(5 + v) * TS] + (2.0 / 3.0) * fma(a.a, K, pre[(10 + v) * TS]);
       }
       break;

@@ -97,7 +97,7 @@ struct Plan {
   static constexpr int OFF_B = (MODE == 0)          ? OFF_ROE + (5 + 4) * NP * W
                                : (END_T > NQ * NP * W) ? (END_T + 1) / 2 * 2
                                                        : OFF_Q + NQ * NP * W;
-  static constexpr int OFF_FV = (MODE == 1) ? OFF_B + 15 * TP * W : OFF_ROE + 5 * NP * W;
+  static constexpr int OFF_FV = (MODE == 1) ? OFF_B + 20 * TP * W : OFF_ROE + 5 * NP * W;
   static constexpr int OFF_S = OFF_B + NQ * (MODE == 0 ? 4 : 3) * NW * W;  // MODE 1: third differences
   static constexpr int OFF_G = OFF_S + (MODE == 1 ? NQ * NW * W : 0);
   static constexpr int OFF_R = OFF_G + (MODE == 1 ? NQ * NG * W : 0);
@@ -515,7 +515,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
   //      false), where the operands were written by other CTAs before the last grid-wide
   //      barrier, it sees them exactly as the plain loads it replaces would.
   static_assert(PL::TP * PL::W <= PL::THREADS, "one epilogue point per thread");
-  static_assert(15 * PL::TP * PL::W <= NQ * 3 * PL::NW * PL::W, "prefetch slots fit the indicator space");
+  static_assert(20 * PL::TP * PL::W <= NQ * 3 * PL::NW * PL::W, "prefetch slots fit the indicator space");
   //      The z pass with nx even takes two x-adjacent points (lines 2j, 2j + 1 of the tile: their flat
   //      index is even) per 16-byte copy, past L1: half the copies.  U_n and the stage input may be
   //      the caller's and only 8-byte aligned; the rest is the library's.  z pass with the RK4
@@ -524,7 +524,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
   //      just read three of their five planes through L1).
   const bool pair16 = D == 2 && W % 2 == 0 && (na & 1) == 0 && (((uintptr_t)a.un | (uintptr_t)a.u) & 15) == 0;
   constexpr int TS = TP * W;
-  double* pre = sm + PL::OFF_B;  // [15][TP*W]
+  double* pre = sm + PL::OFF_B;  // [20][TP*W]
   const int ft = tid - PL::FETCH0;
   auto fetch_epilogue = [&](auto pair) {
     constexpr bool PAIR = decltype(pair)::value;

@@ -29,6 +29,7 @@ DirArgs base_args(ns3d_ctx* c, const double* u) {
   a.fv = (c->p.mu_eff > 0.0) ? c->fv : nullptr;
   a.fv_dstride = c->lean ? 0 : 4;
   a.k = c->k;
+  a.k2 = nullptr;
   a.epi = EPI_ACC_WRITE;
   a.out = nullptr;
   a.un = nullptr;
@@ -131,9 +132,15 @@ int rhs_pass(ns3d_ctx* c, const double* u, int epi, double* out, const double* u
   } else {
     if ((rc = prim(0, g.n[2]))) return rc;
     if (visc && !c->lean && (rc = visc_flux(-1, 0, -1))) return rc;
-    for (int d = 0; d < 2; ++d) {
-      if (visc && c->lean && (rc = visc_flux(d, 0, -1))) return rc;
-      if ((rc = dir(d, 0, -1))) return rc;
+    if (c->k2 && !c->timing) {  // the x and y passes in one launch (timed apart, they are launched apart)
+      if ((rc = timed(c, kid[0], [&] { return launch_dir_xy(a, c->k2, c->stream); }, "x- and y-direction kernel")))
+        return rc;
+      a.k2 = c->k2;
+    } else {
+      for (int d = 0; d < 2; ++d) {
+        if (visc && c->lean && (rc = visc_flux(d, 0, -1))) return rc;
+        if ((rc = dir(d, 0, -1))) return rc;
+      }
     }
   }
   if (visc && c->lean && (rc = visc_flux(2, 0, -1))) return rc;
@@ -333,6 +340,8 @@ int ns3d_init(const ns3d_params* p, void* cuda_stream, ns3d_ctx** out) {
     ns3d_free(c);
     return NS3D_ENOMEM;
   }
+  const bool xy = p->precision != NS3D_FP32_BULK && !(visc && c->lean) && dir_xy_merged(c->g.N);
+  if (xy) dev_alloc(c, (void**)&c->k2, sizeof(double) * 5 * N);  // without it the passes are launched apart
   if (cudaMallocHost((void**)&c->stats_host, sizeof(double) * NS3D_STATS_NDOUBLE) != cudaSuccess) {
     cudaGetLastError();
     ns3d_free(c);
@@ -365,6 +374,7 @@ void ns3d_free(ns3d_ctx* c) {
   cudaFree(c->pm);
   cudaFree(c->fv);
   cudaFree(c->k);
+  cudaFree(c->k2);
   cudaFree(c->ua);
   cudaFree(c->ub);
   cudaFree(c->acc);

@@ -37,6 +37,11 @@ namespace {
 
 constexpr int MAX_STAGES = 4;
 constexpr int BT = 256;  // threads of the pointwise batched kernels
+// Instances up to this size run their x and y passes in one launch (launch_dir_xy).  GRAPH schedule:
+// 48 grids of 12^3-24^3 2.03 -> 1.77 ms per step, 8 of them 0.40 -> 0.36 ms; larger instances fill the
+// gaps of one another already (16 grids of 24^3-48^3 2.43 ms apart, 2.48 with all of them merged,
+// 2.41 with this line; 48 of 32^3-128^3 79.5, 80.0, 79.7 ms).
+constexpr long long BATCH_XY_POINTS = 1LL << 15;
 
 struct Inst {
   Grid g;
@@ -265,10 +270,10 @@ int rebuild(ns3d_batch* b) {
     Inst& in = b->inst[i];
     in.variant = (b->mode == 1) ? b->ivar[i] : 0;
     double* u = b->u[i];
-    double* ua = b->bufs[6 * i + 2];
-    double* ub = b->bufs[6 * i + 3];
-    double* acc = b->bufs[6 * i + 4];
-    double* k = b->bufs[6 * i + 5];
+    double* ua = b->bufs[7 * i + 2];
+    double* ub = b->bufs[7 * i + 3];
+    double* acc = b->bufs[7 * i + 4];
+    double* k = b->bufs[7 * i + 5];
     const double dt = b->dt[i];
     const double* uin4[4] = {u, ua, ub, ua};
     double* out4[4] = {ua, ub, ua, u};
@@ -344,7 +349,15 @@ cudaError_t step_instance(const ns3d_batch* b, int i, cudaStream_t st) {
   for (int s = 0; s < b->nstages && e == cudaSuccess; ++s) {
     e = launch_prim(in.g, in.uin[s], in.pm, in.gamma, b->d_status, st, b->mode);
     if (e == cudaSuccess && in.fv) e = launch_visc(in.g, in.pm, in.fv, in.mu, in.kappa, st, -1, b->mode);
-    for (int d = 0; d < 3 && e == cudaSuccess; ++d) e = launch_dir(d, in.dir[s][d], st);
+    double* k2 = b->bufs[7 * i + 6];
+    if (k2 == nullptr) {
+      for (int d = 0; d < 3 && e == cudaSuccess; ++d) e = launch_dir(d, in.dir[s][d], st);
+      continue;
+    }
+    if (e == cudaSuccess) e = launch_dir_xy(in.dir[s][0], k2, st);
+    DirArgs z = in.dir[s][2];
+    z.k2 = k2;
+    if (e == cudaSuccess) e = launch_dir(2, z, st);
   }
   return e;
 }
@@ -590,22 +603,27 @@ int ns3d_batch_init(const ns3d_params* params, int count, void* cuda_stream, ns3
     b->pt_off[i + 1] = b->pt_off[i] + in.g.N;
     b->nstat_blocks = std::max(b->nstat_blocks, stats_num_blocks(in.g));
     // scratch: primitives, viscous fluxes, two stage states, RK accumulator, RHS accumulator
-    const size_t sizes[6] = {7, 12, 5, 5, 5, 5};
-    for (int a = 0; a < 6; ++a) {
+    // and, where the x and y passes share a launch, the y contribution
+    const size_t sizes[7] = {7, 12, 5, 5, 5, 5, 5};
+    for (int a = 0; a < 7; ++a) {
       double* ptr = nullptr;
-      if (a == 1 && p.mu_eff == 0.0) {
+      if ((a == 1 && p.mu_eff == 0.0) || (a == 6 && in.g.N > BATCH_XY_POINTS)) {
         b->bufs.push_back(nullptr);
         continue;
       }
       if (cudaMalloc(&ptr, sizeof(double) * sizes[a] * (size_t)in.g.N) != cudaSuccess) {
         cudaGetLastError();
+        if (a == 6) {  // the passes are then launched apart
+          b->bufs.push_back(nullptr);
+          continue;
+        }
         ns3d_batch_free(b);
         return NS3D_ENOMEM;
       }
       b->bufs.push_back(ptr);
     }
-    in.pm = b->bufs[6 * i + 0];
-    in.fv = b->bufs[6 * i + 1];
+    in.pm = b->bufs[7 * i + 0];
+    in.fv = b->bufs[7 * i + 1];
   }
   bool ok = cudaMalloc(&b->d_inst, sizeof(Inst) * count) == cudaSuccess &&
             cudaMalloc(&b->d_pt_off, sizeof(long long) * (count + 1)) == cudaSuccess &&

@@ -22,6 +22,7 @@ struct ns3d_ctx {
   double* pm = nullptr;        // [NPRIM][N]
   double* fv = nullptr;        // [NVISC][N] (viscous only)
   double* k = nullptr;         // [5][N] RHS accumulator
+  double* k2 = nullptr;        // [5][N] y contribution of launch_dir_xy (small grids, all viscous fluxes stored)
   double* ua = nullptr;        // [5][N] stage state
   double* ub = nullptr;        // [5][N] stage state
   double* acc = nullptr;       // [5][N] RK4 accumulator

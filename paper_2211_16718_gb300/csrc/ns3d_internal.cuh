@@ -59,6 +59,7 @@ struct DirArgs {
   const double* fv;  // viscous fluxes [NVISC][N] or nullptr (inviscid); FP32-bulk: FP32 planes
   int fv_dstride;    // planes per direction in fv: 4 ([12][N], all directions) or 0 ([4][N], this direction)
   double* k;         // RHS accumulator [5][N]
+  const double* k2;  // z pass: the y contribution, if the x and y passes did not accumulate into k (launch_dir_xy)
   int epi;           // Epi
   double* out;       // EPI_RHS_OUT: destination; RK modes: next stage state
   const double* un;  // RK base state U_n
@@ -97,6 +98,11 @@ cudaError_t launch_visc32(const Grid& g, const double* u, float* fv, double gamm
                           cudaStream_t s, int only_d = -1);
 cudaError_t prepare_dir_kernels();  // per device, before the first launch
 cudaError_t launch_dir(int d, const DirArgs& a, cudaStream_t s);  // dispatches on a.mode, a.variant
+// The x and y passes in one launch, their contributions in a.k and k2 (the z pass then gets both:
+// DirArgs::k2; the same sums in the same order).  MODE 0 and 1, all viscous fluxes stored.
+cudaError_t launch_dir_xy(const DirArgs& a, double* k2, cudaStream_t s);
+// Whether it pays on a grid (and its 5*N doubles are kept): see k_dir_xy.
+inline bool dir_xy_merged(long long N) { return N <= (1LL << 20); }
 // The tiles [lo, hi) of a direction pass along its range axis: planes z for d = 0, 1, tiles along z
 // (dir_tile_start) for d = 2.  MODE 0 and 1 only.
 cudaError_t launch_dir_range(int d, const DirArgs& a, cudaStream_t s, int lo, int hi);

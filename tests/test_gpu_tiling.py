@@ -130,3 +130,22 @@ def test_adjoint_tiles(ns3d, nx, ny, nz):
         s.check()
         s.close()
     assert rel_err(out[0], out[1]) <= 1e-11
+
+
+@pytest.mark.parametrize("prec,rk", [(0, 0), (0, 1), (2, 0)])
+@pytest.mark.parametrize("nx,ny,nz", [(25, 30, 9), (64, 5, 1), (33, 26, 50)])
+def test_merged_xy_passes_give_the_same_bits(ns3d, prec, rk, nx, ny, nz):
+    """The x and y passes in one launch (small grids) against separate launches: contexts whose
+    kernels are timed, and lean storage, launch them apart."""
+    import torch
+    u = _gpu(I.random_smooth(nx, ny, nz, seed=10, amp=0.1, mach=0.5))
+    out = []
+    for timed, storage in ((False, 1), (True, 1), (False, 2)):
+        s = ns3d.Solver(nx, ny, nz, mu_eff=0.003, precision=prec, rk=rk, storage=storage)
+        s.timing_enable(timed)
+        v = u.clone()
+        s.rk_step(v, 0.01, 2)
+        out.append((s.rhs(u), v))
+        s.close()
+    for r, v in out[1:]:
+        assert torch.equal(r, out[0][0]) and torch.equal(v, out[0][1])
