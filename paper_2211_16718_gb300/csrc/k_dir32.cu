@@ -19,8 +19,8 @@
 //      part, the viscous interface flux (-f_{i-1} + 7 f_i + 7 f_{i+1} - f_{i+2})/12,
 //      divided by dx and widened to FP64;
 //  E   per point: FP64 difference of its two interface fluxes, then the
-//      accumulation / RK epilogue (its operands prefetched by cp.async during D; in the y
-//      and z passes a thread takes two x-adjacent points and moves 16-byte pairs).
+//      accumulation / RK epilogue (its operands prefetched by cp.async during D, in the y
+//      and z passes two x-adjacent points per 16-byte copy).
 #include <math.h>
 
 #include "df.cuh"
@@ -32,32 +32,38 @@ namespace ns3d {
 namespace {
 
 constexpr int THREADS = 256;
-constexpr int TP = 27, W = 8;   // 27 points: 19 tiles cover 512 (513), 38 cover 1024 (1026)
+// At most 27 points along x, 26 along y and z (balanced tiles, k_dir_common.cuh) x 8 lines.  26 are 256
+// points with the halo, one per thread in phase A; 27 take a second round of 8, but the x pass gains
+// more from the smaller share of halo.  512^3 passes, x / y / z: 5.57 / 6.23 / 10.35 ms with 27,
+// 5.80 / 6.21 / 10.13 ms with 26; the step with 24 everywhere 2 % slower, with 23 5 %.  Before, full tiles
+// of 27 with a remainder computed in full and two points per thread in E: 5.59 / 6.85 / 10.21 ms (and
+// 69 % of the work wasted on a 32-point line).
+__host__ __device__ constexpr int tile_max(int d) { return d == 0 ? 27 : 26; }
+constexpr int TP = tile_max(0), W = 8;
 constexpr int NP = TP + 6;      // positions per line: 3-point halo on each side
 constexpr int NI = TP + 1;      // interfaces per line
 constexpr int SEG = 4;          // interfaces per reconstruction item
-constexpr int NSEG = NI / SEG;  // 7
-static_assert(NI % SEG == 0, "whole segments");
+constexpr int NSEG = (NI + SEG - 1) / SEG;  // 7
 constexpr int NQ = 9;           // reconstructed scalars: 5 conserved, 4 flux components (f_0 = u_{1+D})
+constexpr int RS = 28;          // line stride (floats) of the reconstruction results: whole segments
 constexpr int NREC = 10;        // per interface: 5 jumps, the sum of u_{1+D}, 4 flux sums
 constexpr int LS = 36;          // line stride (floats) of the scalar planes: >= SEG*NSEG + 5 and a multiple of 4
 constexpr int L4 = NP;          // line stride (float4) of the Roe-input and viscous planes (odd: no bank conflicts)
-static_assert(SEG * (NSEG - 1) + 12 <= LS && LS % 4 == 0, "segment reads (three float4) stay in the line");
+static_assert(SEG * (NSEG - 1) + 12 <= LS && LS % 4 == 0 && RS == SEG * NSEG, "segment reads (three float4) stay in the line");
 // shared-memory plan (bytes)
-constexpr int OFF_Q = 0;                              // float  [NQ][W][LS]
-constexpr int OFF_R4 = OFF_Q + NQ * W * LS * 4;       // float4 [W][L4]: sqrt(rho), u, v, w
+constexpr int OFF_R4 = 0;                             // float4 [W][L4]: sqrt(rho), u, v, w
 constexpr int OFF_H = OFF_R4 + W * L4 * 16;           // float  [W][L4]: H
 constexpr int OFF_V4 = OFF_H + ((W * L4 * 4 + 15) & ~15);  // float4 [W][L4]: viscous flux of this direction
-constexpr int OFF_REC = OFF_V4 + W * L4 * 16;         // float  [NREC][W][NI]
+constexpr int OFF_REC = OFF_V4 + W * L4 * 16;         // float  [NREC][W][RS]
 constexpr int FS = 30;          // line stride (doubles) of the interface fluxes (no bank conflicts in y, z)
-constexpr int OFF_F = OFF_REC + NREC * W * NI * 4;    // double [5][W][FS]: interface flux / dx
-constexpr int OFF_P2 = OFF_F + 5 * W * FS * 8;         // double [TP*W][10]: epilogue operands U_n and acc / u
-constexpr int BYTES = OFF_P2 + 10 * TP * W * 8;
+constexpr int OFF_F = OFF_REC + NREC * W * RS * 4;    // double [5][W][FS]: interface flux / dx
+constexpr int OFF_Q = OFF_F + 5 * W * FS * 8;          // float  [NQ][W][LS]; dead after BC: the epilogue operands,
+constexpr int TS = TP * W;                            //   double [15][TP*W], from here on
+constexpr int BYTES = OFF_Q + 15 * TS * 8;
 static_assert(FS >= NI, "interface-flux line");
-// epilogue operand k (5 doubles per point) prefetched into the scalar planes, dead after BC
-static_assert(5 * TP * W * 8 <= NQ * W * LS * 4, "prefetch slots fit the scalar planes");
+static_assert(NQ * W * LS * 4 <= 15 * TS * 8, "the scalar planes fit the operands' space");
 static_assert(BYTES + 1024 <= 233472 / 4, "four CTAs per SM");
-static_assert(OFF_R4 % 16 == 0 && OFF_V4 % 16 == 0 && OFF_F % 8 == 0 && OFF_REC % 16 == 0, "alignment");
+static_assert(OFF_Q % 16 == 0 && OFF_V4 % 16 == 0 && OFF_F % 8 == 0 && OFF_REC % 16 == 0, "alignment");
 static_assert(TP * W <= THREADS && NI * W <= THREADS, "one point / interface per thread in D and E");
 
 // FP64 -> FP32 by truncating the bit pattern (integer instructions only): sign and exponent
@@ -111,145 +117,6 @@ __device__ __forceinline__ float weno_safe(float B1, float B2, float B3, float c
   return c + __fdiv_rn(num, den);
 }
 
-// Accumulation / RK epilogue with its operands from the prefetch slots: kp = k, ops = U_n then
-// acc or the stage input; the arithmetic of dir_epilogue_pre.
-__device__ __forceinline__ void dir_epilogue_pre32(const DirArgs& a, long long p, const double cv[5], const double* kp,
-                                                   const double* ops) {
-  const long long N = a.g.N;
-  switch (a.epi) {
-    case EPI_ACC_WRITE:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) a.k[v * N + p] = cv[v];
-      break;
-    case EPI_ACC_ADD:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) a.k[v * N + p] = kp[v] + cv[v];
-      break;
-    case EPI_RHS_OUT:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) a.out[v * N + p] = kp[v] + cv[v];
-      break;
-    case EPI_RK4_FIRST:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = kp[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, ops[v]);
-        a.acc[v * N + p] = K;
-      }
-      break;
-    case EPI_RK4_MID:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = kp[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, ops[v]);
-        a.acc[v * N + p] = fma(2.0, K, ops[5 + v]);
-      }
-      break;
-    case EPI_RK4_LAST:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = kp[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, ops[5 + v] + K, ops[v]);
-      }
-      break;
-    case EPI_SSP_1:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = kp[v] + cv[v];
-        a.out[v * N + p] = fma(a.a, K, ops[v]);
-      }
-      break;
-    case EPI_SSP_2:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = kp[v] + cv[v];
-        a.out[v * N + p] = 0.75 * ops[v] + 0.25 * fma(a.a, K, ops[5 + v]);
-      }
-      break;
-    case EPI_SSP_3:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K = kp[v] + cv[v];
-        a.out[v * N + p] = (1.0 / 3.0) * ops[v] + (2.0 / 3.0) * fma(a.a, K, ops[5 + v]);
-      }
-      break;
-    default:
-      break;
-  }
-}
-
-// dir_epilogue_pre32 for two x-adjacent points p and p + 1 (p even), their operands and results
-// moved as 16-byte pairs: kp[v] = (k at p, k at p + 1), ops[j] likewise; the same arithmetic.
-__device__ __forceinline__ void dir_epilogue_pre32x2(const DirArgs& a, long long p, const double c0[5],
-                                                     const double c1[5], const double2* kp, const double2* ops) {
-  const long long N = a.g.N;
-  auto st = [&](double* base, int v, double x0, double x1) {
-    *reinterpret_cast<double2*>(base + v * N + p) = make_double2(x0, x1);
-  };
-  switch (a.epi) {
-    case EPI_ACC_WRITE:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) st(a.k, v, c0[v], c1[v]);
-      break;
-    case EPI_ACC_ADD:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) st(a.k, v, kp[v].x + c0[v], kp[v].y + c1[v]);
-      break;
-    case EPI_RHS_OUT:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) st(a.out, v, kp[v].x + c0[v], kp[v].y + c1[v]);
-      break;
-    case EPI_RK4_FIRST:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K0 = kp[v].x + c0[v], K1 = kp[v].y + c1[v];
-        st(a.out, v, fma(a.a, K0, ops[v].x), fma(a.a, K1, ops[v].y));
-        st(a.acc, v, K0, K1);
-      }
-      break;
-    case EPI_RK4_MID:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K0 = kp[v].x + c0[v], K1 = kp[v].y + c1[v];
-        st(a.out, v, fma(a.a, K0, ops[v].x), fma(a.a, K1, ops[v].y));
-        st(a.acc, v, fma(2.0, K0, ops[5 + v].x), fma(2.0, K1, ops[5 + v].y));
-      }
-      break;
-    case EPI_RK4_LAST:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K0 = kp[v].x + c0[v], K1 = kp[v].y + c1[v];
-        st(a.out, v, fma(a.a, ops[5 + v].x + K0, ops[v].x), fma(a.a, ops[5 + v].y + K1, ops[v].y));
-      }
-      break;
-    case EPI_SSP_1:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K0 = kp[v].x + c0[v], K1 = kp[v].y + c1[v];
-        st(a.out, v, fma(a.a, K0, ops[v].x), fma(a.a, K1, ops[v].y));
-      }
-      break;
-    case EPI_SSP_2:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K0 = kp[v].x + c0[v], K1 = kp[v].y + c1[v];
-        st(a.out, v, 0.75 * ops[v].x + 0.25 * fma(a.a, K0, ops[5 + v].x),
-           0.75 * ops[v].y + 0.25 * fma(a.a, K1, ops[5 + v].y));
-      }
-      break;
-    case EPI_SSP_3:
-#pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double K0 = kp[v].x + c0[v], K1 = kp[v].y + c1[v];
-        st(a.out, v, (1.0 / 3.0) * ops[v].x + (2.0 / 3.0) * fma(a.a, K0, ops[5 + v].x),
-           (1.0 / 3.0) * ops[v].y + (2.0 / 3.0) * fma(a.a, K1, ops[5 + v].y));
-      }
-      break;
-    default:
-      break;
-  }
-}
-
 template <int D>
 __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -260,13 +127,14 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
   float* REC = reinterpret_cast<float*>(smem + OFF_REC);
   double* FD = reinterpret_cast<double*>(smem + OFF_F);
   double* PRE = reinterpret_cast<double*>(smem + OFF_Q);
-  double* PRE2 = reinterpret_cast<double*>(smem + OFF_P2);
 
   constexpr int AX = (D == 0) ? 1 : 0;
   const int nD = a.g.n[D], na = a.g.n[AX];
   const long long N = a.g.N;
   const bool swap = (D == 2 && a.zorder);  // z pass with the line groups first (dir_zorder)
-  const int s0 = (swap ? blockIdx.y : blockIdx.x) * TP;
+  int s0, len;
+  tile_span(1, nD, a.tile_u, a.tile_r, swap ? blockIdx.y : blockIdx.x, s0, len);
+  const int np = len + 6, ni = len + 1, nseg = (ni + SEG - 1) / SEG;  // this tile's positions, interfaces, segments
   const int a0 = (swap ? blockIdx.x : blockIdx.y) * W;
   const int bz = blockIdx.z;
   const int tid = threadIdx.x;
@@ -277,11 +145,11 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
 
   // ---- A: load, convert, primitive variables and point fluxes -------------------------
   int bad = 0;
-  for (int it = tid; it < NP * W; it += THREADS) {
+  for (int it = tid; it < np * W; it += THREADS) {
     int pos, line;
     if (D == 0) {
-      line = it / NP;
-      pos = it - line * NP;
+      line = (int)(((unsigned)it * c_rcp20.v[np]) >> 20);
+      pos = it - line * np;
     } else {
       pos = it / W;
       line = it - pos * W;
@@ -306,15 +174,17 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
     bad |= !(rho > 0.0f && rho < INFINITY && pr > 0.0f && pr < INFINITY);
     const float un = (D == 0) ? vx : (D == 1) ? vy : vz;
     float* q = Q + line * LS + pos;
-    q[0 * W * LS] = rho;
-    q[1 * W * LS] = mx;
-    q[2 * W * LS] = my;
-    q[3 * W * LS] = mz;
-    q[4 * W * LS] = e;
-    q[5 * W * LS] = (D == 0) ? fmaf(mx, un, pr) : mx * un;
-    q[6 * W * LS] = (D == 1) ? fmaf(my, un, pr) : my * un;
-    q[7 * W * LS] = (D == 2) ? fmaf(mz, un, pr) : mz * un;
-    q[8 * W * LS] = ep * un;
+    const float sc[NQ] = {rho, mx, my, mz, e, (D == 0) ? fmaf(mx, un, pr) : mx * un, (D == 1) ? fmaf(my, un, pr) : my * un,
+                          (D == 2) ? fmaf(mz, un, pr) : mz * un, ep * un};
+#pragma unroll
+    for (int m = 0; m < NQ; ++m) q[m * W * LS] = sc[m];
+    // the last segment's points beyond the tile repeat the last one (no difference, no effect on the
+    // segment's choice of arithmetic); their interfaces are never read
+    if (pos == np - 1) {
+      for (int k = 1; k <= nseg * SEG - ni; ++k)
+#pragma unroll
+        for (int m = 0; m < NQ; ++m) q[m * W * LS + k] = sc[m];
+    }
     float sr;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(sr) : "f"(rho));
     R4[line * L4 + pos] = make_float4(sr, vx, vy, vz);
@@ -329,10 +199,10 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
   {
     const float eps4 = a.eps4_hi;
     const bool eps_ok = eps4 >= 1e-9f && eps4 <= 1.0f;  // unscaled products stay in range (see below)
-    for (int it = tid; it < NQ * W * NSEG; it += THREADS) {
-      const int m = it / (W * NSEG);
-      const int rem = it - m * (W * NSEG);
-      const int seg = rem / W, line = rem - seg * W;
+    const unsigned rcp_nseg = c_rcp20.v[nseg];
+    for (int it = tid; it < NQ * W * nseg; it += THREADS) {
+      const int ms = it / W, line = it - ms * W;
+      const int m = (int)(((unsigned)ms * rcp_nseg) >> 20), seg = ms - m * nseg;
       const float* q = Q + (m * W + line) * LS + SEG * seg;
       const float4 qa = *reinterpret_cast<const float4*>(q);
       const float4 qb = *reinterpret_cast<const float4*>(q + 4);
@@ -387,92 +257,65 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
           vR[j] = weno_safe(B[j + 3][2], B[j + 2][1], B[j + 1][0], eL, T3[j + 2], T2[j + 1]);
         }
       }
-      float* r = REC + line * NI + SEG * seg;
+      float* r = REC + line * RS + SEG * seg;
       if (m < 5) {
-        *reinterpret_cast<float4*>(r + m * W * NI) =
+        *reinterpret_cast<float4*>(r + m * W * RS) =
             make_float4(vR[0] - vL[0], vR[1] - vL[1], vR[2] - vL[2], vR[3] - vL[3]);
         if (m == 1 + D)
-          *reinterpret_cast<float4*>(r + 5 * W * NI) =
+          *reinterpret_cast<float4*>(r + 5 * W * RS) =
               make_float4(vL[0] + vR[0], vL[1] + vR[1], vL[2] + vR[2], vL[3] + vR[3]);
       } else {
-        *reinterpret_cast<float4*>(r + (m + 1) * W * NI) =
+        *reinterpret_cast<float4*>(r + (m + 1) * W * RS) =
             make_float4(vL[0] + vR[0], vL[1] + vR[1], vL[2] + vR[2], vL[3] + vR[3]);
       }
     }
   }
   __syncthreads();
 
-  // ---- epilogue operand k: fetched asynchronously into the dead scalar planes while D runs;
-  //      each thread later reads only its own point's slots
+  // ---- epilogue operands: fetched asynchronously into the dead scalar planes and behind them while D
+  //      runs.  y and z passes on grids with nx even take two x-adjacent points (lines 2j, 2j+1 of the
+  //      tile; their flat index is even) per 16-byte copy.  U_n and the stage input may be the
+  //      caller's and only 8-byte aligned; the rest is the library's.
+  const bool pairs = D != 0 && (a.g.n[0] & 1) == 0 && (((uintptr_t)a.un | (uintptr_t)a.u) & 15) == 0;
   auto point_of = [&](int it, int& pp, int& line) {
     if (D == 0) {
-      line = it / TP;
-      pp = it - line * TP;
+      line = (int)(((unsigned)it * c_rcp20.v[len]) >> 20);
+      pp = it - line * len;
     } else {
       pp = it / W;
       line = it - pp * W;
     }
   };
-  const int nops = epilogue_operands(a.epi);  // k, then U_n, then acc or the stage input
-  // y and z passes on grids with nx even: a thread owns two x-adjacent points (lines 2j, 2j+1 of
-  // the tile; their flat index is even, so every operand pair is 16-byte aligned)
-  const bool pairs = (D != 0) && ((a.g.n[0] & 1) == 0);
-  const double* third = (a.epi == EPI_SSP_2 || a.epi == EPI_SSP_3) ? a.u : a.acc;
   if (pairs) {
-    if (nops > 0 && tid < TP * W / 2) {
+    if (tid < len * W / 2) {
       const int pp = tid / (W / 2), l0 = 2 * (tid - pp * (W / 2));
-      if (s0 + pp < nD && a0 + l0 < na) {  // na = nx is even: the second point exists too
-        const long long p = tile_flat<D>(a.g, s0 + pp, a0 + l0, bz);
-        double2* kp = reinterpret_cast<double2*>(PRE) + 5 * tid;
-        double2* op = reinterpret_cast<double2*>(PRE2) + 10 * tid;
-#pragma unroll
-        for (int v = 0; v < 5; ++v) cp_async16(kp + v, a.k + v * N + p);
-        if (nops >= 10) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) cp_async16(op + v, a.un + v * N + p);
-        }
-        if (nops == 15) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) cp_async16(op + 5 + v, third + v * N + p);
-        }
-      }
+      if (a0 + l0 < na)  // na = nx is even: the second point exists too
+        epilogue_prefetch<true, TS>(a, tile_flat<D>(a.g, s0 + pp, a0 + l0, bz), PRE + 2 * tid);
     }
-  } else if (nops > 0 && tid < TP * W) {
+  } else if (tid < len * W) {
     int pp, line;
     point_of(tid, pp, line);
-    if (s0 + pp < nD && a0 + line < na) {
-      const long long p = tile_flat<D>(a.g, s0 + pp, a0 + line, bz);
-#pragma unroll
-      for (int v = 0; v < 5; ++v) cp_async8(PRE + 5 * tid + v, a.k + v * N + p);
-      if (nops >= 10) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) cp_async8(PRE2 + 10 * tid + v, a.un + v * N + p);
-      }
-      if (nops == 15) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) cp_async8(PRE2 + 10 * tid + 5 + v, third + v * N + p);
-      }
-    }
+    if (a0 + line < na) epilogue_prefetch<false, TS>(a, tile_flat<D>(a.g, s0 + pp, a0 + line, bz), PRE + tid);
   }
   cp_async_commit();
 
   // ---- D: Roe flux + viscous interface flux, / dx, widened to FP64 ----------------------
-  if (tid < NI * W) {
+  if (tid < ni * W) {
     int r, line;
     if (D == 0) {
-      line = tid / NI;
-      r = tid - line * NI;
+      line = (int)(((unsigned)tid * c_rcp20.v[ni]) >> 20);
+      r = tid - line * ni;
     } else {
       r = tid / W;
       line = tid - r * W;
     }
     // interface r lies between the tile's points r - 1 and r, i.e. positions r + 2 and r + 3
-    const float* rc_ = REC + line * NI + r;
+    const float* rc_ = REC + line * RS + r;
     float du[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) du[v] = rc_[v * W * NI];
-    const float S0 = rc_[5 * W * NI];
-    const float S1 = rc_[6 * W * NI], S2 = rc_[7 * W * NI], S3 = rc_[8 * W * NI], S4 = rc_[9 * W * NI];
+    for (int v = 0; v < 5; ++v) du[v] = rc_[v * W * RS];
+    const float S0 = rc_[5 * W * RS];
+    const float S1 = rc_[6 * W * RS], S2 = rc_[7 * W * RS], S3 = rc_[8 * W * RS], S4 = rc_[9 * W * RS];
     const float4 qa = R4[line * L4 + r + 2], qb = R4[line * L4 + r + 3];
     const float Ha = HS[line * L4 + r + 2], Hb = HS[line * L4 + r + 3];
     const float rs = rcp_a(qa.x + qb.x);
@@ -538,33 +381,17 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
   cp_async_wait_all();
   __syncthreads();
 
-  // ---- E: FP64 conservative difference + epilogue ----------------------------------------
-  if (pairs) {
-    if (tid < TP * W / 2) {
-      const int pp = tid / (W / 2), l0 = 2 * (tid - pp * (W / 2));
-      if (s0 + pp < nD && a0 + l0 < na) {
-        const double* f0 = FD + l0 * FS + pp;
-        const double* f1 = f0 + FS;
-        double c0[5], c1[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          c0[v] = f0[v * W * FS] - f0[v * W * FS + 1];
-          c1[v] = f1[v * W * FS] - f1[v * W * FS + 1];
-        }
-        dir_epilogue_pre32x2(a, tile_flat<D>(a.g, s0 + pp, a0 + l0, bz), c0, c1,
-                             reinterpret_cast<const double2*>(PRE) + 5 * tid,
-                             reinterpret_cast<const double2*>(PRE2) + 10 * tid);
-      }
-    }
-  } else if (tid < TP * W) {
+  // ---- E: FP64 difference + epilogue, one point per thread (the FP64 work then spreads over
+  //      seven warps; two points per thread left it on four.  512^3 y pass 6.85 -> 6.23 ms)
+  if (tid < len * W) {
     int pp, line;
     point_of(tid, pp, line);
-    if (s0 + pp < nD && a0 + line < na) {
+    if (a0 + line < na) {
       const double* fd = FD + line * FS + pp;
       double cv[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) cv[v] = fd[v * W * FS] - fd[v * W * FS + 1];
-      dir_epilogue_pre32(a, tile_flat<D>(a.g, s0 + pp, a0 + line, bz), cv, PRE + 5 * tid, PRE2 + 10 * tid);
+      dir_epilogue_pre<TS>(a, tile_flat<D>(a.g, s0 + pp, a0 + line, bz), cv, PRE + tid);
     }
   }
 }
@@ -573,13 +400,16 @@ template <int D>
 cudaError_t launch32(const DirArgs& a, cudaStream_t s) {
   constexpr int AX = (D == 0) ? 1 : 0;
   constexpr int BX = (D == 2) ? 1 : 2;
-  dim3 grid((a.g.n[D] + TP - 1) / TP, (a.g.n[AX] + W - 1) / W, a.g.n[BX]);
+  constexpr int TM = tile_max(D);
+  dim3 grid((a.g.n[D] + TM - 1) / TM, (a.g.n[AX] + W - 1) / W, a.g.n[BX]);
   if (D == 2 && a.zorder) {
     const unsigned t = grid.x;
     grid.x = grid.y;
     grid.y = t;
   }
-  k_dir32<D><<<grid, THREADS, BYTES, s>>>(a);
+  DirArgs r = a;
+  tile_split_units(1, a.g.n[D], (a.g.n[D] + TM - 1) / TM, r.tile_u, r.tile_r);  // units of one point
+  k_dir32<D><<<grid, THREADS, BYTES, s>>>(r);
   return cudaGetLastError();
 }
 
@@ -600,7 +430,7 @@ cudaError_t prepare_dir32_kernels() {
   return e;
 }
 
-// One tile shape (27 x 8) for every pass; the tile variants of the FP64 modes do not apply.
+// One tile shape for every pass; the tile variants of the FP64 modes do not apply.
 cudaError_t launch_dir32(int d, const DirArgs& a, cudaStream_t s) {
   if (d == 0) return launch32<0>(a, s);
   if (d == 1) return launch32<1>(a, s);

@@ -168,9 +168,10 @@ __device__ __forceinline__ float d2f_trunc_fast(double x) {
   return __uint_as_float(b | (h & 0x80000000u));
 }
 
+// Five CTAs per SM (48 registers) instead of four: 512^3 2.69 -> 2.51 ms; six spill (step 2.3 % slower).
 constexpr int V32_SMEM = VT_RING * VT_PLANE * (int)sizeof(float4);  // 34,560 bytes
 
-__global__ void __launch_bounds__(VT_X * VT_Y, 4) k_visc32t(const double* __restrict__ u, float* __restrict__ fv,
+__global__ void __launch_bounds__(VT_X * VT_Y, 5) k_visc32t(const double* __restrict__ u, float* __restrict__ fv,
                                                              const Grid g, float gamma, float mu, float kappa,
                                                              int only_d, int cz) {
   extern __shared__ float4 ring4[];  // [VT_RING][VT_HY][VT_HX]: u, v, w, T
@@ -511,7 +512,7 @@ cudaError_t prepare_visc_kernels() {
 
 cudaError_t launch_visc32(const Grid& g, const double* u, float* fv, double gamma, double mu, double kappa,
                           cudaStream_t s, int only_d) {
-  const int cz = visc_chunk(g, g.n[2], 4 * 152);
+  const int cz = visc_chunk(g, g.n[2], 5 * 152);
   const dim3 grid((g.n[0] + VT_X - 1) / VT_X, (g.n[1] + VT_Y - 1) / VT_Y, (g.n[2] + cz - 1) / cz);
   k_visc32t<<<grid, VT_X * VT_Y, V32_SMEM, s>>>(u, fv, g, (float)gamma, (float)mu, (float)kappa, only_d, cz);
   return cudaGetLastError();

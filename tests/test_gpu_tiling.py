@@ -99,8 +99,9 @@ def test_balanced_tiles(ns3d, orc, nx, ny, nz):
 
 
 
+@pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("nx", [24, 26, 27])
-def test_step_of_a_state_on_8_byte_boundaries(ns3d, nx):
+def test_step_of_a_state_on_8_byte_boundaries(ns3d, nx, prec):
     """The z pass takes 16-byte copies only where U_n allows it: the same bits either way."""
     import torch
     u = _gpu(I.random_smooth(nx, 10, 30, seed=8, amp=0.1, mach=0.4))
@@ -108,7 +109,7 @@ def test_step_of_a_state_on_8_byte_boundaries(ns3d, nx):
     v = buf[1:].view(u.shape)
     v.copy_(u)
     assert v.data_ptr() % 16 == 8
-    s = ns3d.Solver(nx, 10, 30, mu_eff=0.003)
+    s = ns3d.Solver(nx, 10, 30, mu_eff=0.003, precision=prec)
     s.rk_step(u, 0.01, 2)
     s.rk_step(v, 0.01, 2)
     s.check()
@@ -149,3 +150,16 @@ def test_merged_xy_passes_give_the_same_bits(ns3d, prec, rk, nx, ny, nz):
         s.close()
     for r, v in out[1:]:
         assert torch.equal(r, out[0][0]) and torch.equal(v, out[0][1])
+
+
+# FP32-bulk tiles: lines of one and two tiles, lengths whose last segment of four interfaces is partial
+@pytest.mark.parametrize("nx,ny,nz", [(27, 26, 28), (53, 29, 3), (1, 55, 27), (30, 2, 79)])
+def test_balanced_tiles_fp32_bulk(ns3d, orc, nx, ny, nz):
+    u = I.random_smooth(nx, ny, nz, seed=11, amp=0.1, mach=0.5)
+    ref = orc.rhs(orc.Params(nx, ny, nz, mu_eff=0.003), u)
+    s = ns3d.Solver(nx, ny, nz, mu_eff=0.003, precision=1)
+    r = s.rhs(_gpu(u)).cpu().numpy()
+    s.check()
+    s.close()
+    # FP32 fluxes: 1e-5 of the flux scale over the smallest spacing (as the FP32-bulk tests)
+    assert np.abs(r - ref).max() <= 1e-5 * flux_scale(u, (2 * np.pi,) * 3)
