@@ -42,12 +42,12 @@ RK_STAGES = 4
 # one direction pass, counted from each formulation without the halo's share:
 #  NS3D_FP64 (double-float weights, offsets, interface jumps and sums, Roe dissipation and
 #   viscous divergence): point fluxes 5, first differences 9, per flux component the interface
-#   flux P_i/dx + (t - diss)/(2 dx) 2 x 5, flux difference 5, adding the double-float viscous
-#   divergence 2 x 4.
+#   flux 2 P_i + (t - diss) 2 x 5, flux difference 5, its scaling and the double-float viscous
+#   divergence 1 + 2 x 4.
 #  NS3D_FP64_STRICT: point fluxes 5, windows (differences, indicators, their products) 9 x 16,
 #   interfaces (two offsets with their cubic reciprocals, jump, sum) 5 x 22 + 4 x 25 + 6 = 9 x 24,
 #   Roe flux 73, difference and viscous divergence 21.
-OPS_DIR_FP64 = 5 + 9 + 10 + 5 + 8
+OPS_DIR_FP64 = 5 + 9 + 10 + 5 + 9
 OPS_DIR_STRICT = 5 + 9 * 16 + 9 * 24 + 73 + 21
 OPS_RK_EPI = 15            # RK4 stage update in the z pass (5 components x 3)
 # The method's FP64 flops per point and pass (FMA = 2) in its all-FP64 form, for context.
