@@ -569,7 +569,7 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
         // Phase E divides the difference by 2 dx in FP64.  Formed in double-float here, (t - diss)/(2 dx)
         // rounded at 2^-48 of a jump: mean error of 48 shock-tube right-hand sides 1.311e-14, now
         // 1.288e-14 (1.296e-14 with the sums in FP64), for one FP64 operation more per point (128^3
-        // step 5.73 -> 5.80 ms)
+        // step 5.73 -> 5.77 ms)
         const float2* rf = reinterpret_cast<const float2*>(r);
         auto ldr = [&](int k, int sp) { const float2 v = rf[k * NR * W + sp]; return df{v.x, v.y}; };
         const float2* rj = reinterpret_cast<const float2*>(rec);
@@ -711,11 +711,12 @@ __device__ __forceinline__ void dir_tile(const DirArgs& a, double* sm, int s0, i
       if (MODE == 1) {  // twice the interface fluxes; viscous fluxes double-float
         const double hr = a.g.hrh[D];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-          cv[v] = F[v * NI * W + om] - F[v * NI * W + op];
-          if (v == 0 || a.fv == nullptr) cv[v] *= hr;
-        }
-        if (a.fv != nullptr) {
+        for (int v = 0; v < 5; ++v) cv[v] = F[v * NI * W + om] - F[v * NI * W + op];
+        cv[0] *= hr;
+        if (a.fv == nullptr) {
+#pragma unroll
+          for (int v = 1; v < 5; ++v) cv[v] *= hr;
+        } else {
           const df r12d = d2df_bits(r12);
 #pragma unroll
           for (int cc = 0; cc < 4; ++cc) {
