@@ -154,13 +154,28 @@ __device__ __forceinline__ df2 df2_sixth() {
   return df2_splat(df{hi, lo});
 }
 
+// Exponent of the power of two that the rescaling of df2_offset3 divides by, and the cut it applies
+// to the rescaled B_k (2 at most; they are normalised to rounding, so lo drops out with hi).
+__device__ __forceinline__ int offset_scale_exponent(float B1, float B2, float B3) {
+  const int e1 = exponent_of(B1), e2 = exponent_of(B2), e3 = exponent_of(B3);
+  return min(min(max(e1, max(e2, e3)), min(e1, min(e2, e3)) + 96), 126);
+}
+__device__ __forceinline__ df2 df2_cut2(df2 x) {
+  const bool c0 = !(x.hi.x < 2.0f), c1 = !(x.hi.y < 2.0f);
+  return df2{make_float2(c0 ? 2.0f : x.hi.x, c1 ? 2.0f : x.hi.y), make_float2(c0 ? 0.0f : x.lo.x, c1 ? 0.0f : x.lo.y)};
+}
+
 // Offset omega_1 (F_1 - F_2) + omega_3 (F_3 - F_2) of one reconstruction from its candidate 2, in
 // double-float, from the three squared scaled indicators B_k (candidate order 1, 2, 3) and the third
 // differences ta = 3 (F_1 - F_2), tb = 6 (F_3 - F_2), both given divided by 6; with
 // omega_k = c_k prod_{m!=k} B_m / den and den = B2 B3 + 6 B1 B3 + 3 B1 B2,
 //   d = B2 [2 B3 ta/6 + 3 B1 tb/6] / [B2 B3 + 3 B1 (2 B3 + B2)]        (one division).
-// SCALE: rescale the B_k by a common power of two first (the weights are scale-free);
-// without it every B_k must lie in [DFB_LO^2, DFB_HI^2).
+// SCALE: rescale the B_k by a common power of two first (the weights are scale-free), the largest
+// to [1, 2); without it every B_k must lie in [DFB_LO^2, DFB_HI^2).  den is at least the product of
+// the two largest B_k.  Next to constant data two of them are (4 eps)^2 and the third goes with the
+// fourth power of the jump, so a B_k more than 2^96 above the smallest is cut to that ratio: den then
+// stays above 2^-96, with its error terms normal floats.  The weight of such a window is below 2^-95
+// either way, far under the rounding of the largest difference.
 // The numerator and denominator are renormalised and the division's seed refined (8 of the 71 packed
 // operations): at a jump the offsets are a third of it, and their rounding is what is left of the
 // reconstruction's error there.  In units of 2^-48 of the largest difference, against long double:
@@ -171,12 +186,12 @@ __device__ __forceinline__ df2 df2_sixth() {
 template <bool SCALE = true>
 __device__ __forceinline__ df2 df2_offset3(df2 B1, df2 B2, df2 B3, df2 ta6, df2 tb6) {
   if (SCALE) {
-    const int E0 = max(exponent_of(B1.hi.x), max(exponent_of(B2.hi.x), exponent_of(B3.hi.x)));
-    const int E1 = max(exponent_of(B1.hi.y), max(exponent_of(B2.hi.y), exponent_of(B3.hi.y)));
+    const int E0 = offset_scale_exponent(B1.hi.x, B2.hi.x, B3.hi.x);
+    const int E1 = offset_scale_exponent(B1.hi.y, B2.hi.y, B3.hi.y);
     const float2 sc = make_float2(pow2f(-E0), pow2f(-E1));
-    B1 = df2_scale(B1, sc);
-    B2 = df2_scale(B2, sc);
-    B3 = df2_scale(B3, sc);
+    B1 = df2_cut2(df2_scale(B1, sc));
+    B2 = df2_cut2(df2_scale(B2, sc));
+    B3 = df2_cut2(df2_scale(B3, sc));
   }
   const df2 b1 = df2_mul_f_u(B1, 3.0f), b3 = df2_twice(B3);
   const df2 den = df2_add_pos_u(df2_mul_u(B2, B3), df2_mul_u(b1, df2_add_pos_u(b3, B2)));

@@ -370,6 +370,33 @@ def test_double_float_range_is_reported(ns3d):
     assert bool(np.isfinite(r.cpu().numpy()).all())
 
 
+# jumps next to exactly constant data, where two smoothness indicators keep the value 4 eps and the
+# third grows with the square of the jump; ERANGE is allowed from differences of ~1e9 of the data (the
+# energy flux differs by ~3 times the pressure jump)
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("eps,jump", [(1e-6, 1e5), (1e-6, 3e6), (1e-6, 1e7), (1e-6, 1e8), (1e-15, 1e3), (1e-15, 1e7)])
+def test_jump_next_to_constant_data(ns3d, axis, eps, jump):
+    shp = [6, 6, 6]
+    shp[axis] = 30
+    p = np.ones(30)
+    p[8:18] += jump
+    p = p[tuple(slice(None) if k == axis else None for k in range(3))] * np.ones(shp)
+    u = _gpu(I.to_conserved(np.ones(shp), *(np.full(shp, 0.3 * (m + 1)) for m in range(3)), p))
+    strict = ns3d.Solver(*shp[::-1], precision=ns3d.NS3D_FP64_STRICT, weno_eps=eps)
+    ref = strict.rhs(u).cpu().numpy()
+    strict.check()
+    strict.close()
+    s = ns3d.Solver(*shp[::-1], weno_eps=eps)
+    got = s.rhs(u).cpu().numpy()
+    try:
+        s.check()
+    except ns3d.Ns3dError as e:
+        assert e.code == ns3d.NS3D_ERANGE and jump >= 1e8
+    else:
+        assert rel_err(got, ref) <= RHS_TOL
+    s.close()
+
+
 def test_zero_steps_is_identity(ns3d):
     u0 = I.taylor_green(8)
     s = ns3d.Solver(8, 8, 8)
