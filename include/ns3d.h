@@ -55,7 +55,7 @@ enum {
                               returns it: no kernel of the library spins on a flag (the
                               persistent ensemble kernel separates its phases with the grid
                               barriers of a cooperative launch, whose CTAs are co-resident) */
-  NS3D_ERANGE = -6         /* data beyond the range of the double-float WENO weights
+  NS3D_ERANGE = -6         /* data beyond the range of the FP32 or double-float WENO weights
                               (differences of the data above ~1e9): use NS3D_FP64_STRICT */
 };
 

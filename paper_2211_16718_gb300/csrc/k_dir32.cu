@@ -103,14 +103,18 @@ __device__ __forceinline__ float weno_fast(float B1, float B2, float B3, float c
   return fmaf(num, rcp_a(den), c);
 }
 
-// The same with the indicators rescaled by their common power of two and an IEEE division: any
-// data whose indicators are finite.
-__device__ __forceinline__ float weno_safe(float B1, float B2, float B3, float c, float d1, float d3x3) {
-  const int E = max(exponent_of(B1), max(exponent_of(B2), exponent_of(B3)));
-  const float sc = pow2f(max(-E, -126));
-  B1 *= sc;
-  B2 *= sc;
-  B3 *= sc;
+// The same for any data whose squared indicators are finite (differences up to ~1e9; else bit 1 of
+// bad is set): the B_k rescaled by a common power of two, the largest to [1, 2), and an IEEE
+// division.  A B_k more than 2^96 above the smallest is cut to that ratio (constant data next to a
+// large jump), so that den, at least the product of the two largest, stays a normal float.
+__device__ __forceinline__ float weno_safe(float B1, float B2, float B3, float c, float d1, float d3x3, int& bad) {
+  const int e1 = exponent_of(B1), e2 = exponent_of(B2), e3 = exponent_of(B3);
+  const int top = max(e1, max(e2, e3));
+  bad |= (top >= 128) ? 2 : 0;
+  const float sc = pow2f(-min(min(top, min(e1, min(e2, e3)) + 96), 126));
+  B1 = fminf(B1 * sc, 2.0f);
+  B2 = fminf(B2 * sc, 2.0f);
+  B3 = fminf(B3 * sc, 2.0f);
   const float p23 = B2 * B3, p12 = B1 * B2;
   const float den = fmaf(6.0f * B1, B3, fmaf(3.0f, p12, p23));
   const float num = fmaf(p23, d1, p12 * d3x3);
@@ -144,7 +148,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
   const float gm1 = a.gm1_hi;
 
   // ---- A: load, convert, primitive variables and point fluxes -------------------------
-  int bad = 0;
+  int bad = 0;  // bit 0: non-physical, bit 1: differences beyond the indicators' range
   for (int it = tid; it < np * W; it += THREADS) {
     int pos, line;
     if (D == 0) {
@@ -253,8 +257,8 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
           vL[j] = weno_fast(B[j][0], B[j + 1][1], B[j + 2][2], eR, -T3[j], -T2[j + 1]);
           vR[j] = weno_fast(B[j + 3][2], B[j + 2][1], B[j + 1][0], eL, T3[j + 2], T2[j + 1]);
         } else {
-          vL[j] = weno_safe(B[j][0], B[j + 1][1], B[j + 2][2], eR, -T3[j], -T2[j + 1]);
-          vR[j] = weno_safe(B[j + 3][2], B[j + 2][1], B[j + 1][0], eL, T3[j + 2], T2[j + 1]);
+          vL[j] = weno_safe(B[j][0], B[j + 1][1], B[j + 2][2], eR, -T3[j], -T2[j + 1], bad);
+          vR[j] = weno_safe(B[j + 3][2], B[j + 2][1], B[j + 1][0], eL, T3[j + 2], T2[j + 1], bad);
         }
       }
       float* r = REC + line * RS + SEG * seg;
@@ -377,7 +381,10 @@ __global__ void __launch_bounds__(THREADS, 4) k_dir32(const DirArgs a) {
     fd[3 * W * FS] = f2d_bits(F3 * rdx);
     fd[4 * W * FS] = f2d_bits(F4 * rdx);
   }
-  if (__any_sync(0xffffffffu, bad) && (tid & 31) == 0) atomicOr(a.status, ST_NONPHYS);
+  if (__any_sync(0xffffffffu, bad)) {
+    const int any = __reduce_or_sync(0xffffffffu, bad);
+    if ((tid & 31) == 0) atomicOr(a.status, ((any & 1) ? ST_NONPHYS : 0) | ((any & 2) ? ST_DF_RANGE : 0));
+  }
   cp_async_wait_all();
   __syncthreads();
 

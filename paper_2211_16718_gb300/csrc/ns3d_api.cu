@@ -275,7 +275,7 @@ const char* ns3d_strerror(int code) {
     case NS3D_ECUDA: return "CUDA error";
     case NS3D_ENONPHYSICAL: return "non-physical state (rho <= 0, p <= 0, or non-finite value)";
     case NS3D_ETIMEOUT: return "device-side wait timed out (reserved: no call returns it)";
-    case NS3D_ERANGE: return "data beyond the range of the double-float WENO weights (use NS3D_FP64_STRICT)";
+    case NS3D_ERANGE: return "data beyond the range of the FP32 or double-float WENO weights (use NS3D_FP64_STRICT)";
     default: return "unknown error";
   }
 }

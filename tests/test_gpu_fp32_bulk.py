@@ -156,3 +156,35 @@ def test_fp32_bulk_hit256_sampled_points(ns3d, orc):
     r64 = orc.rhs_points(orc.Params(n, n, n, mu_eff=mu), u, idx).T
     err = np.abs(r32 - r64).max() / flux_scale(u, (2 * math.pi,) * 3)
     assert err <= FLUX_TOL, err
+
+
+# jumps next to exactly constant data, where two smoothness indicators keep the value 4 eps and the
+# third grows with the square of the jump; the energy flux differs by ~3 times the pressure jump
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("eps,jump", [(1e-6, 1e6), (1e-6, 1e8), (1e-15, 1e5), (1e-15, 1e8), (1e-6, 1e10)])
+def test_fp32_bulk_jump_next_to_constant_data(ns3d, axis, eps, jump):
+    shp = [6, 6, 6]
+    shp[axis] = 61  # three tiles along every axis
+    p = np.ones(61)
+    p[8:28] += jump
+    p = p[tuple(slice(None) if k == axis else None for k in range(3))] * np.ones(shp)
+    u0 = I.to_conserved(np.ones(shp), *(np.full(shp, 0.3 * (m + 1)) for m in range(3)), p)
+    u = _gpu(u0)
+    s = ns3d.Solver(*shp[::-1], precision=ns3d.NS3D_FP32_BULK, weno_eps=eps)
+    got = s.rhs(u).cpu().numpy()
+    if jump > 1e9:
+        with pytest.raises(ns3d.Ns3dError) as ei:
+            s.check()
+        assert ei.value.code == ns3d.NS3D_ERANGE
+        s.close()
+        return
+    s.check()
+    s.close()
+    strict = ns3d.Solver(*shp[::-1], precision=ns3d.NS3D_FP64_STRICT, weno_eps=eps)
+    ref = strict.rhs(u).cpu().numpy()
+    strict.check()
+    strict.close()
+    # the interface flux at such a jump is its dissipation, of up to (|u| + c) max|U| (10 to 1e4 times
+    # the flux of the points), so its rounding is that much larger: the bound relative to it
+    scale = (0.9 + math.sqrt(1.4 * (1.0 + jump))) * np.abs(u0).max() / (2 * math.pi / 61)
+    assert np.abs(got - ref).max() <= FLUX_TOL * scale
