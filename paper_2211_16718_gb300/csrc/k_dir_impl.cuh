@@ -121,10 +121,12 @@ __host__ __device__ constexpr int scalar_of(int c) {
   return (c == 1 + D) ? 4 : (c == 1 + T1) ? 1 : (c == 1 + T2) ? 2 : 3;
 }
 
-// FP64 reciprocal and reciprocal square root from the special-function unit's approximations (PTX
-// rcp / rsqrt.approx.ftz.f64, about 20 correct bits) and one cubic correction: three and five FP64
-// operations where the IEEE division and square root take nine and ten, error below 1 ulp.
-// Reciprocals of magnitudes outside [2^-1021, 2^1020) and of non-finite values are IEEE divisions.
+// FP64 reciprocal and reciprocal square root: the special-function unit's approximation (PTX
+// rcp / rsqrt.approx.ftz.f64) and one third-order Householder correction, that is the series of 1/x in
+// e = 1 - x r (r + r e + r e^2) or of x^(-1/2) in e = 1 - x r^2 (r + r e/2 + 3 r e^2/8) cut before e^3.
+// Three and five FP64 operations.  The first rounds once at full size (error below 0.6 ulp), the second
+// also in x r (below 1.1 ulp).  What the approximations flush or overflow on (rcp: magnitudes outside
+// [2^-1021, 2^1020); rsqrt: subnormals), zeros and non-finite values take the IEEE operations.
 __device__ __forceinline__ double rcp_cubic(double x) {
   const uint32_t e11 = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
   if (e11 - 2u >= 2041u) return 1.0 / x;
@@ -134,6 +136,8 @@ __device__ __forceinline__ double rcp_cubic(double x) {
   return fma(r, fma(e, e, e), r);
 }
 __device__ __forceinline__ double rsqrt_cubic(double x) {
+  const uint32_t e11 = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
+  if (e11 - 1u >= 2046u) return 1.0 / sqrt(x);
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   const double e = fma(-x * r, r, 1.0);

@@ -131,6 +131,31 @@ __global__ void k_check(int n, uint64_t seed, int* bad) {
     if (!same(df2_lane0(r2[o]), r[0][o]) || !same(df2_lane1(r2[o]), r[1][o])) atomicAdd(&bad[o], 1);
 }
 
+// rcp_cubic (what = 0) and rsqrt_cubic (1) at the positive doubles of biased exponent
+// e11 = blockIdx.x and a pseudo-random mantissa per thread (thread 0: zero, so 0, powers of two and
+// infinity; thread 1: all ones): where both operand and IEEE result are normal, the error in ulps of
+// the result into *ulp (as an integer of 1e-6 ulp); elsewhere the bits of the IEEE operations, counted
+// in *bad where they differ.
+__global__ void k_check_cubic(int what, uint64_t seed, int* ulp, int* bad) {
+  const uint64_t key = seed + blockIdx.x * 4096ull + threadIdx.x;
+  const uint64_t m = threadIdx.x == 0 ? 0 : threadIdx.x == 1 ? 0xfffffffffffffull : mix64(key) >> 12;
+  const double x = __longlong_as_double(((long long)blockIdx.x << 52) | (long long)m);
+  const double r = what ? rsqrt_cubic(x) : rcp_cubic(x);
+  const double ref = what ? 1.0 / sqrt(x) : 1.0 / x;
+  const int er = (int)((__double_as_longlong(ref) >> 52) & 0x7ff);
+  if (blockIdx.x == 0 || blockIdx.x == 0x7ff || er == 0 || er == 0x7ff) {
+    if (!(r == ref || (isnan(r) && isnan(ref)))) atomicAdd(bad, 1);
+    return;
+  }
+  // relative error: 1 - x r exactly; (1 - x r^2)/2 with x r as a sum of two doubles
+  const double p = x * r, pe = fma(x, r, -p);
+  const double rel = what ? 0.5 * fma(-pe, r, fma(-p, r, 1.0)) : fma(-x, r, 1.0);
+  const double mant = __longlong_as_double((__double_as_longlong(ref) & 0xfffffffffffffll) | (1023ll << 52));
+  const double err = fabs(rel) * mant * 0x1p52 * 1e6;
+  if (!(err < 2e9)) atomicAdd(bad, 1);
+  else atomicMax(ulp, (int)err);
+}
+
 }  // namespace
 
 // Runs n lane pairs; bad_host receives NOPS mismatch counts (add_fast, sub, mul_u, mul, sqr_u,
@@ -149,3 +174,20 @@ extern "C" int df2_check(int n, unsigned long long seed, int* bad_host) {
 }
 
 extern "C" int df2_check_nops() { return NOPS; }
+
+// Largest error (1e-6 ulp) of rcp_cubic (what = 0) or rsqrt_cubic (1) over all exponents, and the number
+// of wrong special values.  Returns a cudaError_t.
+extern "C" int cubic_check(int what, unsigned long long seed, int* ulp_host, int* bad_host) {
+  int* d = nullptr;
+  cudaError_t e = cudaMalloc(&d, 2 * sizeof(int));
+  if (e != cudaSuccess) return (int)e;
+  cudaMemset(d, 0, 2 * sizeof(int));
+  k_check_cubic<<<2048, 1024>>>(what, seed, d, d + 1);
+  e = cudaGetLastError();
+  int h[2] = {0, 0};
+  if (e == cudaSuccess) e = cudaMemcpy(h, d, sizeof(h), cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  *ulp_host = h[0];
+  *bad_host = h[1];
+  return (int)e;
+}

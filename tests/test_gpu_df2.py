@@ -41,3 +41,17 @@ def test_two_lane_double_float_equals_scalar_bitwise(checker, seed):
     assert checker.df2_check(1 << 20, seed, bad) == 0
     mismatches = {n: bad[i] for i, n in enumerate(NAMES) if bad[i]}
     assert not mismatches, mismatches
+
+
+# bounds: the final rounding (0.5 ulp) and the seed's error cubed (it is below 2^-18, so 0.13 ulp at
+# most), and for the root half of the rounding of x r (0.5 ulp)
+@pytest.mark.gpu
+@pytest.mark.parametrize("what,bound", [(0, 0.6), (1, 1.1)])
+def test_cubic_reciprocals_of_the_all_fp64_mode(checker, what, bound):
+    """rcp_cubic and rsqrt_cubic (csrc/k_dir_impl.cuh) over every exponent: the error in ulps, and
+    the IEEE results for zero, subnormal, overflowing and infinite operands and for NaN."""
+    ulp, bad = ctypes.c_int(), ctypes.c_int()
+    for seed in (1, 20261205):
+        assert checker.cubic_check(what, ctypes.c_ulonglong(seed), ctypes.byref(ulp), ctypes.byref(bad)) == 0
+        assert bad.value == 0
+        assert ulp.value * 1e-6 <= bound

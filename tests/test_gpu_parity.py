@@ -397,6 +397,24 @@ def test_jump_next_to_constant_data(ns3d, axis, eps, jump):
     s.close()
 
 
+def test_strict_at_a_subnormal_squared_sound_speed(ns3d, orc):
+    """c^2 of about 1.3e-308 (a dense cold gas at rest): the all-FP64 mode's reciprocal root must not
+    flush it."""
+    n = (16, 7, 6)
+    shp = n[::-1]
+    # rough: the largest part of the result is the mass equation's, the jumps of the pressure alone.  On
+    # a wave (0.1 sin x: jumps of 3e-5 p) the rounding of p, a few 2^-53, is 1e-11 of it
+    p = 0.9e-158 * (1.0 + 0.1 * np.random.default_rng(2).uniform(-1.0, 1.0, shp))
+    zero = np.zeros(shp)
+    u = I.to_conserved(np.full(shp, 1e150), zero, zero, zero, p)
+    s = ns3d.Solver(*n, precision=ns3d.NS3D_FP64_STRICT)
+    got = s.rhs(_gpu(u)).cpu().numpy()
+    s.check()
+    s.close()
+    # c^2 has 51 bits left
+    assert rel_err(got, orc.rhs(orc.Params(*n), u)) <= RHS_TOL
+
+
 def test_zero_steps_is_identity(ns3d):
     u0 = I.taylor_green(8)
     s = ns3d.Solver(8, 8, 8)
