@@ -355,12 +355,17 @@ enum {
 };
 
 /* on != 0: record CUDA events around every kernel launch of ctx (on its stream)
- * and accumulate their durations; on == 0 stops recording.  Resets counters. */
+ * and accumulate their durations; on == 0 stops recording.  Resets counters.
+ * The x and y passes, which share one launch on grids of up to 2^20 points (not in
+ * NS3D_FP32_BULK contexts, with viscous lean storage or in the slab-wise stages of
+ * ns3d_step_host), are launched apart while on: an untimed step is shorter than the
+ * sum of the times (32^3 RK4 step 0.197 ms against 0.264, 64^3 0.820 against 0.875). */
 int ns3d_timing_enable(ns3d_ctx *ctx, int on);
 
 /* Synchronise and read the accumulated device time (ms_out[k], milliseconds)
  * and launch counts (launches_out[k]) per kernel id, k < n (<= NS3D_K_COUNT);
- * either pointer may be NULL. */
+ * a shared launch of the x and y passes counts under both ids.  Launches are
+ * counted with recording on or off; either pointer may be NULL. */
 int ns3d_timing_read(ns3d_ctx *ctx, double *ms_out, long long *launches_out, int n);
 
 /* FP64 / FP32 arithmetic throughput of the current device in G lane-ops/s,

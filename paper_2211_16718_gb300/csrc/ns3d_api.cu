@@ -135,6 +135,7 @@ int rhs_pass(ns3d_ctx* c, const double* u, int epi, double* out, const double* u
     if (c->k2 && !c->timing) {  // the x and y passes in one launch (timed apart, they are launched apart)
       if ((rc = timed(c, kid[0], [&] { return launch_dir_xy(a, c->k2, c->stream); }, "x- and y-direction kernel")))
         return rc;
+      c->launches[kid[1]] += 1;  // one launch of both passes
       a.k2 = c->k2;
     } else {
       for (int d = 0; d < 2; ++d) {

@@ -433,6 +433,16 @@ def test_timing_counts_launches(ns3d):
     assert all(ms >= 0 for ms, _ in t.values()) and t["dir_x"][0] > 0
 
 
+def test_untimed_launches_are_counted_per_pass(ns3d):
+    """Without recording, small grids run the x and y passes in one launch: counted under both."""
+    s = ns3d.Solver(16, 16, 16, mu_eff=1e-3)
+    u = _gpu(I.taylor_green(16))
+    s.timing_enable(False)
+    s.rk_step(u, 0.01, 2)
+    t = s.timing_read()
+    assert [t[k][1] for k in ("prim", "visc", "dir_x", "dir_y", "dir_z")] == [8] * 5
+
+
 # ---- full sizes (the launch configuration the benchmark times) --------------------
 @pytest.mark.parametrize("prec", list(PRECISIONS))
 def test_hit256_rhs_sampled_points(ns3d, orc, prec):
