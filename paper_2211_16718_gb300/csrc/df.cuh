@@ -156,8 +156,8 @@ __device__ __forceinline__ float sqrt_seed(float y) {
 }
 
 // Division x / y (y a normal float magnitude): float quotient q1 from the reciprocal
-// seed, exact remainder x - q1*y (TwoProd), one correction q2 = remainder / y.  Error
-// about eps_seed^2 + 2^-48 relative (eps_seed ~ 2^-23).
+// seed, remainder x - q1*y (TwoProd), one correction q2 = remainder / y.  Relative error in
+// units of 2^-48 on random operands: 0.65 on average, 11 at most (33 by first-order analysis).
 __device__ __forceinline__ df df_div(df x, df y) {
   const float r = rcp_seed(y.hi);
   const float q1 = __fmul_rn(x.hi, r);
@@ -171,8 +171,9 @@ __device__ __forceinline__ df df_div(df x, df y) {
   return fast_two_sum(q1, q2);
 }
 
-// The same with the reciprocal seed refined once (two more FMAs): the remainder is then multiplied
-// by a reciprocal of error 2^-24 instead of up to 2^-23, and the error falls to about 2^-47.5.
+// The same with the reciprocal seed refined once (two more FMAs): the remainder is smaller and is
+// multiplied by a reciprocal of error 2^-24 instead of up to 2^-23.  0.60 on average, 8.8 at most (22);
+// what it gains most on are operands on which the seed is worst, and the two states of a jump can be such.
 __device__ __forceinline__ df df_div_r(df x, df y) {
   float r = rcp_seed(y.hi);
   r = __fmaf_rn(r, __fmaf_rn(-y.hi, r, 1.0f), r);
@@ -186,7 +187,8 @@ __device__ __forceinline__ df df_div_r(df x, df y) {
 }
 
 // Square root of a positive double-word (hi a normal float): float seed r, one
-// correction (x - r^2)/(2r) with the exact square of the seed (Dekker's method).
+// correction (x - r^2)/(2r) with the exact square of the seed (Dekker's method).  Error in units of
+// 2^-48: 0.32 on average, 6.5 at most (18.5).
 __device__ __forceinline__ df df_sqrt(df x) {
   const float r = sqrt_seed(x.hi);
   const df p = two_prod(r, r);
@@ -197,7 +199,8 @@ __device__ __forceinline__ df df_sqrt(df x) {
 }
 
 // The same with the reciprocal in the correction refined once and the correction's second-order
-// term -q^2/(2r) added (five more operations): the seed's error then enters with its cube.
+// term -q^2/(2r) added (five more operations): the seed's error then enters with its cube.  0.30 on
+// average, 6.0 at most (13).
 __device__ __forceinline__ df df_sqrt_r(df x) {
   const float r = sqrt_seed(x.hi);
   const df p = two_prod(r, r);

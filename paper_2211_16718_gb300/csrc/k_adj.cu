@@ -653,16 +653,6 @@ __device__ __forceinline__ void set_rec_lane(float4* r, int line, df x) {
 // double-float operation (df2_mul_u and friends: the same values, |lo| a few ulp(hi)).
 __device__ __forceinline__ df2 df2_sub(df2 x, df2 y) { return df2_add_fast(x, df2_neg(y)); }
 
-// 1/y for a normalised y, refined seed, unnormalised result (df2_div_ru with x = 1).
-__device__ __forceinline__ df2 df2_rcp_ru(df2 y) {
-  const float2 one = f2splat(1.0f);
-  float2 r = make_float2(rcp_seed(y.hi.x), rcp_seed(y.hi.y));
-  r = f2fma(r, f2fma(f2neg(y.hi), r, one), r);
-  const df2 p = two_prod2(r, y.hi);
-  const float2 rem = f2fma(f2neg(r), y.lo, f2sub(f2sub(one, p.hi), p.lo));
-  return df2{r, f2mul(rem, r)};
-}
-
 // The three weights of one reconstruction from the reciprocals r_k = 1/b_k of its window
 // terms (candidate order 0, 1, 2; optimal weights 1, 6, 3 over 10):
 // omega_k = c_k r_k^2 / sum_j c_j r_j^2.  With the window terms' range checked (b <= 1e18,

@@ -203,22 +203,6 @@ __device__ __forceinline__ df2 df2_offset3(df2 B1, df2 B2, df2 B3, df2 ta6, df2 
   return df2_div_ru(num, fast_two_sum2(den.hi, den.lo));
 }
 
-// The same reconstruction as an offset from the point value, its linear part e/6 over the common
-// denominator 6 den: d = [den e + 2 B2 B3 ta + 3 B1 B2 tb] / (6 den), for B_k that need no rescaling.
-// The direction pass used this form until its linear parts were combined across the interface
-// (phase C); it stays as the composition that the two-lane check compares with scalar code.
-template <bool SCALE>
-__device__ __forceinline__ df2 df2_offset(df2 B1, df2 B2, df2 B3, df2 e, df2 ta, df2 tb) {
-  static_assert(!SCALE, "unscaled form only");
-  const df2 p23 = df2_mul_u(B2, B3);
-  const df2 p13 = df2_mul_u(B1, B3);
-  const df2 p12 = df2_mul_u(B1, B2);
-  const df2 den = df2_add_pos_u(p23, df2_add_pos_u(df2_mul_f_u(p13, 6.0f), df2_mul_f_u(p12, 3.0f)));
-  const df2 num = df2_add_fast(df2_mul_u(den, e),
-                               df2_add_fast(df2_twice(df2_mul_u(p23, ta)), df2_mul_f_u(df2_mul_u(p12, tb), 3.0f)));
-  return df2_div(num, df2_mul_f_u(den, 6.0f));
-}
-
 // One tile of the direction-D pass, executed by the whole CTA on the shared memory sm (PL::BYTES):
 // the points [s0, s0 + len) along D (len <= TP), line group ty, tile row bz.  Used by the standalone
 // kernels (one tile per CTA), the batched kernels and the persistent ensemble kernel (many tiles per

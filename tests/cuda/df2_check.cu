@@ -14,7 +14,7 @@ using namespace ns3d;
 
 namespace {
 
-constexpr int NOPS = 16;
+constexpr int NOPS = 19;
 
 __device__ uint64_t mix64(uint64_t z) {  // SplitMix64 finaliser
   z += 0x9e3779b97f4a7c15ull;
@@ -38,7 +38,7 @@ __device__ bool same(df a, df b) {
   return __float_as_uint(a.hi) == __float_as_uint(b.hi) && __float_as_uint(a.lo) == __float_as_uint(b.lo);
 }
 
-// scalar references of df2_div / df2_sqrt (last step in the fma form)
+// scalar reference of df2_div (last step in the fma form)
 __device__ df ref_div(df x, df y) {
   const float r = rcp_seed(y.hi);
   const float q1 = __fmul_rn(x.hi, r);
@@ -51,12 +51,41 @@ __device__ df ref_div(df x, df y) {
   return df{s, __fmaf_rn(rem, r, -__fsub_rn(s, q1))};
 }
 
-// scalar reference of df2_offset<false> (the WENO5 offset of the direction pass)
-__device__ df ref_offset(df B1, df B2, df B3, df e, df ta, df tb) {
-  const df p23 = df_mul_u(B2, B3), p13 = df_mul_u(B1, B3), p12 = df_mul_u(B1, B2);
-  const df den = df_add_pos_u(p23, df_add_pos_u(df_mul_f_u(p13, 6.0f), df_mul_f_u(p12, 3.0f)));
-  const df num = df_add_fast(df_mul_u(den, e), df_add_fast(df_twice(df_mul_u(p23, ta)), df_mul_f_u(df_mul_u(p12, tb), 3.0f)));
-  return ref_div(num, df_mul_f_u(den, 6.0f));
+// scalar references of df2_div_ru and df2_rcp_ru (unnormalised results)
+__device__ df ref_div_ru(df x, df y) {
+  float r = rcp_seed(y.hi);
+  r = __fmaf_rn(r, __fmaf_rn(-y.hi, r, 1.0f), r);
+  const float q1 = __fmul_rn(x.hi, r);
+  const df p = two_prod(q1, y.hi);
+  float rem = __fsub_rn(x.hi, p.hi);
+  rem = __fsub_rn(rem, p.lo);
+  rem = __fadd_rn(rem, x.lo);
+  rem = __fmaf_rn(-q1, y.lo, rem);
+  return df{q1, __fmul_rn(rem, r)};
+}
+__device__ df ref_rcp_ru(df y) {
+  float r = rcp_seed(y.hi);
+  r = __fmaf_rn(r, __fmaf_rn(-y.hi, r, 1.0f), r);
+  const df p = two_prod(r, y.hi);
+  const float rem = __fmaf_rn(-r, y.lo, __fsub_rn(__fsub_rn(1.0f, p.hi), p.lo));
+  return df{r, __fmul_rn(rem, r)};
+}
+
+// scalar reference of df2_offset3 (the WENO5 offset of the direction pass)
+__device__ df ref_offset3(bool scale, df B1, df B2, df B3, df ta6, df tb6) {
+  if (scale) {
+    const int e1 = exponent_of(B1.hi), e2 = exponent_of(B2.hi), e3 = exponent_of(B3.hi);
+    const float sc = pow2f(-min(min(max(e1, max(e2, e3)), min(e1, min(e2, e3)) + 96), 126));
+    df* B[3] = {&B1, &B2, &B3};
+    for (int k = 0; k < 3; ++k) {
+      *B[k] = df{B[k]->hi * sc, B[k]->lo * sc};
+      if (B[k]->hi >= 2.0f) *B[k] = df{2.0f, 0.0f};
+    }
+  }
+  const df b1 = df_mul_f_u(B1, 3.0f), b3 = df_twice(B3);
+  const df den = df_add_pos_u(df_mul_u(B2, B3), df_mul_u(b1, df_add_pos_u(b3, B2)));
+  const df num = df_mul(B2, df_add_fast(df_mul_u(b3, ta6), df_mul_u(b1, tb6)));
+  return ref_div_ru(num, fast_two_sum(den.hi, den.lo));
 }
 
 // scalar reference of the squared indicators of phase B of the direction pass
@@ -108,8 +137,20 @@ __global__ void k_check(int n, uint64_t seed, int* bad) {
   r2[9] = df2_twice(p[1]);
   r2[10] = two_prod2(p[0].hi, p[1].hi);
   r2[11] = df2_div(p[0], p[2]);
-  r2[12] = df2_offset<false>(p[2], p[3], p[4], p[0], p[1], p[5]);
+  r2[12] = df2_offset3<false>(p[2], p[3], p[4], p[0], p[1]);
   new_indicators(p[0], p[1], df2_splat(c133), df2_splat(eps4), r2[13], r2[14], r2[15]);
+  // the rescaled form: indicators of their own powers of two in [2^-90, 2^118), so that the lanes'
+  // scales differ and about a third of the triples is cut
+  df b[2][3];
+  for (int l = 0; l < 2; ++l)
+    for (int j = 0; j < 3; ++j) {
+      const int e = (int)(mix64(~seed + 12ull * (uint64_t)t + 6ull * l + j) % 148) - 50;
+      b[l][j] = df{ldexpf(a[l][2 + j].hi, e), ldexpf(a[l][2 + j].lo, e)};
+    }
+  r2[16] = df2_offset3<true>(df2_pack(b[0][0], b[1][0]), df2_pack(b[0][1], b[1][1]), df2_pack(b[0][2], b[1][2]), p[0],
+                             p[1]);
+  r2[17] = df2_div_ru(p[0], p[2]);
+  r2[18] = df2_rcp_ru(p[2]);
   for (int l = 0; l < 2; ++l) {
     const df* x = a[l];
     r[l][0] = df_add_fast(x[0], x[1]);
@@ -124,11 +165,37 @@ __global__ void k_check(int n, uint64_t seed, int* bad) {
     r[l][9] = df_twice(x[1]);
     r[l][10] = two_prod(x[0].hi, x[1].hi);
     r[l][11] = ref_div(x[0], x[2]);
-    r[l][12] = ref_offset(x[2], x[3], x[4], x[0], x[1], x[5]);
+    r[l][12] = ref_offset3(false, x[2], x[3], x[4], x[0], x[1]);
     ref_indicators(x[0], x[1], c133, eps4, r[l][13], r[l][14], r[l][15]);
+    r[l][16] = ref_offset3(true, b[l][0], b[l][1], b[l][2], x[0], x[1]);
+    r[l][17] = ref_div_ru(x[0], x[2]);
+    r[l][18] = ref_rcp_ru(x[2]);
   }
   for (int o = 0; o < NOPS; ++o)
     if (!same(df2_lane0(r2[o]), r[0][o]) || !same(df2_lane1(r2[o]), r[1][o])) atomicAdd(&bad[o], 1);
+}
+
+// Relative errors of the divisions and square roots on normalised random operands, against FP64, in
+// units of 2^-48: the largest (1e-3 units) and the sum (for the mean) of df_div, df2_div, df_div_r,
+// df2_div_ru, df2_rcp_ru, df_sqrt, df_sqrt_r.
+constexpr int NERR = 7;
+__global__ void k_check_errors(int n, uint64_t seed, int* emax, double* esum) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  auto norm = [](df x) { return fast_two_sum(x.hi, x.lo); };
+  const df x = norm(rand_df(seed + 2ull * (uint64_t)t, false)), y = norm(rand_df(seed + 2ull * (uint64_t)t + 1, true));
+  auto val = [](df q) { return (double)q.hi + (double)q.lo; };
+  auto lane = [](df2 q) { return df2_lane1(q); };
+  const df2 x2 = df2_splat(x), y2 = df2_splat(y);
+  const double vx = val(x), vy = val(y);
+  const df got[NERR] = {df_div(x, y), lane(df2_div(x2, y2)), df_div_r(x, y), lane(df2_div_ru(x2, y2)),
+                        lane(df2_rcp_ru(y2)), df_sqrt(y), df_sqrt_r(y)};
+  const double ref[NERR] = {vx / vy, vx / vy, vx / vy, vx / vy, 1.0 / vy, sqrt(vy), sqrt(vy)};
+  for (int o = 0; o < NERR; ++o) {
+    const double e = fabs(val(got[o]) / ref[o] - 1.0) * 0x1p48;
+    atomicMax(&emax[o], e < 1e6 ? (int)(e * 1e3) : 1000000000);
+    atomicAdd(&esum[o], e);
+  }
 }
 
 // rcp_cubic (what = 0) and rsqrt_cubic (1) at the positive doubles of biased exponent
@@ -160,7 +227,7 @@ __global__ void k_check_cubic(int what, uint64_t seed, int* ulp, int* bad) {
 
 // Runs n lane pairs; bad_host receives NOPS mismatch counts (add_fast, sub, mul_u, mul, sqr_u,
 // mul_f_u, add_pos_u, add_ordered_u, add_ordered, twice, two_prod, div, offset, indicator
-// B1, B2, B3).  Returns a cudaError_t.
+// B1, B2, B3, rescaled offset, div_ru, rcp_ru).  Returns a cudaError_t.
 extern "C" int df2_check(int n, unsigned long long seed, int* bad_host) {
   int* bad = nullptr;
   cudaError_t e = cudaMalloc(&bad, sizeof(int) * NOPS);
@@ -191,3 +258,27 @@ extern "C" int cubic_check(int what, unsigned long long seed, int* ulp_host, int
   *bad_host = h[1];
   return (int)e;
 }
+
+// Largest and mean relative error (units of 2^-48) of the operations of k_check_errors over n operand
+// pairs: NERR doubles each.  Returns a cudaError_t.
+extern "C" int error_check(int n, unsigned long long seed, double* max_host, double* mean_host) {
+  double* d = nullptr;  // NERR sums, then NERR ints
+  cudaError_t e = cudaMalloc(&d, 2 * NERR * sizeof(double));
+  if (e != cudaSuccess) return (int)e;
+  cudaMemset(d, 0, 2 * NERR * sizeof(double));
+  int* m = reinterpret_cast<int*>(d + NERR);
+  k_check_errors<<<(n + 255) / 256, 256>>>(n, seed, m, d);
+  e = cudaGetLastError();
+  double sum[NERR];
+  int mx[NERR];
+  if (e == cudaSuccess) e = cudaMemcpy(sum, d, sizeof(sum), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(mx, m, sizeof(mx), cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  for (int o = 0; o < NERR && e == cudaSuccess; ++o) {
+    max_host[o] = mx[o] * 1e-3;
+    mean_host[o] = sum[o] / n;
+  }
+  return (int)e;
+}
+
+extern "C" int error_check_nops() { return NERR; }

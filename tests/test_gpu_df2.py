@@ -1,8 +1,9 @@
 """The two-lane double-float operations (csrc/df2.cuh, packed FP32 instructions) against the
 scalar ones (csrc/df.cuh), bit for bit, lane by lane, on a million pseudo-random lane pairs:
-every operation the direction and adjoint passes use, the WENO5 offset of the direction pass
-and its squared smoothness indicators.  The division's last step takes its error term from the
-exact product (df2.cuh); its reference is written out in that form in tests/cuda/df2_check.cu.
+the operations of the direction and adjoint passes, the WENO5 offset of the direction pass (with
+and without rescaling) and its squared smoothness indicators.  What has no scalar form in df.cuh
+(df2_div, df2_div_ru, df2_rcp_ru, the offset) is written out in tests/cuda/df2_check.cu.  Then the
+errors of the divisions, square roots and FP64 reciprocals.
 The check is built here from its own source into a temporary library; nothing of it is in
 libns3d.so."""
 import ctypes
@@ -13,7 +14,16 @@ import pytest
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 NAMES = ["add_fast", "sub", "mul_u", "mul", "sqr_u", "mul_f_u", "add_pos_u", "add_ordered_u", "add_ordered",
-         "twice", "two_prod", "div", "weno_offset", "indicator_B1", "indicator_B2", "indicator_B3"]
+         "twice", "two_prod", "div", "weno_offset", "indicator_B1", "indicator_B2", "indicator_B3",
+         "weno_offset_rescaled", "div_ru", "rcp_ru"]
+# relative errors in units of u^2 = 2^-48 (u = 2^-24): first-order bounds, and the means that the comments state.
+# A division's remainder, of up to 4 u (seed error 2 u unrefined: 5 u), rounds three times on the way to it
+# (2 + 3 + 4, 3 + 4 + 5) and is multiplied by a reciprocal in error by the seed's u (2 u), y.lo and a rounding:
+# 9 + 4 * 3 (12 + 5 * 4), and a rounding of the result; 3 + 2 * 3 for a reciprocal (no x.lo).  A root's
+# correction: half of the remainder's roundings 4 + 5, 2.5 u times the error of its factor (4 u, refined 3 u),
+# and unrefined the second-order term (2.5 u)^2 / 2
+ERRORS = {"df_div": (33, 0.66), "df2_div": (33, 0.63), "df_div_r": (22, 0.60), "df2_div_ru": (22, 0.60),
+          "df2_rcp_ru": (9.5, 0.40), "df_sqrt": (18.5, 0.33), "df_sqrt_r": (13, 0.31)}
 
 
 @pytest.fixture(scope="module")
@@ -31,6 +41,8 @@ def checker(tmp_path_factory):
     lib.df2_check.argtypes = [ctypes.c_int, ctypes.c_ulonglong, ctypes.POINTER(ctypes.c_int)]
     lib.df2_check_nops.restype = ctypes.c_int
     assert lib.df2_check_nops() == len(NAMES)
+    lib.error_check.argtypes = [ctypes.c_int, ctypes.c_ulonglong, ctypes.c_void_p, ctypes.c_void_p]
+    assert lib.error_check_nops() == len(ERRORS)
     return lib
 
 
@@ -55,3 +67,12 @@ def test_cubic_reciprocals_of_the_all_fp64_mode(checker, what, bound):
         assert checker.cubic_check(what, ctypes.c_ulonglong(seed), ctypes.byref(ulp), ctypes.byref(bad)) == 0
         assert bad.value == 0
         assert ulp.value * 1e-6 <= bound
+
+
+@pytest.mark.gpu
+def test_double_float_division_and_root_errors(checker):
+    """Errors of the divisions and square roots on four million normalised operands."""
+    mx, mean = (ctypes.c_double * len(ERRORS))(), (ctypes.c_double * len(ERRORS))()
+    assert checker.error_check(1 << 22, 20261205, mx, mean) == 0
+    for k, (name, (bound, avg)) in enumerate(ERRORS.items()):
+        assert mx[k] <= bound and mean[k] <= avg, (name, mx[k], mean[k])
