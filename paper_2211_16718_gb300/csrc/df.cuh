@@ -4,7 +4,7 @@
 // |lo| <= ulp(hi)/2, about 48 significant bits.
 //
 // Building blocks are the classical error-free transformations: Knuth's TwoSum,
-// Dekker's Fast2Sum and the FMA-based TwoProd; df_add/df_mul/df_div follow the
+// Dekker's Fast2Sum and the FMA-based TwoProd; the sums, df_mul and df_div follow the
 // usual double-word algorithms (Dekker 1971; Joldes, Muller, Popescu 2017).
 // Conversions from and to FP64 use integer bit manipulation only, so they do
 // not occupy the FP64 pipe.
@@ -18,8 +18,6 @@ namespace ns3d {
 struct df {
   float hi, lo;
 };
-
-__device__ __forceinline__ df df_make(float hi, float lo) { return df{hi, lo}; }
 
 // Fast2Sum (Dekker): exact s + e = a + b when |a| >= |b| (or a == 0).
 __device__ __forceinline__ df fast_two_sum(float a, float b) {
@@ -41,16 +39,6 @@ __device__ __forceinline__ df two_prod(float a, float b) {
   const float p = __fmul_rn(a, b);
   const float e = __fmaf_rn(a, b, -p);
   return df{p, e};
-}
-
-// Accurate double-word addition (two TwoSums), safe under cancellation.
-__device__ __forceinline__ df df_add(df x, df y) {
-  df s = two_sum(x.hi, y.hi);
-  df t = two_sum(x.lo, y.lo);
-  s.lo = __fadd_rn(s.lo, t.hi);
-  s = fast_two_sum(s.hi, s.lo);
-  s.lo = __fadd_rn(s.lo, t.lo);
-  return fast_two_sum(s.hi, s.lo);
 }
 
 // Double-word addition with one TwoSum: absolute error ~2^-47 (|x| + |y|), i.e.
@@ -105,13 +93,6 @@ __device__ __forceinline__ df df_mul(df x, df y) {
 __device__ __forceinline__ df df_sqr(df x) {
   df p = two_prod(x.hi, x.hi);
   const float e = __fmaf_rn(__fadd_rn(x.hi, x.hi), x.lo, p.lo);
-  return fast_two_sum(p.hi, e);
-}
-
-// Multiplication by a float (exact small integers, or any float).
-__device__ __forceinline__ df df_mul_f(df x, float c) {
-  df p = two_prod(x.hi, c);
-  const float e = __fmaf_rn(x.lo, c, p.lo);
   return fast_two_sum(p.hi, e);
 }
 
@@ -258,44 +239,20 @@ __device__ __forceinline__ df d2df_bits(double x) {
   return df{__uint_as_float(hb), lo};
 }
 
-// Round-to-nearest FP64 -> FP32 by bit manipulation (finite values in the float
-// range; smaller magnitudes flush to zero, larger ones saturate to infinity).
-__device__ __forceinline__ float d2f_rn(double x) {
-  const uint32_t h = (uint32_t)__double2hiint(x);
-  const uint32_t l = (uint32_t)__double2loint(x);
-  const uint32_t sign = h & 0x80000000u;
-  const int e8 = (int)((h >> 20) & 0x7ffu) - 896;
-  if (e8 <= 0) return __uint_as_float(sign);
-  if (e8 >= 255) return __uint_as_float(sign | 0x7f800000u);
-  uint32_t bits = ((uint32_t)e8 << 23) | ((h & 0xfffffu) << 3) | (l >> 29);
-  bits += (l >> 28) & 1u;  // round half up on the first dropped bit (carry may bump the exponent)
-  return __uint_as_float(sign | bits);
-}
-
 // Nearest-float of a double (truncated to 24 bits; enough for correction terms).
 __device__ __forceinline__ float d2f_trunc(double x) { return d2df_bits(x).hi; }
 
 // Largest power of two not above |x| (x finite, nonzero, normal float).
 __device__ __forceinline__ int exponent_of(float x) { return (int)((__float_as_uint(x) >> 23) & 0xffu) - 127; }
 
-// ---- FP64 reciprocal and reciprocal square root by Newton-Raphson -------------
-// Seeds from the FP32 MUFU approximations (relative error ~2^-22 after the
-// truncating conversion); each Newton step squares the error, two steps reach
-// FP64 rounding.  For x in the normal float range (positive for rsqrt).
+// ---- FP64 reciprocal by Newton-Raphson ------------------------------------------
+// Seed from the FP32 reciprocal (relative error ~2^-22 after the truncating conversion); each
+// Newton step squares the error, two steps reach FP64 rounding.  For x in the normal float range.
 __device__ __forceinline__ double rcp_newton(double x) {
   double r = f2d_bits(__frcp_rn(d2f_trunc(x)));
   double e = fma(-x, r, 1.0);
   r = fma(r, e, r);
   e = fma(-x, r, 1.0);
-  return fma(r, e, r);
-}
-
-__device__ __forceinline__ double rsqrt_newton(double x) {
-  double r = f2d_bits(rsqrtf(d2f_trunc(x)));
-  const double hx = 0.5 * x;
-  double e = fma(-hx * r, r, 0.5);  // (1 - x r^2)/2
-  r = fma(r, e, r);
-  e = fma(-hx * r, r, 0.5);
   return fma(r, e, r);
 }
 

@@ -146,11 +146,10 @@ __device__ __forceinline__ void weno_adjoint(double q0, double q1, double q2, do
 }
 
 // |lambda| with Harten's fix (acoustic fields): value and derivatives d/dlambda, d/ddelta.
-template <bool FAST>
 __device__ __forceinline__ double harten(double lam, double delta, double& dl, double& dd) {
   const double a = fabs(lam);
   if (a < delta) {
-    const double rd = FAST ? rcp_newton(delta) : 1.0 / delta;
+    const double rd = 1.0 / delta;
     dl = lam * rd;
     dd = 0.5 - 0.5 * (lam * rd) * (lam * rd);
     return 0.5 * (lam * lam + delta * delta) * rd;
@@ -164,10 +163,8 @@ __device__ __forceinline__ double harten(double lam, double delta, double& dl, d
 // algebra of the forward pass): given du = u^R - u^L, Lh = adjoint of the interface flux,
 // and the two point states a = i, b = i+1 (sqrt(rho), velocity, H, rho, e), returns
 // dub = adjoint of du and ga, gb = adjoint of the conserved states a, b through the Roe
-// average.  FAST: FP32-seeded Newton reciprocals instead of IEEE division and square
-// root (FP64-accurate).  Returns 1 for a non-physical Roe state, 2 for values outside the
-// range of the Newton seeds.
-template <int D, bool FAST>
+// average.  Returns 1 for a non-physical Roe state.
+template <int D>
 __device__ __forceinline__ int roe_adjoint(const double du[5], const double Lh[5], double ra, double rb,
                                            const double Va[3], const double Vb[3], double Ha, double Hb,
                                            double rho_a, double e_a, double rho_b, double e_b, double gamma,
@@ -176,7 +173,7 @@ __device__ __forceinline__ int roe_adjoint(const double du[5], const double Lh[5
   constexpr int T2 = (D == 2) ? 1 : 2;
   const double gm1 = gamma - 1.0;
   const double rsum = ra + rb;
-  const double rs = FAST ? rcp_newton(rsum) : 1.0 / rsum;
+  const double rs = 1.0 / rsum;
   const double wa = ra * rs, wb = rb * rs;
   double V[3];
 #pragma unroll
@@ -184,18 +181,7 @@ __device__ __forceinline__ int roe_adjoint(const double du[5], const double Lh[5
   const double H = fma(wa, Ha, wb * Hb);
   const double q2h = 0.5 * fma(V[0], V[0], fma(V[1], V[1], V[2] * V[2]));
   const double c2 = gm1 * (H - q2h);
-  int flags = !(c2 > 0.0) ? 1 : 0;
-  double c, rc;
-  if (FAST) {
-    // the float seeds of the Newton reciprocals need these inside the float range
-    flags |= (c2 > 1e-36 && c2 < 1e36 && rsum > 1e-36 && rsum < 1e36 && rho_a > 1e-36 && rho_a < 1e36 &&
-              rho_b > 1e-36 && rho_b < 1e36) ? 0 : 2;
-    rc = rsqrt_newton(c2);
-    c = c2 * rc;
-  } else {
-    c = sqrt(c2);
-    rc = 1.0 / c;
-  }
+  const double c = sqrt(c2), rc = 1.0 / c;
   const double un = V[D], vt1 = V[T1], vt2 = V[T2];
   const double b1 = gm1 * (rc * rc);
   const double vdm = fma(V[0], du[1], fma(V[1], du[2], V[2] * du[3]));
@@ -209,8 +195,8 @@ __device__ __forceinline__ int roe_adjoint(const double du[5], const double Lh[5
   const double a1 = 0.5 * phi + ach, a5 = 0.5 * phi - ach;
   const double delta = hdelta * c;
   double dl1, dd1, dl5, dd5;
-  const double l1 = harten<FAST>(un - c, delta, dl1, dd1);
-  const double l5 = harten<FAST>(un + c, delta, dl5, dd5);
+  const double l1 = harten(un - c, delta, dl1, dd1);
+  const double l5 = harten(un + c, delta, dl5, dd5);
   const double l2 = fabs(un);
   const double sg2 = (un > 0.0) ? 1.0 : (un < 0.0 ? -1.0 : 0.0);
   const double A1 = l1 * a1, A2 = l2 * a2, A3 = l2 * a3, A4 = l2 * a4, A5 = l5 * a5;
@@ -290,7 +276,7 @@ __device__ __forceinline__ int roe_adjoint(const double du[5], const double Lh[5
     const double wgt = side ? wb : wa;
     const double* Vp = side ? Vb : Va;
     const double rho = side ? rho_b : rho_a, e = side ? e_b : e_a, sr = side ? rb : ra;
-    const double rr = FAST ? rcp_newton(rho) : 1.0 / rho;
+    const double rr = 1.0 / rho;
     const double Hb_ = wgt * Hbar;
     const double srb = side ? rbb : rab;
     double Vt[3], vdot = 0.0;
@@ -306,7 +292,7 @@ __device__ __forceinline__ int roe_adjoint(const double du[5], const double Lh[5
 #pragma unroll
     for (int m = 0; m < 3; ++m) gs[1 + m] = Vt[m] * rr;
   }
-  return flags;
+  return !(c2 > 0.0) ? 1 : 0;
 }
 
 __device__ __forceinline__ void adj_epilogue(const AdjArgs& a, long long p, const double cv[5]) {
@@ -464,8 +450,8 @@ __global__ void __launch_bounds__(APL::THREADS, 2) k_adj_dir(const AdjArgs a) {
         Vb[m] = ri[(1 + m) * NP * W + sb];
       }
       double dub[5], ga[5], gb[5];
-      bad |= roe_adjoint<D, false>(du, Lh, ri[sa], ri[sb], Va, Vb, ri[4 * NP * W + sa], ri[4 * NP * W + sb], q[sa],
-                                   q[4 * NP * W + sa], q[sb], q[4 * NP * W + sb], a.gamma, a.hdelta, dub, ga, gb);
+      bad |= roe_adjoint<D>(du, Lh, ri[sa], ri[sb], Va, Vb, ri[4 * NP * W + sa], ri[4 * NP * W + sb], q[sa],
+                            q[4 * NP * W + sa], q[sb], q[4 * NP * W + sb], a.gamma, a.hdelta, dub, ga, gb);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
         rd[(5 + v) * NI * W + o] = ga[v];
