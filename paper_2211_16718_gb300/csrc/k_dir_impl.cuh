@@ -158,12 +158,7 @@ __device__ __forceinline__ df2 df2_sixth() {
   return df2_splat(df{hi, lo});
 }
 
-// Exponent of the power of two that the rescaling of df2_offset3 divides by, and the cut it applies
-// to the rescaled B_k (2 at most; they are normalised to rounding, so lo drops out with hi).
-__device__ __forceinline__ int offset_scale_exponent(float B1, float B2, float B3) {
-  const int e1 = exponent_of(B1), e2 = exponent_of(B2), e3 = exponent_of(B3);
-  return min(min(max(e1, max(e2, e3)), min(e1, min(e2, e3)) + 96), 126);
-}
+// The cut of df2_offset3 for rescaled B_k: 2 at most (lo drops out with hi).
 __device__ __forceinline__ df2 df2_cut2(df2 x) {
   const bool c0 = !(x.hi.x < 2.0f), c1 = !(x.hi.y < 2.0f);
   return df2{make_float2(c0 ? 2.0f : x.hi.x, c1 ? 2.0f : x.hi.y), make_float2(c0 ? 0.0f : x.lo.x, c1 ? 0.0f : x.lo.y)};
@@ -190,12 +185,22 @@ __device__ __forceinline__ df2 df2_cut2(df2 x) {
 template <bool SCALE = true>
 __device__ __forceinline__ df2 df2_offset3(df2 B1, df2 B2, df2 B3, df2 ta6, df2 tb6) {
   if (SCALE) {
-    const int E0 = offset_scale_exponent(B1.hi.x, B2.hi.x, B3.hi.x);
-    const int E1 = offset_scale_exponent(B1.hi.y, B2.hi.y, B3.hi.y);
+    const int x1 = exponent_of(B1.hi.x), x2 = exponent_of(B2.hi.x), x3 = exponent_of(B3.hi.x);
+    const int y1 = exponent_of(B1.hi.y), y2 = exponent_of(B2.hi.y), y3 = exponent_of(B3.hi.y);
+    int E0 = max(x1, max(x2, x3)), E1 = max(y1, max(y2, y3));
+    const int cut0 = min(x1, min(x2, x3)) + 96, cut1 = min(y1, min(y2, y3)) + 96;
+    const bool wide = E0 > cut0 || E1 > cut1;
+    E0 = min(E0, cut0);
+    E1 = min(E1, cut1);
     const float2 sc = make_float2(pow2f(-E0), pow2f(-E1));
-    B1 = df2_cut2(df2_scale(B1, sc));
-    B2 = df2_cut2(df2_scale(B2, sc));
-    B3 = df2_cut2(df2_scale(B3, sc));
+    B1 = df2_scale(B1, sc);
+    B2 = df2_scale(B2, sc);
+    B3 = df2_scale(B3, sc);
+    if (wide) {
+      B1 = df2_cut2(B1);
+      B2 = df2_cut2(B2);
+      B3 = df2_cut2(B3);
+    }
   }
   const df2 b1 = df2_mul_f_u(B1, 3.0f), b3 = df2_twice(B3);
   const df2 den = df2_add_pos_u(df2_mul_u(B2, B3), df2_mul_u(b1, df2_add_pos_u(b3, B2)));
