@@ -62,9 +62,10 @@ enum {
 enum { NS3D_RK4 = 0, NS3D_SSPRK3 = 1 };           /* time integrators (Sec. 2.2) */
 /* Arithmetic of the reconstruction and upwinding:
  *  NS3D_FP64        FP64 state, point values and their first differences, point fluxes,
- *                   interface-flux sums and RK update; what only multiplies small
- *                   differences or enters through a dissipation or viscous term (the
- *                   nonlinear WENO weights and offsets, the interface jumps, the Roe
+ *                   interface fluxes and their difference, and RK update; what only
+ *                   multiplies small differences or enters through a dissipation or viscous
+ *                   term (the nonlinear WENO weights and offsets, the interface jumps, the
+ *                   interface flux's difference from the point flux, the Roe
  *                   dissipation, the viscous fluxes and their divergence, the statistics'
  *                   kinetic energy, vorticity and wave speed) in double-float arithmetic
  *                   (two FP32 words, ~48 bits) on the FP32 pipe.  Agrees with the all-FP64
@@ -204,7 +205,8 @@ int ns3d_dt_from_cfl(ns3d_ctx *ctx, const double *u_dev, double cfl, double *dt_
  * returns, also when it fails. */
 int ns3d_step_host(ns3d_ctx *ctx, double *u_host, double dt, int nsteps, ns3d_stats_t *stats_host);
 
-/* Read and clear the sticky status word (synchronises): NS3D_OK or NS3D_ENONPHYSICAL. */
+/* Read and clear the sticky status word (synchronises): NS3D_OK, NS3D_ENONPHYSICAL or
+ * NS3D_ERANGE. */
 int ns3d_check(ns3d_ctx *ctx);
 
 /* Static description of a code. */
@@ -220,8 +222,8 @@ const char *ns3d_last_error(const ns3d_ctx *ctx);
  * precision, which must be NS3D_FP64 or NS3D_FP64_STRICT, and rk), its own
  * caller-owned state and its own dt.  The schedules compute bitwise identical
  * results:
- *  NS3D_BATCH_SEQUENTIAL  per-instance launches (5 per RK stage per instance), one
- *                         instance after the other on the batch's stream;
+ *  NS3D_BATCH_SEQUENTIAL  per-instance launches (5 per RK stage per instance, 4 up to
+ *                         2^15 points), one instance after the other on the batch's stream;
  *  NS3D_BATCH_GRAPH       the same per-instance launches for one step, captured once
  *                         in a CUDA graph whose parallel branches each advance a share
  *                         of the instances (balanced by points, largest first), so that
@@ -255,7 +257,7 @@ int ns3d_batch_set_dt_from_cfl(ns3d_batch *b, double cfl, double *dt_out);
 /* Read and clear the batch's sticky status word (synchronises). */
 int ns3d_batch_check(ns3d_batch *b);
 /* Tile shape of the direction passes: variant 0 (24 x 4), 1 (16 x 4), 2 (40 x 2)
- * points x lines, for every instance and the persistent kernel; results do not
+ * points (at most) x lines, for every instance and the persistent kernel; results do not
  * depend on it.  NS3D_FP64_STRICT batches have the one shape 0 (32 x 4). */
 int ns3d_batch_set_variant(ns3d_batch *b, int variant);
 /* Tile shape of instance i alone (SEQUENTIAL and GRAPH schedules; the persistent
@@ -299,9 +301,9 @@ int ns3d_storage_info(const ns3d_ctx *ctx, int *storage, size_t *device_bytes);
  * Exact discrete adjoints of the operators above (the paper has none; they serve
  * gradients of statistics of the flow with respect to its initial state).
  * NS3D_FP64_STRICT contexts evaluate them all in FP64; NS3D_FP64 contexts run the
- * derivatives of the WENO5 reconstructions in double-float arithmetic (relative
- * rounding ~1e-14, data range as for the forward weights, NS3D_ERANGE beyond it) and
- * the rest in FP64; NS3D_FP32_BULK contexts return NS3D_EINVAL.
+ * derivatives of the WENO5 reconstructions, the Roe flux and the viscous terms in
+ * double-float arithmetic (relative rounding ~1e-14, data range as for the forward
+ * weights, NS3D_ERANGE beyond it) and the rest in FP64; NS3D_FP32_BULK contexts return NS3D_EINVAL.
  * Derivatives follow the discretisation as written: the WENO5 weights (smooth,
  * eps > 0), the Roe average, Harten's quadratic branch, and |lambda| with the
  * subgradient sign(0) = 0 at its kink.  The first adjoint call of a context
@@ -357,8 +359,8 @@ enum {
 /* on != 0: record CUDA events around every kernel launch of ctx (on its stream)
  * and accumulate their durations; on == 0 stops recording.  Resets counters.
  * The x and y passes, which share one launch on grids of up to 2^20 points (not in
- * NS3D_FP32_BULK contexts, with viscous lean storage or in the slab-wise stages of
- * ns3d_step_host), are launched apart while on: an untimed step is shorter than the
+ * NS3D_FP32_BULK contexts, with viscous lean storage or in the first stage of an
+ * ns3d_step_host in slabs), are launched apart while on: an untimed step is shorter than the
  * sum of the times (32^3 RK4 step 0.197 ms against 0.264, 64^3 0.820 against 0.875). */
 int ns3d_timing_enable(ns3d_ctx *ctx, int on);
 

@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(APL::THREADS, 2) k_adj_dir(const AdjArgs a) {
 // The per-point sums are converted back to FP64 once.  To keep double-float values inside the float
 // range whatever the scale of the adjoint input, each tile divides the interface differences of
 // lambda by the power of two of lambda's largest magnitude and multiplies its results back (exact).
-// What bounds it: latency at 16 warps per SM (128 registers; 103 KB of shared memory).  365 warp
+// What bounds it: latency at 16 warps per SM (128 registers; 106.6 KB of shared memory).  365 warp
 // instructions per point where carrying every reconstruction to its points took 488: 128^3 pass
 // 2.15 / 2.24 / 2.13 -> 1.63 / 1.85 / 1.81 ms (x / y / z).  More warps with fewer registers lose: the
 // Roe adjoint's chain then spills 430 bytes (384 threads of 80 registers: 2.18 / 2.28 / 2.23 ms).

@@ -25,8 +25,8 @@ __global__ void __launch_bounds__(Plan<MODE, TP, W>::THREADS, Plan<MODE, TP, W>:
 // The x pass (blocks below nbx) and the y pass side by side in one launch: neither reads what the
 // other writes.  It fills the second pass's launch gap and the last, partly filled round of CTAs:
 // 40x25x18 right-hand side 34.8 -> 30.2 us, 32^3 RK4 step 240 -> 215 us, 64^3 passes 115 -> 112 us,
-// 96^3 all-FP64 step 8.97 -> 8.91 ms, but 128^3 passes 805 -> 816 us (the two code paths share the
-// instruction caches), so only grids of up to 2^20 points (dir_xy_merged).
+// 96^3 all-FP64 step 8.97 -> 8.91 ms, but 128^3 passes 805 -> 816 us (why was not measured), so only
+// grids of up to 2^20 points (dir_xy_merged).
 template <int MODE, int TP, int W>
 __global__ void __launch_bounds__(Plan<MODE, TP, W>::THREADS, Plan<MODE, TP, W>::MIN_CTAS) k_dir_xy(const DirArgs ax,
                                                                                                 const DirArgs ay,

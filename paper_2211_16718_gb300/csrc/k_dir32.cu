@@ -33,13 +33,17 @@ namespace {
 
 constexpr int THREADS = 256;
 // At most 27 points along x, 26 along y and z (balanced tiles, k_dir_common.cuh) x 8 lines.  26 are 256
-// points with the halo, one per thread in phase A; 27 take a second round of 8, and pay along x where
-// they save a tile: x pass of 2^24 points 27 against 26 at nx = 54 156 / 184 us, 160 451 / 462, 320
-// 675 / 725, 500 646 / 696; where the number of tiles is the same, and at 512 (19 against 20 tiles), the
-// two are within 0.2 % of one another.  At 512^3 (x / y / z): 5.57 / 6.23 / 10.35 ms with 27, 5.80 / 6.21 /
-// 10.13 ms with 26; the step with 24 everywhere 2 % slower, with 23 5 %.  Before, full tiles of 27 with a
-// remainder computed in full and two points per thread in E: 5.59 / 6.85 / 10.21 ms (and 69 % of the work
-// wasted on a 32-point line).
+// points with the halo, one per thread in phase A; 27 take a second round of 8, and pay where they save a
+// short line a tile.  Passes over 2^24 points with 27 / 26, where the number of tiles differs (elsewhere
+// the two are equal):
+//   x at nx = 54 156 / 184 us, 160 451 / 462, 320 675 / 725, 500 646 / 696, 512 663 / 661
+//   y at ny = 54 182 / 216 us, 160 509 / 521, 320 795 / 799, 400 789 / 787, 512 768 / 756
+//   z at nz = 54 241 / 283 us, 160 702 / 732, 320 1058 / 1057, 400 1048 / 1039, 512 1023 / 1012
+// so that 27 is the better limit along x at every length, while along y and z 26 is the better one only
+// from 400 points up, the sizes that this mode is for.  The 512^3 step with 24 everywhere is 2 % slower,
+// with 23 5 %.  Before, full tiles of 27 with a remainder computed in full and two points per thread in E:
+// 5.59 / 6.85 / 10.21 ms at 512^3 where these take 5.55 / 6.26 / 10.28 (and 69 % of the work wasted on a
+// 32-point line).
 __host__ __device__ constexpr int tile_max(int d) { return d == 0 ? 27 : 26; }
 constexpr int TP = tile_max(0), W = 8;
 constexpr int NP = TP + 6;      // positions per line: 3-point halo on each side

@@ -24,16 +24,14 @@
 // at one interface and the right-biased one at another, so each is computed once.
 //
 // Since sum omega = 1, fhat = F_2 + omega_1 (F_1 - F_2) + omega_3 (F_3 - F_2): the reconstructions
-// are candidate 2 and an offset from third differences of the data.
+// are candidate 2 and an offset, F_1 - F_2 and F_3 - F_2 being third differences of the data.
 // MODE 0 (all FP64): bound by the FP64 pipe (2 lanes per SM and clock), so written for its operation
 // count: with D = B_2/6 the offset is D [B_3 (F_1 - F_2) + 3 B_1 (F_3 - F_2)] / [D B_3 + B_1 (B_3 + 3 D)],
 // six operations and a reciprocal; jump and sum of the two reconstructions share their linear parts.
-// 495 FP64 operations per point and pass where candidates, IEEE divisions and separate left and right
-// values took 726: 96^3 pass 1.26 / 1.31 / 1.35 -> 0.91 / 0.92 / 0.95 ms (x / y / z, FP64 pipe 87 %
+// 496 FP64 operations per point and pass with the halo's share (459 without) where candidates, IEEE
+// divisions and separate left and right values took 726: 96^3 pass 1.26 / 1.31 / 1.35 -> 0.91 / 0.92 / 0.95 ms (x / y / z, FP64 pipe 87 %
 // busy), the error of a right-hand side against 64 bits 13-19 % smaller.
-// MODE 1 (FP64 values, double-float weights): since sum omega = 1,
-//   fhat = F_2 + omega_1 (F_1 - F_2) + omega_3 (F_3 - F_2),
-// where F_1 - F_2 and F_3 - F_2 are third differences of the data and the weights, which only multiply these small
+// MODE 1 (FP64 values, double-float weights): the weights, which only multiply these small
 // differences, are evaluated in double-float arithmetic (~48 bits) on the FP32
 // pipe.  The reconstructed values themselves are never formed: the Roe flux needs
 // fhat_L + fhat_R and the jump fhat_R - fhat_L, whose linear parts combine (phase C),

@@ -286,7 +286,7 @@ __device__ __forceinline__ double warp_fold(double x) {
 }
 
 // Fold of one quantity (0..NSUM-1: sum, NSUM and NSUM+1: minimum, last: maximum) by one warp over
-// n values v[0], v[stride], ...: every lane folds its values in order, then the lanes.
+// the n values v[0 .. n): every lane folds its values in order, then the lanes.
 __device__ __forceinline__ double fold_column(int q, const double* v, int n, int lane) {
   double x = (q < NSUM) ? 0.0 : (q < NRED - 1) ? INFINITY : 0.0;
   if (q < NSUM) {

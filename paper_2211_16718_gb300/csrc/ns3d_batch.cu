@@ -37,10 +37,10 @@ namespace {
 
 constexpr int MAX_STAGES = 4;
 constexpr int BT = 256;  // threads of the pointwise batched kernels
-// Instances up to this size run their x and y passes in one launch (launch_dir_xy).  GRAPH schedule:
-// 48 grids of 12^3-24^3 2.03 -> 1.77 ms per step, 8 of them 0.40 -> 0.36 ms; larger instances fill the
-// gaps of one another already (16 grids of 24^3-48^3 2.43 ms apart, 2.48 with all of them merged,
-// 2.41 with this line; 48 of 32^3-128^3 79.5, 80.0, 79.7 ms).
+// Instances up to this size run their x and y passes in one launch (launch_dir_xy): it pays for sets of
+// small grids.  GRAPH schedule: 48 grids of 12^3-24^3 2.03 -> 1.77 ms per step, 8 of them 0.40 -> 0.36 ms;
+// larger instances fill the gaps of one another already (16 grids of 24^3-48^3 2.43 ms apart, 2.48 with
+// all of them merged, 2.41 with this line; 48 of 32^3-128^3 79.5, 80.0, 79.7 ms, equal within the runs).
 constexpr long long BATCH_XY_POINTS = 1LL << 15;
 
 struct Inst {

@@ -26,7 +26,7 @@ struct ns3d_ctx {
   double* ua = nullptr;        // [5][N] stage state
   double* ub = nullptr;        // [5][N] stage state
   double* acc = nullptr;       // [5][N] RK4 accumulator
-  double* partials = nullptr;  // [stats blocks][10]
+  double* partials = nullptr;  // [10][stats blocks]
   double* stats_dev = nullptr; // [NS3D_STATS_NDOUBLE]
   int* status = nullptr;       // sticky status word
   double* uhost_dev = nullptr; // device state for ns3d_step_host (lazy)

@@ -164,9 +164,9 @@ def test_fp32_bulk_hit256_sampled_points(ns3d, orc):
 @pytest.mark.parametrize("eps,jump", [(1e-6, 1e6), (1e-6, 1e8), (1e-15, 1e5), (1e-15, 1e8), (1e-6, 1e10)])
 def test_fp32_bulk_jump_next_to_constant_data(ns3d, axis, eps, jump):
     shp = [6, 6, 6]
-    shp[axis] = 61  # three tiles along every axis
+    shp[axis] = 61
     p = np.ones(61)
-    p[8:28] += jump
+    p[21:41] += jump  # the jumps lie between the tiles of 21, 20 and 20 points
     p = p[tuple(slice(None) if k == axis else None for k in range(3))] * np.ones(shp)
     u0 = I.to_conserved(np.ones(shp), *(np.full(shp, 0.3 * (m + 1)) for m in range(3)), p)
     u = _gpu(u0)

@@ -98,7 +98,6 @@ def test_balanced_tiles(ns3d, orc, nx, ny, nz):
             assert np.array_equal(out[0], out[-1]), (prec, v)
 
 
-
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("nx", [24, 26, 27])
 def test_step_of_a_state_on_8_byte_boundaries(ns3d, nx, prec):
@@ -163,3 +162,26 @@ def test_balanced_tiles_fp32_bulk(ns3d, orc, nx, ny, nz):
     s.close()
     # FP32 fluxes: 1e-5 of the flux scale over the smallest spacing (as the FP32-bulk tests)
     assert np.abs(r - ref).max() <= 1e-5 * flux_scale(u, (2 * np.pi,) * 3)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_adjoint_of_jumps_between_tiles(ns3d, axis):
+    """A shock tube whose jumps lie between the adjoint's tiles (along x 24, 24 and 17 points of 65,
+    else 22, 22 and 21), and one with them inside; as test_adjoint_tiles."""
+    shp = [5, 4, 6]
+    shp[axis] = 65
+    lam = _gpu(np.random.default_rng(6).normal(size=[5] + shp))
+    for lo, hi in ((24, 48) if axis == 2 else (22, 44), (10, 33)):
+        left = np.ones(65, dtype=bool)
+        left[lo:hi] = False
+        left = left[tuple(slice(None) if k == axis else None for k in range(3))]
+        wave = 1.0 + 0.02 * np.random.default_rng(7).uniform(-1.0, 1.0, shp)
+        vel = [0.1 * (m + 1) * (wave - 1.0) for m in range(3)]
+        u = _gpu(I.to_conserved(np.where(left, 1.0, 0.125) * wave, *vel, np.where(left, 1.0, 0.1) * wave / 1.4))
+        out = []
+        for prec in (0, 2):
+            s = ns3d.Solver(*shp[::-1], mu_eff=0.003, precision=prec)
+            out.append(s.rhs_vjp(u, lam).cpu().numpy())
+            s.check()
+            s.close()
+        assert rel_err(out[0], out[1]) <= 1e-11
