@@ -516,7 +516,7 @@ def run_ours(args, world, rank, local):
         "method_fp64_frac": (FLOPS_DIR + 5) * N / avg_launch_s / 1e12 / FP64_PEAK_TFLOPS,
         "fp64_peak_tflops": FP64_PEAK_TFLOPS,
         "pipes": {"fp64_pipe_lane_ops_per_point": OPS_DIR_FP64 + OPS_RK_EPI / 3.0,
-                  "fp64_pipe_part": "point values, first differences, point fluxes, interface-flux sums, flux "
+                  "fp64_pipe_part": "point values, first differences, point fluxes, interface fluxes, flux "
                                     "difference, RK update",
                   "fp32_pipe_part": "WENO weights and offsets, interface jumps, Roe dissipation, viscous "
                                     "fluxes and divergence, as double-float; the differences, indicators and "
@@ -543,7 +543,8 @@ def run_ours(args, world, rank, local):
     del solver
 
     modes = {"fp64": {"value": value, "ms_per_step": ms / K,
-                      "weights": "double-float (FP32 pairs), all else FP64"}}
+                      "weights": "double-float (FP32 pairs), as the offsets, jumps, Roe dissipation and viscous "
+                                 "terms; all else FP64"}}
     if not args.no_strict:
         def strict():
             Ks, Ws = 2, 1
@@ -678,8 +679,8 @@ def _fp32_compare(timed_loop, u64, st64, n_cmp, K, W, value64, world, N, ns3d) -
     scale = u64.abs().reshape(5, -1).amax(dim=1).cpu().numpy()
     del u3
     return {"value": v3, "ms_per_step": ms3 / K, "speedup_vs_fp64": v3 / value64,
-            "arithmetic": "FP32 indicators, weights, interface values, Roe flux; FP64 state, difference, "
-                          "viscous terms, RK, reductions",
+            "arithmetic": "FP32 indicators, weights, interface values, Roe and viscous fluxes; FP64 state, "
+                          "difference, RK, reductions",
             "steps_compared": n_cmp, "dt": "the FP64 headline's",
             "ke_rel_err_max_over_steps": float((np.abs(b[:, 5] - a[:, 5]) / np.abs(a[:, 5])).max()),
             "enstrophy_rel_err_max_over_steps": float((np.abs(b[:, 6] - a[:, 6]) / np.abs(a[:, 6])).max()),

@@ -1,5 +1,5 @@
-"""FP32-bulk mode (NS3D_FP32_BULK): smoothness indicators, weights, interface values and
-Roe flux in FP32; state, conservative difference, viscous terms, RK and reductions FP64.
+"""FP32-bulk mode (NS3D_FP32_BULK): smoothness indicators, weights, interface values, Roe
+and viscous fluxes in FP32; state, conservative difference, RK and reductions FP64.
 
 Tolerance, derived from the arithmetic: each interface flux carries a relative FP32
 rounding error of order c * 2^-24 (c ~ 10-30 for the WENO + Roe evaluation), and the
